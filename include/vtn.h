@@ -62,7 +62,9 @@ typedef enum {
 } vtn_status;
 
 typedef enum {
-    VTN_FP64 = 0,          /* every contraction in IEEE double (SIMT FP64 FMA)           */
+    VTN_FP64 = 0,          /* every contraction to IEEE double accuracy: FP64 FMA, or (large
+                              products) exact sums of 8-bit digit products on the tensor
+                              cores, rounded once                                        */
     VTN_TF32X3 = 1,        /* reserved: three-term TF32 split products (VTN_EUNSUPPORTED) */
     VTN_BF16X3 = 2         /* H_eff psi and the environment updates on the tensor cores:
                               each FP64 operand split into bf16 hi + lo, products

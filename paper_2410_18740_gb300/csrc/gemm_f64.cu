@@ -1,12 +1,15 @@
-// Complex FP64 GEMM for the FP64 solver path (SIMT DFMA; GB300 has no FP64 tensor-core
-// rate worth using, and FP64 FMA throughput is the roofline of this kernel):
+// Complex FP64 GEMM for the FP64 solver path:
 //   C[batch] (=|+=) sum_{kb} op(A[batch, kb]) op(B[batch, kb]),  op in {X, X^dag}.
 // Every contraction of the two-site effective Hamiltonian, the environment updates and
-// the reduced density matrix is one call.  Tiles of 64 x 64 outputs per 256-thread CTA,
-// 4 x 4 complex micro-tile per thread, K staged through shared memory in steps of 8.
-// One CTA alone keeps an SM's FP64 pipe only about half busy, so a call with fewer output
-// tiles than two per SM splits the summation range (kb, K) over S CTAs per tile; the S
-// partial tiles are summed in a fixed order by a second kernel (deterministic).
+// the reduced density matrix is one call.
+//
+// Large products go to the tensor cores by exact integer slices (oz_gemm.cu).  The kernel here is for
+// the small ones and for callers that cannot use a workspace: SIMT DFMA, of which GB300 issues one warp
+// instruction per 64 cycles and SM sub-partition, so a call is bound by the number of SMs that work.
+// Hence tiles of 16 x 16 outputs, one per thread of a 256-thread CTA (a 64 x 64 tile takes an SM 40 us per 8
+// terms whatever part of it is used: the 454 products of a 4-mode chi = 16 solve took 103 us each, 5 us with
+// these), and a summation that is split over CTAs while there are fewer than two per SM; the partial
+// sums are added in a fixed order by a second kernel (deterministic).
 #include <algorithm>
 
 #include "vtn_internal.cuh"
@@ -14,7 +17,7 @@
 namespace vtn {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4, NT = 256;
+constexpr int BT = 16, BK = 16, NT = 256;  // output tile edge, summation step, threads
 
 struct GemmP {
     int M, N, K, kb;
@@ -25,6 +28,7 @@ struct GemmP {
     int accumulate;
     int herm_lower;
     int negate;
+    int batch;
     int splits;          // S: CTAs per output tile along the summation range
     double2* part;       // S > 1: partial tiles [S][batch][M][N]
 };
@@ -32,106 +36,72 @@ struct GemmP {
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 
 __global__ void __launch_bounds__(NT) gemm_c64_kernel(GemmP p) {
-    __shared__ double2 As[BK][BM];
-    __shared__ double2 Bs[BK][BN];
+    __shared__ double2 As[BK][BT + 1];
+    __shared__ double2 Bs[BK][BT + 1];
     const int tid = threadIdx.x;
-    const int tx = tid % 16, ty = tid / 16;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const long long bz = blockIdx.z / p.splits;
-    const int split = blockIdx.z % p.splits;
-    if (p.herm_lower && n0 >= m0 + BM) return;  // tile strictly above the diagonal
-    double2 acc[TM][TN];
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = make_double2(0.0, 0.0);
+    const int tx = tid % BT, ty = tid / BT;
+    const int gx = (p.N + BT - 1) / BT, gy = (p.M + BT - 1) / BT;
+    long long id = blockIdx.x;
+    const int n0 = (int)(id % gx) * BT;
+    id /= gx;
+    const int m0 = (int)(id % gy) * BT;
+    id /= gy;
+    const int split = (int)(id % p.splits);
+    const long long bz = id / p.splits;
+    if (p.herm_lower && n0 > m0) return;  // tile strictly above the diagonal
+    double2 acc = make_double2(0.0, 0.0);
 
     // this CTA's share [t0, t1) of the kb * ceil(K / BK) steps of the summation
     const int nk = (p.K + BK - 1) / BK;
     const long long T = (long long)nk * p.kb;
     const long long t0 = T * split / p.splits, t1 = T * (split + 1) / p.splits;
     int kb = (int)(t0 / nk), k0 = (int)(t0 % nk) * BK;
-    for (long long t = t0; t < t1; ++t) {
+    // the staged element of each thread: along the contiguous index of its operand
+    const int am = p.opA == OP_N ? ty : tx, ak = p.opA == OP_N ? tx : ty;
+    const int bn = p.opB == OP_N ? tx : ty, bk = p.opB == OP_N ? ty : tx;
+    auto load = [&](double2& a, double2& b) {
         const double2* A = p.A + bz * p.sA_batch + (long long)kb * p.sA_kb;
         const double2* B = p.B + bz * p.sB_batch + (long long)kb * p.sB_kb;
-        {
-            // ---- stage op(A)[m0:m0+64, k0:k0+8]
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                int idx = tid + r * NT;
-                int ml, kl;
-                if (p.opA == OP_N) { ml = idx / BK; kl = idx % BK; }
-                else { ml = idx % BM; kl = idx / BM; }
-                int m = m0 + ml, k = k0 + kl;
-                double2 v = make_double2(0.0, 0.0);
-                if (m < p.M && k < p.K) {
-                    v = (p.opA == OP_N) ? A[(long long)m * p.lda + k] : cconj(A[(long long)k * p.lda + m]);
-                }
-                As[kl][ml] = v;
-            }
-            // ---- stage op(B)[k0:k0+8, n0:n0+64]
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                int idx = tid + r * NT;
-                int nl, kl;
-                if (p.opB == OP_N) { nl = idx % BN; kl = idx / BN; }
-                else { kl = idx % BK; nl = idx / BK; }
-                int n = n0 + nl, k = k0 + kl;
-                double2 v = make_double2(0.0, 0.0);
-                if (n < p.N && k < p.K) {
-                    v = (p.opB == OP_N) ? B[(long long)k * p.ldb + n] : cconj(B[(long long)n * p.ldb + k]);
-                }
-                Bs[kl][nl] = v;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < BK; ++kk) {
-                double2 a[TM], b[TN];
-#pragma unroll
-                for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-                for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-                for (int i = 0; i < TM; ++i)
-#pragma unroll
-                    for (int j = 0; j < TN; ++j) {
-                        acc[i][j].x = fma(a[i].x, b[j].x, acc[i][j].x);
-                        acc[i][j].x = fma(-a[i].y, b[j].y, acc[i][j].x);
-                        acc[i][j].y = fma(a[i].x, b[j].y, acc[i][j].y);
-                        acc[i][j].y = fma(a[i].y, b[j].x, acc[i][j].y);
-                    }
-            }
-            __syncthreads();
-        }
+        const int m = m0 + am, n = n0 + bn, ka = k0 + ak, kk = k0 + bk;
+        a = b = make_double2(0.0, 0.0);
+        if (m < p.M && ka < p.K)
+            a = p.opA == OP_N ? A[(long long)m * p.lda + ka] : cconj(A[(long long)ka * p.lda + m]);
+        if (n < p.N && kk < p.K)
+            b = p.opB == OP_N ? B[(long long)kk * p.ldb + n] : cconj(B[(long long)n * p.ldb + kk]);
+    };
+    double2 ra, rb;
+    if (t0 < t1) load(ra, rb);
+    for (long long t = t0; t < t1; ++t) {
+        As[ak][am] = ra;
+        Bs[bk][bn] = rb;
+        __syncthreads();
+        const int ke = min(BK, p.K - k0);
         k0 += BK;
         if (k0 >= p.K) { k0 = 0; ++kb; }
-    }
-    if (p.negate) {
-#pragma unroll
-        for (int i = 0; i < TM; ++i)
-#pragma unroll
-            for (int j = 0; j < TN; ++j) acc[i][j] = make_double2(-acc[i][j].x, -acc[i][j].y);
-    }
-    const bool to_part = p.splits > 1;
-    double2* C = to_part ? p.part + ((long long)split * (gridDim.z / p.splits) + bz) * p.M * p.N : p.C + bz * p.sC_batch;
-    const long long ldc = to_part ? p.N : p.ldc;
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        int m = m0 + ty + 16 * i;
-        if (m >= p.M) continue;
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            int n = n0 + tx + 16 * j;
-            if (n >= p.N) continue;
-            double2* c = C + (long long)m * ldc + n;
-            if (p.accumulate && !to_part) {
-                double2 o = *c;
-                *c = make_double2(o.x + acc[i][j].x, o.y + acc[i][j].y);
-            } else {
-                *c = acc[i][j];
-            }
+        if (t + 1 < t1) load(ra, rb);  // the next step's elements, in flight during this one
+        for (int kk = 0; kk < ke; ++kk) {
+            const double2 a = As[kk][ty], b = Bs[kk][tx];
+            acc.x = fma(a.x, b.x, acc.x);
+            acc.x = fma(-a.y, b.y, acc.x);
+            acc.y = fma(a.x, b.y, acc.y);
+            acc.y = fma(a.y, b.x, acc.y);
         }
+        __syncthreads();
     }
+    if (p.negate) acc = make_double2(-acc.x, -acc.y);
+    const int m = m0 + ty, n = n0 + tx;
+    if (m >= p.M || n >= p.N) return;
+    if (p.splits > 1) {
+        p.part[(((long long)split * p.batch + bz) * p.M + m) * p.N + n] = acc;
+        return;
+    }
+    double2* c = p.C + bz * p.sC_batch + (long long)m * p.ldc + n;
+    if (p.accumulate) {
+        const double2 o = *c;
+        acc.x += o.x;
+        acc.y += o.y;
+    }
+    *c = acc;
 }
 
 // C[b][m][n] (=|+=) sum_{s < S} part[s][b][m][n], s ascending
@@ -141,7 +111,7 @@ __global__ void splitk_sum(GemmP p, int batch) {
     if (t >= mn * batch) return;
     const long long b = t / mn, e = t % mn;
     const int m = (int)(e / p.N), n = (int)(e % p.N);
-    if (p.herm_lower && n / BN > m / BM) return;
+    if (p.herm_lower && n / BT > m / BT) return;
     double2 acc = p.part[t];
     for (int s = 1; s < p.splits; ++s) {
         const double2 v = p.part[(long long)s * mn * batch + t];
@@ -189,27 +159,43 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     p.herm_lower = g.herm_lower ? 1 : 0;
     p.negate = g.negate ? 1 : 0;
     VTN_REQUIRE(!g.herm_lower || (g.M == g.N && !g.accumulate), "Hermitian GEMM needs a square, non-accumulating C");
-    const int gx = (g.N + BN - 1) / BN, gy = (g.M + BM - 1) / BM;
-    VTN_REQUIRE(gy <= 65535, "gemm M too large");
-    // output tiles that do work; split the summation when they leave SMs short of 2 CTAs
-    const long long tiles = (g.herm_lower ? (long long)gy * (gy + 1) / 2 : (long long)gx * gy) * g.batch;
-    const long long steps = (long long)((g.K + BK - 1) / BK) * g.kb;
-    const long long slots = 2LL * std::max(ctx.num_sms, 1);
+    p.batch = g.batch;
+    const long long gx = (g.N + BT - 1) / BT, gy = (g.M + BT - 1) / BT;
+    VTN_REQUIRE(gy <= 4 * 65535LL, "gemm M too large");
+    const double macs = (double)g.M * g.N * g.K * g.kb * g.batch * (g.herm_lower ? 0.5 : 1.0);
+    // The sliced product costs four launches, about 34 us, and then runs 35 times faster.  Measured, DFMA
+    // against sliced: 128^3 22 | 34 us, 160^3 34 | 35 us, 192^3 55 | 37 us, 256^3 136 | 38 us, 1024 x 16 x 1024
+    // (narrow: padded to 32 columns) 74 | 49 us; at 3072^3 200 ms against 6.1 ms.  Its row sums fit 96-bit integers
+    // for summations of up to 2^19 terms.
+    const bool oz = ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.5e6 && (long long)g.K * g.kb <= (1LL << 19);
     int S = 1;
-    if (tiles < slots) S = (int)std::min<long long>({slots / tiles, steps / 16, 32LL, 65535LL / g.batch});
+    if (oz) {
+        S = oz_splits(ctx, g);
+    } else {
+        // output tiles that do work; split the summation when they leave SMs short of 2 CTAs
+        const long long tiles = (g.herm_lower ? gy * (gy + 1) / 2 : gx * gy) * g.batch;
+        // (a share of fewer than 128 terms costs more in the second pass than it saves)
+        const long long slots = 2LL * std::max(ctx.num_sms, 1);
+        if (tiles < slots) S = (int)std::min<long long>({slots / tiles, (long long)g.K * g.kb / 128, 32LL});
+    }
     if (g.max_splits > 0) S = std::min(S, g.max_splits);
     S = std::max(S, 1);
     p.splits = S;
     p.part = nullptr;
     if (S > 1)
         p.part = (double2*)ctx.workspace(WS_GEMM_SPLIT, sizeof(double2) * (size_t)S * g.batch * g.M * g.N);
-    dim3 grid(gx, gy, g.batch * S);
+    const long long ctas = gx * gy * g.batch * S;
+    VTN_REQUIRE(oz || ctas < (1LL << 31), "gemm too large");
     double flops = 8.0 * g.M * (double)g.N * g.K * g.kb * g.batch * (g.herm_lower ? 0.5 : 1.0);
     int t0 = ctx.tbegin(TC_GEMM, flops);
     int t1 = (timing_class != TC_GEMM) ? ctx.tbegin(timing_class, flops) : -1;
-    gemm_c64_kernel<<<grid, NT, 0, ctx.stream>>>(p);
-    ctx.count_launch();
-    ctx.check_launch("gemm_c64_kernel");
+    if (oz) {
+        oz_gemm(ctx, g, S, p.part);
+    } else {
+        gemm_c64_kernel<<<(unsigned)ctas, NT, 0, ctx.stream>>>(p);
+        ctx.count_launch();
+        ctx.check_launch("gemm_c64_kernel");
+    }
     if (S > 1) {
         const long long cnt = (long long)g.batch * g.M * g.N;
         splitk_sum<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx.stream>>>(p, g.batch);

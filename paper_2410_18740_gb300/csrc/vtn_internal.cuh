@@ -148,7 +148,8 @@ enum WsSlot {
     WS_EIG_Y, WS_EIG_WORK, WS_EIG_U, WS_CORE_A, WS_CORE_B, WS_ENV_TMP, WS_MISC, WS_TC_L, WS_TC_R, WS_TC_B1,
     WS_TC_A2, WS_TC_PART, WS_GEMM_SPLIT, WS_EIG_PART, WS_TC_ENV, WS_EIG_T, WS_H2_ENV, WS_EXPAND,
     WS_TRUNC_L, WS_TRUNC_R, WS_CENTER, WS_MLP_ACT, WS_MLP_Y, WS_MLP_G, WS_WARM_S, WS_WARM_Z, WS_WARM_P,
-    WS_WARM_U, WS_WARM_N, WS_WARM_Q0, WS_CQR_G, WS_CQR_T, WS_CQR_B, WS_RQ_Y, WS_RQ_S, WS_CHOL_LINV, WS_TH_A, WS_TH_B, WS_COUNT
+    WS_WARM_U, WS_WARM_N, WS_WARM_Q0, WS_CQR_G, WS_CQR_T, WS_CQR_B, WS_RQ_Y, WS_RQ_S, WS_CHOL_LINV, WS_TH_A, WS_TH_B,
+    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_COUNT
 };
 
 // ------------------------------------------------------------------ cores
@@ -176,6 +177,11 @@ struct GemmArgs {
 // C[i][j] = conj(C[j][i]) for j > i (n x n, leading dimension ldc)
 void mirror_lower_to_upper(Ctx& ctx, double2* C, int n, long long ldc);
 void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class = TC_GEMM);
+
+// The same product on the tensor cores by exact integer slices (oz_gemm.cu); gemm_c64 chooses.  splits > 1:
+// partial tiles [splits][batch][M][N] go to `part` instead of C.
+int oz_splits(const Ctx& ctx, const GemmArgs& g);
+void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part);
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize, bytes) for kernel fn on the context's
 // device, once per (kernel, device) (the attribute is per device); thread-safe.

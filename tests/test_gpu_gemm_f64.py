@@ -1,0 +1,110 @@
+"""FP64 GEMM on the tensor cores by exact integer slices (csrc/oz_gemm.cu) against exact rational sums.
+
+Reached through vtn_heff_apply with one-channel identity cores of local dimension 1: y = L theta R.  With
+R = I the second product is exact, so y is one product of the sizes asked for."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _product(ctx, L, th, R=None):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    one = vtn.make_core(1, 1, 1, [0], [0], np.ones((1, 1, 1), complex))
+    m, n = L.shape[0], th.shape[1]
+    R = torch.eye(n, dtype=torch.complex128, device="cuda") if R is None else R
+    y = torch.full((m, n), 7.0, dtype=torch.complex128, device="cuda")
+    vtn.vtn_heff_apply(ctx, one, one, m, n, L, R, th, y)
+    torch.cuda.synchronize()
+    return y
+
+
+def _randn(rng, *shape):
+    import torch
+    return torch.from_numpy(rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).cuda()
+
+
+def _worst(L, th, y, rng, count=20):
+    """Largest error of sampled entries over its bound: one rounding of the result and one of the second
+    (exact) product, and the digit pairs left out: below 2^-61 (largest of the row) (largest of the column) a
+    term, which the scaling keeps within 2^5 of the largest term of the sum."""
+    L, th, y = (t.cpu().numpy() for t in (L, th, y))
+    K = L.shape[1]
+    term = float(np.max(np.abs(L.view(float)).reshape(L.shape + (2,)).max((0, 2)) * np.abs(th.view(float)).reshape(th.shape + (2,)).max((1, 2))))
+    worst = 0.0
+    at = [(0, 0), (L.shape[0] - 1, th.shape[1] - 1)] + [(int(rng.integers(L.shape[0])), int(rng.integers(th.shape[1]))) for _ in range(count)]
+    for i, j in at:
+        re = im = Fraction(0)
+        for k in range(K):
+            ar, ai, br, bi = (Fraction(float(v)) for v in (L[i, k].real, L[i, k].imag, th[k, j].real, th[k, j].imag))
+            re += ar * br - ai * bi
+            im += ar * bi + ai * br
+        for got, want in ((y[i, j].real, re), (y[i, j].imag, im)):
+            bound = 2.0 ** -52 * abs(float(want)) + 4 * K * 2.0 ** -56 * term
+            worst = max(worst, abs(float(Fraction(float(got)) - want)) / bound)
+    return worst
+
+
+# rows, columns: around the 128 x 32 tiles, the 16-element summation stages, the drains after 4, 8 and 16
+# stages, and a summation long enough to be split over the CTAs
+@pytest.mark.parametrize("m,n", [(256, 129), (257, 128), (383, 65), (400, 33), (512, 31), (641, 32), (1040, 16), (2300, 3)])
+def test_sliced_product_is_exact_to_one_rounding(ctx, m, n):
+    rng = np.random.default_rng(m * 31 + n)
+    L, th = _randn(rng, m, m), _randn(rng, m, n)
+    assert _worst(L, th, _product(ctx, L, th), rng) <= 1.0
+
+
+@pytest.mark.parametrize("value", [float.fromhex("0x1.fefefefefefefp0"), float.fromhex("0x1.ff7f7f7f7f7f7p0"),
+                                   float.fromhex("0x1.0101010101010p0"), 2.0 - 2.0 ** -52, -1.0 / 3.0])
+def test_sliced_product_with_the_largest_digits(ctx, value):
+    """All terms of one sign and every digit as large as it gets: the FP32 partial sums reach 2^24."""
+    import torch
+    L = torch.full((1100, 1100), complex(value, value), dtype=torch.complex128, device="cuda")
+    th = torch.full((1100, 40), complex(value, -value), dtype=torch.complex128, device="cuda")
+    assert _worst(L, th, _product(ctx, L, th), np.random.default_rng(0), count=2) <= 1.0
+
+
+def test_sliced_product_of_opposed_gradings(ctx):
+    """Columns of the left and rows of the right operand graded against each other over 28 decades."""
+    import torch
+    rng = np.random.default_rng(5)
+    g = torch.logspace(0, -28, 400, dtype=torch.float64, device="cuda")
+    L, th = _randn(rng, 400, 400) * g[None, :], _randn(rng, 400, 64) * g.flip(0)[:, None]
+    assert _worst(L, th, _product(ctx, L, th), rng) <= 1.0
+
+
+def test_sliced_product_with_non_finite_rows_and_extreme_scales(ctx):
+    import torch
+    rng = np.random.default_rng(9)
+    L, th = _randn(rng, 400, 400), _randn(rng, 400, 64)
+    L[17] = 0
+    clean = _product(ctx, L, th)
+    bad = L.clone()
+    bad[3, 5] = float("inf")
+    bad[399, 7] = complex(0.0, float("nan"))
+    got = _product(ctx, bad, th)
+    rows = torch.ones(400, dtype=torch.bool)
+    rows[[3, 399]] = False
+    assert torch.equal(got[rows], clean[rows]) and bool((clean[17] == 0).all())
+    assert not bool(torch.isfinite(torch.view_as_real(got[~rows])).all(-1).any())
+    for s in (2.0 ** -600, 2.0 ** 500):  # powers of two: the same digits
+        assert torch.equal(_product(ctx, L * s, th), clean * s)
+
+
+def test_sliced_products_of_the_environment_updates(ctx):
+    """Conjugated, batched and channel-shared operands, both sides, against plain FP64."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(11)
+    w, d, cl, cr = 3, 2, 150, 171
+    core = vtn.make_core(w, w, d, range(w), range(w), np.array([np.eye(d)] * w, complex))
+    A = _randn(rng, cl, d, cr)
+    for side, ci, co in ((0, cl, cr), (1, cr, cl)):
+        E, out = _randn(rng, w, ci, ci), torch.empty(w, co, co, dtype=torch.complex128, device="cuda")
+        vtn.vtn_env_update(ctx, core, side, cl, cr, E, A, out)
+        ref = torch.einsum("itl,aij,jtk->alk", A.conj(), E, A) if side == 0 else torch.einsum("jtg,agp,itp->aji", A, E, A.conj())
+        # two products of lengths ci and d * (the other): the reference's own rounding, u sqrt(K) each, with room
+        assert float(torch.linalg.norm(out - ref) / torch.linalg.norm(ref)) <= 1e-14
