@@ -166,7 +166,7 @@ void destroy_mps(vtn_mps m) {
 struct TempCore {
     Ctx* c;
     DevCore dc;
-    TempCore(Ctx& ctx, const HostCore& h) : c(&ctx) { upload_core(ctx, h, dc); }
+    TempCore(Ctx& ctx, const HostCore& h, bool fp64 = true) : c(&ctx) { upload_core(ctx, h, dc, fp64); }
     ~TempCore() {
         if (c) {
             cudaStreamSynchronize(c->stream);
@@ -1753,7 +1753,7 @@ vtn_status vtn_heff_apply(vtn_ctx ctx, const vtn_core* Wi, const vtn_core* Wj, i
         use_device(c);
         HostCore hi = core_from_abi(Wi), hj = core_from_abi(Wj);
         VTN_REQUIRE(hi.wr == hj.wl && hi.d == hj.d, "Wi.w_right must equal Wj.w_left and d must agree");
-        TempCore ci(c, hi), cj(c, hj);
+        TempCore ci(c, hi, prec == VTN_FP64), cj(c, hj, prec == VTN_FP64);
         if (prec == VTN_BF16X3) {
             TempTerms tt(c, hi, hj);
             HeffPacked pk;
@@ -1782,7 +1782,7 @@ vtn_status vtn_env_update(vtn_ctx ctx, const vtn_core* W, int side, int chi_l, i
         Ctx& c = ctx->c;
         use_device(c);
         HostCore h = core_from_abi(W);
-        TempCore tc(c, h);
+        TempCore tc(c, h, prec == VTN_FP64);
         const double2* e = (const double2*)env;
         const double2* a = (const double2*)A;
         double2* o = (double2*)out;

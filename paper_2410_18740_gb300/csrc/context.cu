@@ -158,7 +158,7 @@ HostCore core_from_abi(const vtn_core* c) {
     return h;
 }
 
-void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc) {
+void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
     dc.wl = hc.wl;
     dc.wr = hc.wr;
     dc.d = hc.d;
@@ -210,6 +210,30 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc) {
         group(true, true, dcp, dcs, dco);
         group(false, true, drp, drs, dro);
     }
+    // spelled-out terms (FP64 mixing): the groups' entries in order, then the operator's row in order
+    std::vector<int> nzp[2];
+    std::vector<unsigned> nzs[2];
+    std::vector<cplx> nzc[2];
+    for (int dir = 0; dir < (fp64 ? 2 : 0); ++dir) {
+        const std::vector<int>&ptr = dir == 0 ? col_ptr : row_ptr, &src = dir == 0 ? col_src : row_src,
+                              &op = dir == 0 ? col_op : row_op;
+        const int w_out = dir == 0 ? hc.wr : hc.wl;
+        nzp[dir].push_back(0);
+        dc.nz_fma[dir] = 0;
+        for (int b = 0; b < w_out; ++b)
+            for (int sp = 0; sp < d; ++sp) {
+                for (int e = ptr[b]; e < ptr[b + 1]; ++e)
+                    for (int t = 0; t < d; ++t) {
+                        const cplx c = hc.ops[(size_t)op[e] * d * d + sp * d + t];
+                        if (c == cplx(0, 0)) continue;
+                        const unsigned kind = c == cplx(1, 0) ? MIX_ONE : c.imag() == 0.0 ? MIX_REAL : c.real() == 0.0 ? MIX_IMAG : MIX_CPLX;
+                        nzs[dir].push_back((unsigned)(src[e] * d + t) | (kind << 30));
+                        nzc[dir].push_back(c);
+                        dc.nz_fma[dir] += kind == MIX_CPLX ? 4 : 2;
+                    }
+                nzp[dir].push_back((int)nzs[dir].size());
+            }
+    }
     // one allocation holding everything
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
@@ -222,6 +246,12 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc) {
                  o_cid = take(sizeof(float) * std::max(cid.size(), size_t(1))), o_dcp = take(ibytes(dcp)),
                  o_dcs = take(ibytes(dcs)), o_dco = take(ibytes(dco)), o_drp = take(ibytes(drp)),
                  o_drs = take(ibytes(drs)), o_dro = take(ibytes(dro));
+    size_t o_nzp[2], o_nzs[2], o_nzc[2];
+    for (int i = 0; i < 2; ++i) {
+        o_nzp[i] = take(ibytes(nzp[i]));
+        o_nzs[i] = take(sizeof(unsigned) * std::max(nzs[i].size(), size_t(1)));
+        o_nzc[i] = take(sizeof(double2) * std::max(nzc[i].size(), size_t(1)));
+    }
     std::vector<unsigned char> blob(off, 0);
     auto put = [&](size_t o, const void* p, size_t bytes) {
         if (bytes) std::memcpy(&blob[o], p, bytes);
@@ -250,6 +280,11 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc) {
     puti(o_drp, drp);
     puti(o_drs, drs);
     puti(o_dro, dro);
+    for (int i = 0; i < 2; ++i) {
+        puti(o_nzp[i], nzp[i]);
+        put(o_nzs[i], nzs[i].data(), sizeof(unsigned) * nzs[i].size());
+        put(o_nzc[i], nzc[i].data(), sizeof(double2) * nzc[i].size());
+    }
     DevBuf b;
     b.bytes = off;
     b.p = ctx.dalloc(off);
@@ -265,6 +300,11 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc) {
     dc.ops = (double2*)(base + o_ops);
     dc.ident = base + o_id;
     dc.ops_f32 = (float2*)(base + o_f32);
+    for (int i = 0; i < (fp64 ? 2 : 0); ++i) {
+        dc.nz_ptr[i] = (int*)(base + o_nzp[i]);
+        dc.nz_src[i] = (unsigned*)(base + o_nzs[i]);
+        dc.nz_c[i] = (double2*)(base + o_nzc[i]);
+    }
     if (dc.has_cid) {
         dc.cid = (float2*)(base + o_cid);
         dc.dcol_ptr = (int*)(base + o_dcp);

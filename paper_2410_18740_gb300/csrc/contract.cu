@@ -65,6 +65,45 @@ __global__ void __launch_bounds__(256) mix_kernel(int P, int d, int Q, const int
         if (sp < d) y[(long long)sp * Q] = acc[sp];
 }
 
+// The same from the spelled-out terms: one output (channel, level, p, q) per thread.  FP64-issue bound, so
+// a term costs what its coefficient needs: two FMAs when real or imaginary (most entries of the GBS cores: x is
+// real, p imaginary, couplings real), four when complex, and none for a lone pass-through channel, which
+// is a copy.  Zero entries of the d x d operators (x and p have two a row) are not visited.  The terms keep
+// the order of the dense loop above, so the sums are the same.  The terms are the same for all threads of a
+// block; their inputs come from L2 (each is used by a few outputs).
+__global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int Q, const int* __restrict__ ptr,
+                                                        const unsigned* __restrict__ src,
+                                                        const double2* __restrict__ coef,
+                                                        const double2* __restrict__ in, double2* __restrict__ out) {
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    const int o = blockIdx.y;
+    if (t >= PQ) return;
+    const long long p = t / Q, q = t % Q;
+    const long long blk = PQ * d, at = p * d * Q + q;
+    const int e0 = ptr[o], e1 = ptr[o + 1];
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int e = e0; e < e1; ++e) {
+        const unsigned s = src[e];
+        const int ch = (int)(s & 0x3fffffffu);
+        const double2 x = in[(long long)(ch / d) * blk + at + (long long)(ch % d) * Q];
+        const double2 c = coef[e];
+        const unsigned kind = s >> 30;
+        if (kind == MIX_ONE && e == e0) {
+            acc = x;
+        } else if (kind == MIX_REAL || kind == MIX_ONE) {
+            acc.x = fma(c.x, x.x, acc.x);
+            acc.y = fma(c.x, x.y, acc.y);
+        } else if (kind == MIX_IMAG) {
+            acc.x = fma(-c.y, x.y, acc.x);
+            acc.y = fma(c.y, x.x, acc.y);
+        } else {
+            cfma(acc, c, x);
+        }
+    }
+    out[(long long)(o / d) * blk + at + (long long)(o % d) * Q] = acc;
+}
+
 }  // namespace
 
 void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const double2* in, double2* out) {
@@ -80,7 +119,11 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
     // flops: identity entries d complex MACs, dense entries d^2, per (p, q)
     double fl = 8.0 * PQ * ((double)core.n_ident * d + (double)core.n_dense * d * d);
     int t = ctx.tbegin(TC_MIX, fl);
-    if (d <= 4)
+    const int dir = by_col ? 0 : 1;
+    if (core.nz_ptr[dir] != nullptr && (long long)w_out * d <= 65535)
+        mix_terms_kernel<<<dim3((unsigned)((PQ + 255) / 256), w_out * d), 256, 0, ctx.stream>>>(
+            PQ, d, Q, core.nz_ptr[dir], core.nz_src[dir], core.nz_c[dir], in, out);
+    else if (d <= 4)
         mix_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, ptr, src, opi, core.ops, core.ident, in, out);
     else if (d <= 8)
         mix_kernel<8><<<grid, 256, 0, ctx.stream>>>(P, d, Q, ptr, src, opi, core.ops, core.ident, in, out);

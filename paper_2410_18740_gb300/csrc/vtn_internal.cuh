@@ -89,8 +89,16 @@ struct DevCore {
     float2* cid = nullptr;
     int *dcol_ptr = nullptr, *dcol_src = nullptr, *dcol_op = nullptr;
     int *drow_ptr = nullptr, *drow_src = nullptr, *drow_op = nullptr;
+    // the same entries spelled out per output element (channel, level) in the order of the lists above, zero
+    // coefficients dropped: term t of output o adds nz_c[t] * in[nz_src[t]], nz_src = channel * d + level with
+    // the coefficient's kind (MixTerm) in the two topmost bits; [0] by column, [1] by row
+    int* nz_ptr[2] = {nullptr, nullptr};       // [w_out * d + 1]
+    unsigned* nz_src[2] = {nullptr, nullptr};
+    double2* nz_c[2] = {nullptr, nullptr};
+    double nz_fma[2] = {0, 0};                 // FP64 operations per (p, q) element
     std::vector<DevBuf> bufs;
 };
+enum MixTerm : unsigned { MIX_REAL = 0u, MIX_IMAG = 1u, MIX_CPLX = 2u, MIX_ONE = 3u };  // c = 1: the input as it is
 
 struct Ctx {
     int device = 0;
@@ -153,7 +161,8 @@ enum WsSlot {
 };
 
 // ------------------------------------------------------------------ cores
-void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc);
+// fp64 = false leaves out the spelled-out terms of the FP64 mixing
+void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64 = true);
 void free_core(Ctx& ctx, DevCore& dc);
 HostCore core_from_abi(const vtn_core* c);
 

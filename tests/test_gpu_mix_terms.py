@@ -1,0 +1,54 @@
+"""FP64 core mixing from spelled-out terms: every kind of coefficient, empty channels, both directions."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _core(rng, w_l, w_r, d):
+    """Dense W[a, b, s', s] with pass-through, scaled, real, imaginary, complex and banded blocks; column w_r - 1
+    and row w_l - 1 are empty."""
+    W = np.zeros((w_l, w_r, d, d), complex)
+    band = np.triu(np.tril(np.ones((d, d)), 1), -1) - np.eye(d)
+    kinds = [np.eye(d), -1.75 * np.eye(d), band * rng.standard_normal((d, d)), 1j * band * rng.standard_normal((d, d)),
+             rng.standard_normal((d, d)) + 1j * rng.standard_normal((d, d)), 1j * np.eye(d), np.diag(np.arange(d) + 1.0)]
+    n = 0
+    for a in range(w_l - 1):
+        for b in range(w_r - 1):
+            if a == b or rng.random() < 0.5:
+                W[a, b] = kinds[n % len(kinds)]
+                n += 1
+    return W
+
+
+@pytest.mark.parametrize("d,cl,cr", [(1, 5, 9), (2, 1, 1), (3, 17, 5), (6, 9, 31), (8, 16, 33), (16, 3, 4)])
+def test_spelled_out_terms_match_the_dense_core(ctx, d, cl, cr):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(100 * d + cl)
+    wl, wm, wr = 4, 5, 3
+    Wi, Wj = _core(rng, wl, wm, d), _core(rng, wm, wr, d)
+    z = lambda *s: torch.from_numpy(rng.standard_normal(s) + 1j * rng.standard_normal(s)).cuda()
+    t = lambda W: torch.from_numpy(W).cuda()
+    L, R, th = z(wl, cl, cl), z(wr, cr, cr), z(cl, d, d, cr)
+    y = torch.empty_like(th)
+    vtn.vtn_heff_apply(ctx, vtn.core_from_dense(Wi), vtn.core_from_dense(Wj), cl, cr, L, R, th, y)
+    T = torch.einsum("aij,jsvk->aisvk", L, th)
+    T = torch.einsum("abts,aisvk->bitvk", t(Wi), T)
+    T = torch.einsum("bcuv,bitvk->cituk", t(Wj), T)
+    ref = torch.einsum("cituk,ckl->itul", T, R)
+    # four contractions of at most w d chi terms, u sqrt(terms) each, with room
+    assert float(torch.linalg.norm(y - ref)) <= 1e-14 * float(torch.linalg.norm(ref)) + 1e-300
+    for side, ci, co, w_in, w_out in ((0, cl, cr, wl, wm), (1, cr, cl, wm, wl)):
+        A, E = z(cl, d, cr), z(w_in, ci, ci)
+        out = torch.empty(w_out, co, co, dtype=torch.complex128, device="cuda")
+        vtn.vtn_env_update(ctx, vtn.core_from_dense(Wi), side, cl, cr, E, A, out)
+        if side == 0:
+            U = torch.einsum("abts,aisk->bitk", t(Wi), torch.einsum("aij,jsk->aisk", E, A))
+            ref = torch.einsum("itl,bitk->blk", A.conj(), U)
+            assert bool((out[-1] == 0).all())
+        else:
+            U = torch.einsum("abts,bjsp->ajtp", t(Wi), torch.einsum("jsg,bgp->bjsp", A, E))
+            ref = torch.einsum("ajtp,itp->aji", U, A.conj())
+            assert bool((out[-1] == 0).all())
+        assert float(torch.linalg.norm(out - ref)) <= 1e-14 * float(torch.linalg.norm(ref)) + 1e-300
