@@ -211,15 +211,16 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
         group(false, true, drp, drs, dro);
     }
     // spelled-out terms (FP64 mixing): the groups' entries in order, then the operator's row in order
-    std::vector<int> nzp[2];
-    std::vector<unsigned> nzs[2];
-    std::vector<cplx> nzc[2];
-    for (int dir = 0; dir < (fp64 ? 2 : 0); ++dir) {
-        const std::vector<int>&ptr = dir == 0 ? col_ptr : row_ptr, &src = dir == 0 ? col_src : row_src,
-                              &op = dir == 0 ? col_op : row_op;
-        const int w_out = dir == 0 ? hc.wr : hc.wl;
+    std::vector<int> nzp[4];
+    std::vector<unsigned> nzs[4];
+    std::vector<cplx> nzc[4], cid64;
+    for (int dir = 0; dir < (fp64 ? (dc.has_cid ? 4 : 2) : 0); ++dir) {
+        const bool by_col = (dir & 1) == 0;
+        const std::vector<int>&ptr = dir == 0 ? col_ptr : dir == 1 ? row_ptr : dir == 2 ? dcp : drp,
+                              &src = dir == 0 ? col_src : dir == 1 ? row_src : dir == 2 ? dcs : drs,
+                              &op = dir == 0 ? col_op : dir == 1 ? row_op : dir == 2 ? dco : dro;
+        const int w_out = by_col ? hc.wr : hc.wl;
         nzp[dir].push_back(0);
-        dc.nz_fma[dir] = 0;
         for (int b = 0; b < w_out; ++b)
             for (int sp = 0; sp < d; ++sp) {
                 for (int e = ptr[b]; e < ptr[b + 1]; ++e)
@@ -229,10 +230,14 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
                         const unsigned kind = c == cplx(1, 0) ? MIX_ONE : c.imag() == 0.0 ? MIX_REAL : c.real() == 0.0 ? MIX_IMAG : MIX_CPLX;
                         nzs[dir].push_back((unsigned)(src[e] * d + t) | (kind << 30));
                         nzc[dir].push_back(c);
-                        dc.nz_fma[dir] += kind == MIX_CPLX ? 4 : 2;
                     }
                 nzp[dir].push_back((int)nzs[dir].size());
             }
+    }
+    if (fp64 && dc.has_cid) {
+        cid64.assign((size_t)hc.wl * hc.wr, cplx(0, 0));
+        for (int k = 0; k < nnz; ++k)
+            if (hc.ident[k]) cid64[(size_t)hc.rows[k] * hc.wr + hc.cols[k]] += hc.ops[(size_t)k * d * d];
     }
     // one allocation holding everything
     size_t off = 0;
@@ -246,8 +251,9 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
                  o_cid = take(sizeof(float) * std::max(cid.size(), size_t(1))), o_dcp = take(ibytes(dcp)),
                  o_dcs = take(ibytes(dcs)), o_dco = take(ibytes(dco)), o_drp = take(ibytes(drp)),
                  o_drs = take(ibytes(drs)), o_dro = take(ibytes(dro));
-    size_t o_nzp[2], o_nzs[2], o_nzc[2];
-    for (int i = 0; i < 2; ++i) {
+    const size_t o_cid64 = take(sizeof(double2) * std::max(cid64.size(), size_t(1)));
+    size_t o_nzp[4], o_nzs[4], o_nzc[4];
+    for (int i = 0; i < 4; ++i) {
         o_nzp[i] = take(ibytes(nzp[i]));
         o_nzs[i] = take(sizeof(unsigned) * std::max(nzs[i].size(), size_t(1)));
         o_nzc[i] = take(sizeof(double2) * std::max(nzc[i].size(), size_t(1)));
@@ -280,7 +286,8 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
     puti(o_drp, drp);
     puti(o_drs, drs);
     puti(o_dro, dro);
-    for (int i = 0; i < 2; ++i) {
+    put(o_cid64, cid64.data(), sizeof(double2) * cid64.size());
+    for (int i = 0; i < 4; ++i) {
         puti(o_nzp[i], nzp[i]);
         put(o_nzs[i], nzs[i].data(), sizeof(unsigned) * nzs[i].size());
         put(o_nzc[i], nzc[i].data(), sizeof(double2) * nzc[i].size());
@@ -300,7 +307,8 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
     dc.ops = (double2*)(base + o_ops);
     dc.ident = base + o_id;
     dc.ops_f32 = (float2*)(base + o_f32);
-    for (int i = 0; i < (fp64 ? 2 : 0); ++i) {
+    if (fp64 && dc.has_cid) dc.cid64 = (double2*)(base + o_cid64);
+    for (int i = 0; i < (fp64 ? (dc.has_cid ? 4 : 2) : 0); ++i) {
         dc.nz_ptr[i] = (int*)(base + o_nzp[i]);
         dc.nz_src[i] = (unsigned*)(base + o_nzs[i]);
         dc.nz_c[i] = (double2*)(base + o_nzc[i]);

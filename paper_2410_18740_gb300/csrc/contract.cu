@@ -71,6 +71,8 @@ __global__ void __launch_bounds__(256) mix_kernel(int P, int d, int Q, const int
 // is a copy.  Zero entries of the d x d operators (x and p have two a row) are not visited.  The terms keep
 // the order of the dense loop above, so the sums are the same.  The terms are the same for all threads of a
 // block; their inputs come from L2 (each is used by a few outputs).
+// ACC: added to the output instead of replacing it (outputs without a term keep what they hold).
+template <bool ACC>
 __global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int Q, const int* __restrict__ ptr,
                                                         const unsigned* __restrict__ src,
                                                         const double2* __restrict__ coef,
@@ -81,7 +83,9 @@ __global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int
     const long long p = t / Q, q = t % Q;
     const long long blk = PQ * d, at = p * d * Q + q;
     const int e0 = ptr[o], e1 = ptr[o + 1];
-    double2 acc = make_double2(0.0, 0.0);
+    if (ACC && e0 == e1) return;
+    double2* y = out + (long long)(o / d) * blk + at + (long long)(o % d) * Q;
+    double2 acc = ACC ? *y : make_double2(0.0, 0.0);
 #pragma unroll 4
     for (int e = e0; e < e1; ++e) {
         const unsigned s = src[e];
@@ -89,7 +93,7 @@ __global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int
         const double2 x = in[(long long)(ch / d) * blk + at + (long long)(ch % d) * Q];
         const double2 c = coef[e];
         const unsigned kind = s >> 30;
-        if (kind == MIX_ONE && e == e0) {
+        if (!ACC && kind == MIX_ONE && e == e0) {
             acc = x;
         } else if (kind == MIX_REAL || kind == MIX_ONE) {
             acc.x = fma(c.x, x.x, acc.x);
@@ -101,7 +105,7 @@ __global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int
             cfma(acc, c, x);
         }
     }
-    out[(long long)(o / d) * blk + at + (long long)(o % d) * Q] = acc;
+    *y = acc;
 }
 
 }  // namespace
@@ -120,9 +124,27 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
     double fl = 8.0 * PQ * ((double)core.n_ident * d + (double)core.n_dense * d * d);
     int t = ctx.tbegin(TC_MIX, fl);
     const int dir = by_col ? 0 : 1;
-    if (core.nz_ptr[dir] != nullptr && (long long)w_out * d <= 65535)
-        mix_terms_kernel<<<dim3((unsigned)((PQ + 255) / 256), w_out * d), 256, 0, ctx.stream>>>(
-            PQ, d, Q, core.nz_ptr[dir], core.nz_src[dir], core.nz_c[dir], in, out);
+    const bool terms = core.nz_ptr[dir] != nullptr && (long long)w_out * d <= 65535;
+    const dim3 tgrid((unsigned)((PQ + 255) / 256), w_out * d);
+    const long long E = PQ * d;
+    // A collapse core couples all channels to all: its scaled identities are a channel product
+    // out[b][e] = sum_a C[a][b] in[a][e], which the FP64 pipe does at two operations a coupling and element (0.49e12
+    // a second) and the sliced GEMM (rows e, padded to 16 channels a stage) at 0.13 us per 128 elements and
+    // stage plus 35 us: the split workload's centre core at chi = 128 takes 2.6 against 1.1 ms.
+    const double stages = ((by_col ? core.wl : core.wr) + 15) / 16;
+    if (terms && core.cid64 != nullptr && ctx.dstatus != nullptr && E < (1LL << 30) && w_out <= 1024 &&
+        2.0 * core.n_ident * E / 0.49e12 > 1.2 * (35e-6 + E / 128.0 * (stages * 0.05e-6 + 0.03e-6))) {
+        GemmArgs g;
+        g.M = (int)E; g.N = w_out; g.K = by_col ? core.wl : core.wr;
+        g.opA = OP_T; g.A = in; g.lda = E;
+        g.opB = by_col ? OP_N : OP_T; g.B = core.cid64; g.ldb = core.wr;
+        g.C = out; g.ldc = 1; g.sC_n = E;
+        oz_gemm(ctx, g, 1, nullptr);
+        mix_terms_kernel<true><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, core.nz_ptr[2 + dir], core.nz_src[2 + dir],
+                                                              core.nz_c[2 + dir], in, out);
+    } else if (terms)
+        mix_terms_kernel<false><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, core.nz_ptr[dir], core.nz_src[dir],
+                                                               core.nz_c[dir], in, out);
     else if (d <= 4)
         mix_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, ptr, src, opi, core.ops, core.ident, in, out);
     else if (d <= 8)

@@ -72,7 +72,7 @@ struct OzParams {
     int M, N, nkb;
     int tiles_m, tiles_n, batch, splits, kb_per;
     double2* C;
-    long long ldc, sC_batch;
+    long long ldc, sC_n, sC_batch;
     double2* part;
     int accumulate, negate, herm_lower;
     int* status;
@@ -582,7 +582,8 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             if (!ok) break;
             const bool to_part = p.splits > 1;
             double2* C = to_part ? p.part + ((long long)z * p.batch + bz) * p.M * p.N : p.C + (long long)bz * p.sC_batch;
-            double2* dst = C + (long long)m * (to_part ? p.N : p.ldc) + n0;
+            const long long cn = to_part ? 1 : p.sC_n;
+            double2* dst = C + (long long)m * (to_part ? p.N : p.ldc) + n0 * cn;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int en = __shfl_sync(0xffffffffu, eb, j);
@@ -596,11 +597,11 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 }
                 if (p.negate) r = make_double2(-r.x, -r.y);
                 if (p.accumulate && !to_part) {
-                    const double2 o = dst[j];
+                    const double2 o = dst[j * cn];
                     r.x += o.x;
                     r.y += o.y;
                 }
-                dst[j] = r;
+                dst[j * cn] = r;
             }
         }
     }
@@ -666,9 +667,9 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                         o.X = g.A + b0 * g.sA_batch + (g.opA == OP_N ? m0 * g.lda : m0);
                         o.rows = mm; o.tiles = p.tiles_m; o.nb = a_shared ? 1 : nb;
                     } else {
-                        o.kc = g.opB == OP_C; o.conj = g.opB == OP_C;
+                        o.kc = g.opB != OP_N; o.conj = g.opB == OP_C;
                         o.ld = g.ldb; o.s_batch = g.sB_batch; o.s_kb = g.sB_kb;
-                        o.X = g.B + b0 * g.sB_batch + (g.opB == OP_C ? n0 * g.ldb : n0);
+                        o.X = g.B + b0 * g.sB_batch + (g.opB != OP_N ? n0 * g.ldb : n0);
                         o.rows = nn; o.tiles = p.tiles_n; o.nb = b_shared ? 1 : nb;
                     }
                 };
@@ -683,8 +684,8 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 p.b.kx = p.a.kx + nk;
                 p.a.out = (uint4*)ctx.workspace(WS_OZ_A, (size_t)p.a.nb * p.tiles_m * nkb * A_BYTES);
                 p.b.out = (uint4*)ctx.workspace(WS_OZ_B, (size_t)p.b.nb * p.tiles_n * nkb * B_BYTES);
-                p.C = g.C + b0 * g.sC_batch + m0 * g.ldc + n0;
-                p.ldc = g.ldc; p.sC_batch = g.sC_batch;
+                p.C = g.C + b0 * g.sC_batch + m0 * g.ldc + n0 * g.sC_n;
+                p.ldc = g.ldc; p.sC_n = g.sC_n; p.sC_batch = g.sC_batch;
                 p.part = part;
                 p.accumulate = g.accumulate; p.negate = g.negate; p.herm_lower = g.herm_lower;
                 p.status = ctx.dstatus;

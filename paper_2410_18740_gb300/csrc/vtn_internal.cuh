@@ -92,10 +92,11 @@ struct DevCore {
     // the same entries spelled out per output element (channel, level) in the order of the lists above, zero
     // coefficients dropped: term t of output o adds nz_c[t] * in[nz_src[t]], nz_src = channel * d + level with
     // the coefficient's kind (MixTerm) in the two topmost bits; [0] by column, [1] by row
-    int* nz_ptr[2] = {nullptr, nullptr};       // [w_out * d + 1]
-    unsigned* nz_src[2] = {nullptr, nullptr};
-    double2* nz_c[2] = {nullptr, nullptr};
-    double nz_fma[2] = {0, 0};                 // FP64 operations per (p, q) element
+    // ([2], [3]: those of a collapse core without its scaled identities, which cid64 holds)
+    int* nz_ptr[4] = {};       // [w_out * d + 1]
+    unsigned* nz_src[4] = {};
+    double2* nz_c[4] = {};
+    double2* cid64 = nullptr;  // C[a][b] in FP64
     std::vector<DevBuf> bufs;
 };
 enum MixTerm : unsigned { MIX_REAL = 0u, MIX_IMAG = 1u, MIX_CPLX = 2u, MIX_ONE = 3u };  // c = 1: the input as it is
@@ -167,7 +168,7 @@ void free_core(Ctx& ctx, DevCore& dc);
 HostCore core_from_abi(const vtn_core* c);
 
 // ------------------------------------------------------------------ GEMM (complex FP64)
-enum Op { OP_N = 0, OP_C = 1 };  // op(X) = X or X^dag (conjugate transpose)
+enum Op { OP_N = 0, OP_C = 1, OP_T = 2 };  // op(X) = X, X^dag (conjugate transpose) or (oz_gemm only) X^T
 
 struct GemmArgs {
     int M, N, K;          // op(A): M x K, op(B): K x N, C: M x N
@@ -177,6 +178,7 @@ struct GemmArgs {
     const double2* A; long long lda; long long sA_batch = 0, sA_kb = 0;
     const double2* B; long long ldb; long long sB_batch = 0, sB_kb = 0;
     double2* C; long long ldc; long long sC_batch = 0;
+    long long sC_n = 1;   // element stride between columns of C (oz_gemm only; gemm_c64 wants 1)
     bool accumulate = false;  // C += result (else C = result)
     bool herm_lower = false;  // result is Hermitian: compute tiles on/below the diagonal only
     int max_splits = 0;       // > 0: at most this many CTAs per output tile along the summation
