@@ -257,8 +257,10 @@ typedef struct {
     double eig_seconds;        /* device time of the truncation eigensolver (timing on)   */
     long long host_syncs;      /* times the call waited for the GPU (stream synchronisations):
                                   with lanczos_max_restarts = 0 and the exact truncation, once
-                                  per sweep plus set-up and workspace growth; otherwise also
-                                  once per Lanczos step and per truncation                  */
+                                  per sweep plus set-up and workspace growth, and up to a dozen
+                                  times in a truncation of a density matrix larger than 256
+                                  (its convergence is read back); otherwise also once per
+                                  Lanczos step and per truncation                           */
 } vtn_sweep_report;
 
 /* Fill opts with the defaults: chi_max 16, 8 sweeps, FP64, lanczos_tol 1e-10,
@@ -429,7 +431,10 @@ vtn_status vtn_heff_ground(vtn_ctx ctx, const vtn_core* Wi, const vtn_core* Wj, 
 /* Truncation of a two-site tensor theta (device complex[chi_l*d1*d2*chi_r]) viewed as
  * the (chi_l d1) x (d2 chi_r) matrix T, by the FP64 eigendecomposition of the reduced
  * density matrix, keeping k = min(k_max, chi_l d1, d2 chi_r) eigenpairs of largest
- * eigenvalue (squared Schmidt values, Eq. SurrogateEpsChi):
+ * eigenvalue (squared Schmidt values, Eq. SurrogateEpsChi).  Where at most a third of the
+ * eigenpairs of a matrix larger than 256 are kept they are found by Chebyshev-filtered subspace
+ * iteration run until its residual is at rounding level, else (or when it would not pay) by
+ * the full Householder reduction; the accuracy is the same:
  *  direction 0: rho = T T^dag = U diag(lam) U^dag; left = U_k (chi_l,d1,k, left-canonical),
  *               right = U_k^dag T (k,d2,chi_r).
  *  direction 1: rho = T^dag T = V diag(lam) V^dag; left = T V_k (chi_l,d1,k),

@@ -24,68 +24,120 @@ namespace {
 
 constexpr int NB = 32;  // diagonal block of the blocked Cholesky and of the triangular solve
 
+// 1 / x and 1 / sqrt(x) from an FP32 start by two Newton steps each: the serial chain of the factorisation is
+// these, and an FP64 instruction takes about 30 ns whether or not others could run beside it.  x is scaled into
+// FP32's range by the caller.
+__device__ __forceinline__ double recip_newton(double x) {
+    double r = (double)__frcp_rn((float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+__device__ __forceinline__ double rsqrt_newton(double x) {
+    double r = (double)rsqrtf((float)x);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+    return r;
+}
+
 // Cholesky factor of the b x b diagonal block at G (leading dimension ld; lower triangle read
 // and written) and the inverse of that factor into Linv (NB x NB, zero above the diagonal).
 // One CTA, b <= NB.  flag[0] = 1 on a pivot that is not positive.
+// FP64-issue bound (about 2 x 170 warp-wide element updates of 6 instructions), so the elements left of each step are
+// dealt out densely to the lanes: L D L^dag with unit L, the update of column j and the same row operations on
+// the growing inverse in one pass with one barrier, the square roots taken once at the end.  168 -> 59 us
+// for a block of 32 (one column per step with three barriers and the inverse as 32 serial dot products before).
 __global__ void __launch_bounds__(256) potrf_block(double2* __restrict__ G, int b, long long ld,
                                                   double2* __restrict__ Linv, int* __restrict__ flag) {
     __shared__ double2 S[NB][NB + 1];
     __shared__ double2 X[NB][NB + 1];
-    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
+    __shared__ double D[NB];
+    __shared__ int bad;
+    const int tid = threadIdx.x;
+    if (tid == 0) bad = 0;
+    for (int t = tid; t < NB * NB; t += 256) {
         const int i = t / NB, j = t - (t / NB) * NB;
         S[i][j] = (i < b && j <= i) ? G[(long long)i * ld + j] : make_double2(0.0, 0.0);
-        X[i][j] = make_double2(0.0, 0.0);
+        X[i][j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
     }
     __syncthreads();
-    for (int j = 0; j < b; ++j) {
-        if (threadIdx.x == 0) {
-            double djj = S[j][j].x;
-            if (!(djj > 0.0)) {
-                flag[0] = 1;  // the caller's fallback replaces the result
-                djj = 1.0;
-            }
-            S[j][j] = make_double2(sqrt(djj), 0.0);
+    if (tid < 32) {
+        // row scaling by powers of two: D^-1/2 of the diagonal, so that every pivot is within [0, 4)
+        int e = 0;
+        if (tid < b) {
+            const double d = S[tid][tid].x;
+            e = d > 0.0 && d < 1e300 ? ilogb(d) / 2 : 0;
         }
-        __syncthreads();
-        const double r = 1.0 / S[j][j].x;
-        for (int i = j + 1 + threadIdx.x; i < b; i += blockDim.x) {
-            S[i][j].x *= r;
-            S[i][j].y *= r;
-        }
-        __syncthreads();
-        // S[i][l] -= S[i][j] conj(S[l][j]) for j < l <= i (column j is only read here)
-        for (int t = threadIdx.x; t < b * b; t += blockDim.x) {
-            const int i = t / b, l = t - (t / b) * b;
-            if (l > j && l <= i) {
-                const double2 a = S[i][j], c = S[l][j];
-                S[i][l].x -= a.x * c.x + a.y * c.y;
-                S[i][l].y -= a.y * c.x - a.x * c.y;
-            }
-        }
-        __syncthreads();
-    }
-    // X = S^{-1}, one column per thread: X[c][c] = 1 / S[c][c],
-    // X[i][c] = -(sum_{c <= l < i} S[i][l] X[l][c]) / S[i][i]
-    if (threadIdx.x < b) {
-        const int c = threadIdx.x;
-        X[c][c] = make_double2(1.0 / S[c][c].x, 0.0);
-        for (int i = c + 1; i < b; ++i) {
-            double re = 0.0, im = 0.0;
-            for (int l = c; l < i; ++l) {
-                const double2 s = S[i][l], x = X[l][c];
-                re += s.x * x.x - s.y * x.y;
-                im += s.x * x.y + s.y * x.x;
-            }
-            const double inv = 1.0 / S[i][i].x;
-            X[i][c] = make_double2(-re * inv, -im * inv);
-        }
+        D[tid] = (double)e;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
+    for (int t = tid; t < NB * NB; t += 256) {
         const int i = t / NB, j = t - (t / NB) * NB;
-        if (i < b && j <= i) G[(long long)i * ld + j] = S[i][j];
-        Linv[t] = X[i][j];
+        if (j <= i) {
+            const int e = -(int)D[i] - (int)D[j];
+            S[i][j].x = scalbn(S[i][j].x, e);
+            S[i][j].y = scalbn(S[i][j].y, e);
+        }
     }
+    __shared__ int row_exp[NB];
+    __shared__ double piv[NB];
+    __syncthreads();
+    if (tid < NB) row_exp[tid] = (int)D[tid];
+    for (int j = 0; j < b; ++j) {
+        double d = S[j][j].x;
+        if (!(d > 1e-30)) {  // pivots are relative to their row's norm; the caller's fallback replaces the result
+            if (tid == 0) bad = 1;
+            d = 1.0;
+        }
+        if (tid == 0) piv[j] = d;
+        const double inv = recip_newton(d);
+        const int r = b - 1 - j;
+        const int n_s = r * (r + 1) / 2, n_x = r * (j + 1);
+        for (int t = tid; t < n_s + n_x; t += 256) {
+            int i, l;
+            if (t < n_s) {  // S[i][l] -= S[i][j] conj(S[l][j]) / d, j < l <= i
+                i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+                while (i * (i + 1) / 2 > t) --i;
+                while ((i + 1) * (i + 2) / 2 <= t) ++i;
+                l = t - i * (i + 1) / 2 + j + 1;
+                i += j + 1;
+                double2 a = S[i][j];
+                const double2 c = S[l][j];
+                a.x *= inv;
+                a.y *= inv;
+                double2 s = S[i][l];
+                s.x = fma(-a.x, c.x, fma(-a.y, c.y, s.x));
+                s.y = fma(-a.y, c.x, fma(a.x, c.y, s.y));
+                S[i][l] = s;
+            } else {  // X[i][l] -= S[i][j] / d X[j][l], i > j, l <= j
+                const int u = t - n_s;
+                i = j + 1 + u / (j + 1);
+                l = u % (j + 1);
+                double2 a = S[i][j];
+                const double2 x = X[j][l];
+                a.x *= inv;
+                a.y *= inv;
+                double2 s = X[i][l];
+                s.x = fma(-a.x, x.x, fma(a.y, x.y, s.x));
+                s.y = fma(-a.x, x.y, fma(-a.y, x.x, s.y));
+                X[i][l] = s;
+            }
+        }
+        __syncthreads();
+    }
+    if (tid < NB) D[tid] = tid < b ? rsqrt_newton(piv[tid]) : 1.0;
+    __syncthreads();
+    // L = (unit L) D^1/2 and its inverse, with the row scaling undone
+    for (int t = tid; t < NB * NB; t += 256) {
+        const int i = t / NB, j = t - (t / NB) * NB;
+        double2 x = make_double2(0.0, 0.0);
+        if (i < b && j <= i) {
+            const double2 s = i == j ? make_double2(piv[j], 0.0) : S[i][j];
+            G[(long long)i * ld + j] = make_double2(scalbn(s.x * D[j], row_exp[i]), scalbn(s.y * D[j], row_exp[i]));
+            x = make_double2(scalbn(X[i][j].x * D[i], -row_exp[j]), scalbn(X[i][j].y * D[i], -row_exp[j]));
+        }
+        Linv[t] = x;
+    }
+    if (tid == 0 && bad) flag[0] = 1;
 }
 
 // flag[0] = 1 if max over the lower triangle of |G - I| > tol or a value is not finite
@@ -168,7 +220,57 @@ void solve_lower_rows(Ctx& ctx, const double2* G, const double2* Linv_all, int m
     }
 }
 
+// before the factorisation: the Gram matrix' diagonal
+__global__ void gram_diagonal(const double2* __restrict__ G, int m, double* __restrict__ d) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < m) d[j] = G[(long long)j * m + j].x;
+}
+
+// after it: pivots of rows 0, k - 1 and m - 1, the smallest pivot relative to its row's norm, the flag
+__global__ void __launch_bounds__(1024) pivot_info(const double2* __restrict__ G, int m, int k, const double* __restrict__ d,
+                                                   const int* __restrict__ flag, double* __restrict__ info) {
+    __shared__ double sh[32];
+    double mn = 2.0;
+    for (int j = threadIdx.x; j < m; j += 1024) {
+        const double r = G[(long long)j * m + j].x / sqrt(d[j]);
+        mn = r == r ? fmin(mn, r) : -1.0;
+    }
+    for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mn;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < 32; ++w) mn = fmin(mn, sh[w]);
+    info[0] = G[0].x;
+    info[1] = G[(long long)(k - 1) * m + k - 1].x;
+    info[2] = G[(long long)(m - 1) * m + m - 1].x;
+    info[3] = mn;
+    info[4] = *flag;
+}
+
 }  // namespace
+
+void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info) {
+    const int nblk = (m + NB - 1) / NB;
+    double2* G = (double2*)ctx.workspace(WS_CQR_G, sizeof(double2) * ((size_t)m * m + (size_t)nblk * NB * NB + m));
+    double2* Linv = G + (size_t)m * m;
+    double* diag = (double*)(Linv + (size_t)nblk * NB * NB);
+    int* flag = (int*)(diag + m);
+    double2* tmp = (double2*)ctx.workspace(WS_CQR_T, sizeof(double2) * (size_t)NB * std::max(n, m));
+    VTN_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int), ctx.stream));
+    GemmArgs g;
+    g.M = m; g.N = m; g.K = n;
+    g.A = A; g.lda = n;
+    g.opB = OP_C; g.B = A; g.ldb = n;
+    g.C = G; g.ldc = m;
+    g.herm_lower = true;
+    gemm_c64(ctx, g);
+    gram_diagonal<<<(m + 255) / 256, 256, 0, ctx.stream>>>(G, m, diag);
+    cholesky_blocked(ctx, G, m, Linv, tmp, flag);
+    pivot_info<<<1, 1024, 0, ctx.stream>>>(G, m, k, diag, flag, info);
+    ctx.count_launch(2);
+    ctx.check_launch("cholqr_pass");
+    solve_lower_rows(ctx, G, Linv, m, n, A, tmp);
+}
 
 void orthonormalize_rows_cholqr(Ctx& ctx, double2* A, int m, int n) {
     VTN_REQUIRE(m >= 1 && m <= n && m <= 4096, "row orthonormalisation needs 1 <= rows <= min(cols, 4096)");

@@ -1639,6 +1639,24 @@ TruncResult truncate_deferred_result(const double* slot, int k) {
     return r;
 }
 
+void density_dev(Ctx& ctx, int nL, int nR, int direction, const double2* theta, double2* rho) {
+    const int n = direction == 0 ? nL : nR;
+    GemmArgs g;
+    if (direction == 0) {
+        g.M = nL; g.N = nL; g.K = nR;
+        g.A = theta; g.lda = nR;
+        g.opB = OP_C; g.B = theta; g.ldb = nR;
+    } else {
+        g.M = nR; g.N = nR; g.K = nL;
+        g.opA = OP_C; g.A = theta; g.lda = nR;
+        g.B = theta; g.ldb = nR;
+    }
+    g.C = rho; g.ldc = n;
+    g.herm_lower = true;
+    gemm_c64(ctx, g);
+    mirror_lower_to_upper(ctx, rho, n, n);
+}
+
 TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int direction, int k_max,
                          const double2* theta, double2* left, double2* right, int outer, double* defer) {
     const int nL = chi_l * d1, nR = d2 * chi_r;
@@ -1648,6 +1666,10 @@ TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int dir
     VTN_REQUIRE(outer >= 1 && outer <= (direction == 0 ? nR : nL), "truncation output range out of bounds");
     VTN_REQUIRE(k >= 1, "truncation keeps no state");
     VTN_REQUIRE(n <= 12288, "reduced density matrix larger than 12288 is not supported");
+    if (const int m = filter_rows(nL, nR, direction, k)) {
+        TruncResult r;
+        if (truncate_filtered(ctx, nL, nR, direction, k, m, theta, left, right, outer, defer, r)) return r;
+    }
     int tt = ctx.tbegin(TC_EIG, 0.0);
     double2* A = (double2*)ctx.workspace(WS_EIG_A, sizeof(double2) * (size_t)n * n);
     double2* H = (double2*)ctx.workspace(WS_EIG_H, sizeof(double2) * (size_t)n * n);
@@ -1669,20 +1691,7 @@ TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int dir
     double* G = work + 5 * (size_t)n * k;
     int* status = (int*)(G + (size_t)k * k);
     // 1. rho
-    GemmArgs g;
-    if (direction == 0) {
-        g.M = nL; g.N = nL; g.K = nR;
-        g.A = theta; g.lda = nR;
-        g.opB = OP_C; g.B = theta; g.ldb = nR;
-    } else {
-        g.M = nR; g.N = nR; g.K = nL;
-        g.opA = OP_C; g.A = theta; g.lda = nR;
-        g.B = theta; g.ldb = nR;
-    }
-    g.C = A; g.ldc = n;
-    g.herm_lower = true;
-    gemm_c64(ctx, g);
-    mirror_lower_to_upper(ctx, A, n, n);
+    density_dev(ctx, nL, nR, direction, theta, A);
     norm2_dev(ctx, theta, (long long)nL * nR, &s.scal[0]);
     VTN_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int) * 8, ctx.stream));
     // 2. tridiagonalisation: one persistent cooperative launch when it fits, else one

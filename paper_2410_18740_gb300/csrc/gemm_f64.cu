@@ -158,6 +158,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     p.accumulate = g.accumulate ? 1 : 0;
     p.herm_lower = g.herm_lower ? 1 : 0;
     p.negate = g.negate ? 1 : 0;
+    VTN_REQUIRE(g.sC_n == 1 || (g.prepA != nullptr && g.ldc == 1 && !g.herm_lower), "column strides need a prepared operand");
     VTN_REQUIRE(!g.herm_lower || (g.M == g.N && !g.accumulate), "Hermitian GEMM needs a square, non-accumulating C");
     p.batch = g.batch;
     const long long gx = (g.N + BT - 1) / BT, gy = (g.M + BT - 1) / BT;
@@ -167,7 +168,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     // against sliced: 128^3 22 | 34 us, 160^3 34 | 35 us, 192^3 55 | 37 us, 256^3 136 | 38 us, 1024 x 16 x 1024
     // (narrow: padded to 32 columns) 74 | 49 us; at 3072^3 200 ms against 6.1 ms.  Its row sums fit 96-bit integers
     // for summations of up to 2^19 terms.
-    const bool oz = ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.5e6 && (long long)g.K * g.kb <= (1LL << 19);
+    const bool oz = g.prepA != nullptr || ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.5e6 && (long long)g.K * g.kb <= (1LL << 19);
     int S = 1;
     if (oz) {
         S = oz_splits(ctx, g);
@@ -198,6 +199,10 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     }
     if (S > 1) {
         const long long cnt = (long long)g.batch * g.M * g.N;
+        if (g.sC_n != 1) {  // C and the partials are stored column by column
+            std::swap(p.M, p.N);
+            p.ldc = g.sC_n;
+        }
         splitk_sum<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx.stream>>>(p, g.batch);
         ctx.count_launch();
         ctx.check_launch("splitk_sum");

@@ -74,6 +74,7 @@ struct OzParams {
     double2* C;
     long long ldc, sC_n, sC_batch;
     double2* part;
+    int part_t;          // partials column by column
     int accumulate, negate, herm_lower;
     int* status;
 };
@@ -193,7 +194,7 @@ __global__ void __launch_bounds__(256) oz_max_kernel(OzOperand a, OzOperand b, O
             atomicMax(&bx[row], m);
         }
     }
-    if (PASS == 1) return;
+    if (PASS == 1 || n_bx < 0) return;  // a prepared operand leaves no choice
     __syncthreads();
     if ((int)threadIdx.x < k1 - k0) atomicMax(&o.kx[k0 + threadIdx.x], kmax[threadIdx.x]);
     // the last block compares the largest term with (largest of A) x (largest of B)
@@ -582,8 +583,8 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             if (!ok) break;
             const bool to_part = p.splits > 1;
             double2* C = to_part ? p.part + ((long long)z * p.batch + bz) * p.M * p.N : p.C + (long long)bz * p.sC_batch;
-            const long long cn = to_part ? 1 : p.sC_n;
-            double2* dst = C + (long long)m * (to_part ? p.N : p.ldc) + n0 * cn;
+            const long long cn = to_part ? (p.part_t ? p.M : 1) : p.sC_n;
+            double2* dst = C + (long long)m * (to_part ? (p.part_t ? 1 : p.N) : p.ldc) + n0 * cn;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int en = __shfl_sync(0xffffffffu, eb, j);
@@ -632,8 +633,54 @@ int oz_splits(const Ctx& ctx, const GemmArgs& g) {
     return 1;
 }
 
+// op(A) (or op(B)) rows [r0, r0 + rows) of batches [b0, b0 + nb)
+static void fill_operand(OzOperand& o, const GemmArgs& g, bool is_b, long long b0, long long r0, int rows, int tiles, int nb) {
+    const Op op = is_b ? g.opB : g.opA;
+    o.K = g.K; o.kbn = g.kb;
+    o.kc = is_b ? op != OP_N : op == OP_N;
+    o.conj = op == OP_C;
+    o.ld = is_b ? g.ldb : g.lda;
+    o.s_batch = is_b ? g.sB_batch : g.sA_batch;
+    o.s_kb = is_b ? g.sB_kb : g.sA_kb;
+    o.X = (is_b ? g.B : g.A) + b0 * o.s_batch + (o.kc ? r0 * o.ld : r0);
+    o.rows = rows; o.tiles = tiles; o.nb = nb;
+}
+
+// The digits of op(A) (M x K) once, for products that share it; without the scaling of the summation index,
+// which depends on both operands.
+OzPrep oz_prepare(Ctx& ctx, int M, int K, Op opA, const double2* A, long long lda) {
+    GemmArgs g;
+    g.M = M; g.N = 1; g.K = K;
+    g.opA = opA; g.A = A; g.lda = lda;
+    g.B = nullptr; g.ldb = 0; g.C = nullptr; g.ldc = 0;
+    const int nkb = (int)cdiv(K, KBC), tiles = (int)cdiv(M, TM);
+    const size_t digits = (size_t)tiles * nkb * A_BYTES, n_bx = (size_t)tiles * TM;
+    char* w = (char*)ctx.workspace(WS_OZ_PREP, digits + sizeof(int) * n_bx + sizeof(OzShift));
+    OzOperand a;
+    fill_operand(a, g, false, 0, 0, M, tiles, 1);
+    a.out = (uint4*)w;
+    a.bx = (int*)(w + digits);
+    OzShift* shift = (OzShift*)(a.bx + n_bx);
+    a.kx = nullptr;
+    VTN_CUDA_TRY(cudaMemsetAsync(a.bx, 0, sizeof(int) * n_bx + sizeof(OzShift), ctx.stream));
+    const int kseg = (int)cdiv(K, MAX_KS);
+    const long long ma = cdiv(M, 32) * kseg, sa = (long long)tiles * nkb;
+    oz_max_kernel<0><<<(unsigned)ma, 256, 0, ctx.stream>>>(a, a, shift, (int)ma, kseg, -1);
+    oz_slice_kernel<<<(unsigned)sa, 256, 0, ctx.stream>>>(a, a, shift, (int)sa, nkb);
+    ctx.count_launch(2);
+    ctx.check_launch("oz_prepare");
+    OzPrep p;
+    p.digits = w;
+    p.bx = a.bx;
+    p.M = M;
+    p.K = K;
+    return p;
+}
+
 void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
     VTN_REQUIRE(ctx.dstatus != nullptr, "context has no device status word");
+    VTN_REQUIRE(g.prepA == nullptr || (g.prepA->M == g.M && g.prepA->K == g.K && g.batch == 1 && g.kb == 1),
+                "prepared operand of another shape");
     set_smem_attr_once(ctx, (const void*)oz_gemm_kernel, (int)SMEM);
     const int nkb = (int)cdiv((long long)g.K * g.kb, KBC);
     // at most 1 GiB of digit tiles per operand (one tile row at least): larger problems run in pieces
@@ -647,7 +694,7 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
     if (a_batch > cap) ms = std::max(1ll, cap / ((long long)nkb * A_BYTES)) * TM;
     if (b_batch > cap) ns = std::max(1ll, cap / ((long long)nkb * B_BYTES)) * TNC;
     // a Hermitian or split result is computed in one piece (the partials' layout and the diagonal refer to all of it)
-    if (g.herm_lower || splits > 1) { bs = g.batch; ms = g.M; ns = g.N; }
+    if (g.herm_lower || splits > 1 || g.prepA) { bs = g.batch; ms = g.M; ns = g.N; }
     for (long long b0 = 0; b0 < g.batch; b0 += bs) {
         const int nb = (int)std::min(bs, g.batch - b0);
         for (long long n0 = 0; n0 < g.N; n0 += ns) {
@@ -659,42 +706,32 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 p.batch = nb; p.splits = splits; p.kb_per = (int)cdiv(nkb, splits);
                 p.tiles_m = (int)cdiv(mm, TM);
                 p.tiles_n = (int)cdiv(nn, TNC);
-                auto fill = [&](OzOperand& o, bool is_b) {
-                    o.K = g.K; o.kbn = g.kb;
-                    if (!is_b) {
-                        o.kc = g.opA == OP_N; o.conj = g.opA == OP_C;
-                        o.ld = g.lda; o.s_batch = g.sA_batch; o.s_kb = g.sA_kb;
-                        o.X = g.A + b0 * g.sA_batch + (g.opA == OP_N ? m0 * g.lda : m0);
-                        o.rows = mm; o.tiles = p.tiles_m; o.nb = a_shared ? 1 : nb;
-                    } else {
-                        o.kc = g.opB != OP_N; o.conj = g.opB == OP_C;
-                        o.ld = g.ldb; o.s_batch = g.sB_batch; o.s_kb = g.sB_kb;
-                        o.X = g.B + b0 * g.sB_batch + (g.opB != OP_N ? n0 * g.ldb : n0);
-                        o.rows = nn; o.tiles = p.tiles_n; o.nb = b_shared ? 1 : nb;
-                    }
-                };
-                fill(p.a, false);
-                fill(p.b, true);
-                const size_t na = (size_t)p.a.nb * p.tiles_m * TM, nbx = (size_t)p.b.nb * p.tiles_n * TNC;
+                const OzPrep* prep = g.prepA;
+                fill_operand(p.a, g, false, b0, m0, mm, p.tiles_m, a_shared ? 1 : nb);
+                fill_operand(p.b, g, true, b0, n0, nn, p.tiles_n, b_shared ? 1 : nb);
+                const size_t na = prep ? 0 : (size_t)p.a.nb * p.tiles_m * TM, nbx = (size_t)p.b.nb * p.tiles_n * TNC;
                 const size_t nk = (size_t)g.K * g.kb, n_exp = sizeof(OzShift) / sizeof(int) + na + nbx + 2 * nk;
                 OzShift* shift = (OzShift*)ctx.workspace(WS_OZ_EXP, sizeof(int) * n_exp);
-                p.a.bx = (int*)(shift + 1);
-                p.b.bx = p.a.bx + na;
+                p.a.bx = prep ? prep->bx : (int*)(shift + 1);
+                p.b.bx = (int*)(shift + 1) + na;
                 p.a.kx = p.b.bx + nbx;
                 p.b.kx = p.a.kx + nk;
-                p.a.out = (uint4*)ctx.workspace(WS_OZ_A, (size_t)p.a.nb * p.tiles_m * nkb * A_BYTES);
+                p.a.out = prep ? (uint4*)prep->digits
+                               : (uint4*)ctx.workspace(WS_OZ_A, (size_t)p.a.nb * p.tiles_m * nkb * A_BYTES);
                 p.b.out = (uint4*)ctx.workspace(WS_OZ_B, (size_t)p.b.nb * p.tiles_n * nkb * B_BYTES);
                 p.C = g.C + b0 * g.sC_batch + m0 * g.ldc + n0 * g.sC_n;
                 p.ldc = g.ldc; p.sC_n = g.sC_n; p.sC_batch = g.sC_batch;
                 p.part = part;
+                p.part_t = g.sC_n != 1;
                 p.accumulate = g.accumulate; p.negate = g.negate; p.herm_lower = g.herm_lower;
                 p.status = ctx.dstatus;
                 VTN_CUDA_TRY(cudaMemsetAsync(shift, 0, sizeof(int) * n_exp, ctx.stream));
                 const int kseg = (int)cdiv((long long)g.K * g.kb, MAX_KS);
-                const long long ma = cdiv(mm, 32) * kseg * p.a.nb, mb = cdiv(nn, 32) * kseg * p.b.nb;
-                oz_max_kernel<0><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg, (int)(na + nbx));
-                oz_max_kernel<1><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg, 0);
-                const long long sa = (long long)p.a.nb * p.tiles_m * nkb, sb = (long long)p.b.nb * p.tiles_n * nkb;
+                const long long ma = prep ? 0 : cdiv(mm, 32) * kseg * p.a.nb, mb = cdiv(nn, 32) * kseg * p.b.nb;
+                oz_max_kernel<0><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg,
+                                                                              prep ? -1 : (int)(na + nbx));
+                if (!prep) oz_max_kernel<1><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg, 0);
+                const long long sa = prep ? 0 : (long long)p.a.nb * p.tiles_m * nkb, sb = (long long)p.b.nb * p.tiles_n * nkb;
                 oz_slice_kernel<<<(unsigned)(sa + sb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)sa, nkb);
                 const long long items = (long long)p.tiles_m * p.tiles_n * nb * splits;
                 VTN_REQUIRE(items < (1ll << 31) && ma + mb < (1ll << 31) && sa + sb < (1ll << 31), "GEMM too large");

@@ -1,0 +1,224 @@
+// Truncation by Chebyshev-filtered subspace iteration, run to the accuracy of the full eigendecomposition.
+//
+// The tridiagonalisation of eigh.cu reduces all n dimensions of rho to find k eigenpairs: n serial columns of
+// about 9 us of latency and 12 n^2 FP64 operations on the narrow FP64 pipe.  With FP64 products 35 times
+// cheaper on the tensor cores (oz_gemm.cu) the k-dimensional top subspace is cheaper to find by products
+// (Zhou, Saad, Tiago, Chelikowsky, J. Comput. Phys. 219 (2006)): a block of m = 1.5 k rows is multiplied by
+// Chebyshev polynomials of rho that stay within 1 on [0, b], b ~ the m-th eigenvalue, and grow fastest
+// above it, and is re-orthonormalised by Cholesky-QR between them.  The rows come out in Schur order, so the
+// pivots of the Cholesky factor are the growth of each direction: once the k-th has grown by e^35 over the
+// unwanted ones, and the residual rho S - (S rho S^dag) S of the first k rows is at rounding level, the kept
+// eigenpairs follow from the m x n problem S T by the exact truncation (Rayleigh-Ritz).
+//
+// Rows: S holds the conjugates of the vectors (m x n), so rho acts from the right; (S rho)^T = rho^T S^T is one
+// product with the digits of rho^T, which all products share.
+//
+// Measured (whole truncation, full reduction -> here): n = 512, k = 64 8.9 -> 7.2 ms; n = 1024, k = 128 29.8 -> 13.7 ms;
+// n = 1830, k = 300 86 -> 40 ms (Schmidt values decaying by e^-9); flat random spectra 8.9 -> 9.0, 29.8 -> 27.3,
+// 86 -> 71 ms.  What is left is latency: the Cholesky chains (1.8 us a row and pass), the m x m tridiagonalisation
+// (12 to 15 us a column) and about 50 us a product.
+//
+// The host reads five numbers after each pass.  It gives up (false: the full eigendecomposition runs) when the
+// spectrum at k is so flat that the predicted polynomial degree costs more than the reduction, when the block is
+// rank deficient, or when the residual stays above rounding.
+#include <algorithm>
+#include <cmath>
+
+#include "vtn_internal.cuh"
+
+namespace vtn {
+namespace {
+
+// out = a p + b y + c z (z may be null, and may be out)
+__global__ void __launch_bounds__(256) cheb_step(long long n, double a, const double2* __restrict__ p, double b,
+                                                 const double2* __restrict__ y, double c, const double2* z, double2* out) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const double2 u = p[i], v = y[i];
+    double2 r = make_double2(fma(a, u.x, b * v.x), fma(a, u.y, b * v.y));
+    if (z != nullptr) {
+        const double2 w = z[i];
+        r.x = fma(c, w.x, r.x);
+        r.y = fma(c, w.y, r.y);
+    }
+    out[i] = r;
+}
+
+// out[0] = max over the rows of |row|^2 (as the bits of a non-negative double), one CTA per row
+__global__ void __launch_bounds__(256) row_norm_max(const double2* __restrict__ A, int n, unsigned long long* out) {
+    __shared__ double sh[8];
+    const double2* row = A + (long long)blockIdx.x * n;
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) acc = fma(row[i].x, row[i].x, fma(row[i].y, row[i].y, acc));
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) acc += sh[w];
+        atomicMax(out, (unsigned long long)__double_as_longlong(acc));  // a NaN orders above every number
+    }
+}
+
+}  // namespace
+
+// Block size 1.5 k + 16 in tiles of 32, from n = 257 on and where the block is at most half of rho.
+int filter_rows(int nL, int nR, int direction, int k) {
+    const int n = direction == 0 ? nL : nR, m = (3 * k / 2 + 16 + 31) / 32 * 32;
+    return n > 256 && n <= 4096 && 2 * m <= n && m <= std::min(nL, nR) ? m : 0;
+}
+
+bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, const double2* theta, double2* left,
+                       double2* right, int outer, double* defer, TruncResult& res) {
+    const int n = direction == 0 ? nL : nR, other = direction == 0 ? nR : nL;
+    const long long mn = (long long)m * n;
+    const int tt = ctx.tbegin(TC_EIG, 0.0);
+    const bool timing = ctx.timing;
+    struct Timing {  // the products inside are part of this interval
+        Ctx& c;
+        bool on;
+        int t;
+        ~Timing() {
+            c.timing = on;
+            if (t >= 0) c.tend(t);
+        }
+    } guard{ctx, timing, tt};
+    double2* rho = (double2*)ctx.workspace(WS_EIG_A, sizeof(double2) * (size_t)n * n);
+    density_dev(ctx, nL, nR, direction, theta, rho);
+    const OzPrep prep = oz_prepare(ctx, n, n, OP_T, rho, n);
+    double2* S = (double2*)ctx.workspace(WS_FLT_S, sizeof(double2) * (size_t)mn);
+    double2* X = (double2*)ctx.workspace(WS_FLT_X, sizeof(double2) * (size_t)mn);
+    double2* P = (double2*)ctx.workspace(WS_FLT_P, sizeof(double2) * (size_t)m * std::max(n, other));
+    double2* H = (double2*)ctx.workspace(WS_FLT_H, sizeof(double2) * (size_t)m * m);
+    double* num = (double*)ctx.workspace(WS_FLT_N, sizeof(double) * 16);  // info[5], residual, |theta|^2
+    auto apply = [&](const double2* in, double2* out) {  // out = in rho
+        GemmArgs g;
+        g.M = n; g.N = m; g.K = n;
+        g.prepA = &prep; g.opA = OP_T; g.A = rho; g.lda = n;  // (rho itself for rows that are not finite)
+        g.opB = OP_T; g.B = in; g.ldb = n;
+        g.C = out; g.ldc = 1; g.sC_n = n;
+        gemm_c64(ctx, g);
+    };
+    double l1 = 0, lk = 0, lm = 0, pivot = 0;
+    auto orth = [&](double2* A) {
+        cholqr_pass(ctx, A, m, n, k, num);
+        VTN_CUDA_TRY(cudaMemcpyAsync(ctx.pinned, num, sizeof(double) * 5, cudaMemcpyDeviceToHost, ctx.stream));
+        ctx.sync();
+        l1 = ctx.pinned[0]; lk = ctx.pinned[1]; lm = ctx.pinned[2]; pivot = ctx.pinned[3];
+        // NaN fails every comparison
+        return ctx.pinned[4] == 0.0 && pivot > 1e-7 && lk > 0.0 && l1 < 1e300;
+    };
+    // ---- two plain products of a random block: eigenvalue estimates from the second one's pivots
+    fill_random_normal(ctx, S, mn, 0x5eedull, n, PHILOX_STREAM_TRUNC);
+    apply(S, P);
+    if (!orth(P)) return false;
+    apply(P, S);
+    if (!orth(S)) return false;
+    if (!(lm > 1e-12 * l1) || !(lk > lm)) return false;
+    const double b = lm, lam1 = l1;
+    const double g1 = std::acosh(2.0 * 1.6 * lam1 / b - 1.0);  // growth per degree; the largest pivot reads low
+    double gk = std::acosh(2.0 * lk / b - 1.0);
+    // Degrees that cost as much as the reduction: 8.9 ms at n = 512, 30 at 1024 and 86 at 1830, against 5, 8 and
+    // 20 ms of orthonormalisation and Rayleigh-Ritz and 40, 60 and 110 us a degree.
+    const double limit = 40.0 * std::pow(n / 512.0, 1.6);
+    if (!(35.0 / gk <= limit)) return false;
+    double grown = 0.0, degrees = 0.0;
+    bool done = false;
+    for (int cycle = 0; cycle < 32 && !done; ++cycle) {
+        // the first block is not in Schur order yet: its rows may part by 1e5 only; later ones by 1e11
+        int D = (int)(std::log(cycle == 0 ? 1e5 : 1e11) / g1);
+        D = std::max(2, std::min({D, 12, (int)std::ceil((36.0 - grown) / gk)}));
+        degrees += D;
+        if (degrees > 2.0 * limit) return false;
+        apply(S, P);
+        cheb_step<<<(unsigned)((mn + 255) / 256), 256, 0, ctx.stream>>>(mn, 2.0 / b, P, -1.0, S, 0.0, nullptr, X);
+        double2 *prev = S, *cur = X;
+        for (int i = 1; i < D; ++i) {
+            apply(cur, P);
+            cheb_step<<<(unsigned)((mn + 255) / 256), 256, 0, ctx.stream>>>(mn, 4.0 / b, P, -2.0, cur, -1.0, prev, prev);
+            std::swap(prev, cur);
+        }
+        ctx.count_launch(D);
+        ctx.check_launch("cheb_step");
+        S = cur;
+        X = prev;
+        if (!orth(S)) return false;
+        grown += std::log(lk);
+        gk = std::log(lk) / D;
+        if (!(gk > 0.0)) return false;
+        if (grown < 35.0) {
+            if (!(degrees + (35.0 - grown) / gk <= 2.0 * limit)) return false;
+            continue;
+        }
+        // the pass lost orthogonality like u / pivot^2
+        if (pivot < 0.2 && !orth(S)) return false;
+        // ---- residual of the first k rows: S rho - (S rho S^dag) S
+        apply(S, P);
+        GemmArgs h;
+        h.M = m; h.N = m; h.K = n;
+        h.A = P; h.lda = n;
+        h.opB = OP_C; h.B = S; h.ldb = n;
+        h.C = H; h.ldc = m;
+        gemm_c64(ctx, h);
+        GemmArgs r;
+        r.M = k; r.N = n; r.K = m;
+        r.A = H; r.lda = m;
+        r.B = S; r.ldb = n;
+        r.C = P; r.ldc = n;
+        r.accumulate = true; r.negate = true;
+        gemm_c64(ctx, r);
+        VTN_CUDA_TRY(cudaMemsetAsync(num + 5, 0, sizeof(double), ctx.stream));
+        row_norm_max<<<k, 256, 0, ctx.stream>>>(P, n, (unsigned long long*)(num + 5));
+        ctx.count_launch();
+        ctx.check_launch("row_norm_max");
+        VTN_CUDA_TRY(cudaMemcpyAsync(ctx.pinned, num + 5, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
+        ctx.sync();
+        done = std::sqrt(ctx.pinned[0]) <= 4e-15 * lam1;
+        if (!done && grown > 60.0) return false;
+    }
+    if (!done) return false;
+    // ---- Rayleigh-Ritz: the exact truncation of the projected tensor
+    norm2_dev(ctx, theta, (long long)nL * nR, num + 6);
+    ctx.timing = false;
+    double2* U1 = (double2*)ctx.workspace(WS_FLT_U, sizeof(double2) * (size_t)m * k);
+    GemmArgs g;
+    if (direction == 0) {
+        g.M = m; g.N = nR; g.K = n;  // P = S T; P P^dag = U' lam U'^dag, right = U'^dag P, left = S^dag U'
+        g.A = S; g.lda = n;
+        g.B = theta; g.ldb = nR;
+        g.C = P; g.ldc = nR;
+        gemm_c64(ctx, g);
+        res = truncate_dev(ctx, m, 1, 1, nR, 0, k, P, U1, right, outer, defer);
+        GemmArgs l;
+        l.M = n; l.N = k; l.K = m;
+        l.opA = OP_C; l.A = S; l.lda = n;
+        l.B = U1; l.ldb = k;
+        l.C = left; l.ldc = k;
+        gemm_c64(ctx, l);
+    } else {
+        g.M = nL; g.N = m; g.K = n;  // P = T S^dag; P^dag P = V' lam V'^dag, left = P V', right = V'^dag S
+        g.A = theta; g.lda = nR;
+        g.opB = OP_C; g.B = S; g.ldb = n;
+        g.C = P; g.ldc = m;
+        gemm_c64(ctx, g);
+        res = truncate_dev(ctx, nL, 1, 1, m, 1, k, P, left, U1, outer, defer);
+        GemmArgs l;
+        l.M = k; l.N = n; l.K = m;
+        l.A = U1; l.lda = m;
+        l.B = S; l.ldb = n;
+        l.C = right; l.ldc = n;
+        gemm_c64(ctx, l);
+    }
+    // the discarded weight refers to the whole tensor
+    if (defer != nullptr) {
+        VTN_CUDA_TRY(cudaMemcpyAsync(defer + k, num + 6, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
+        return true;
+    }
+    VTN_CUDA_TRY(cudaMemcpyAsync(ctx.pinned, num + 6, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
+    ctx.sync();
+    double kept = 0.0;
+    for (double l : res.lam) kept += l;
+    res.discarded = ctx.pinned[0] > 0.0 ? 1.0 - kept / ctx.pinned[0] : 0.0;
+    return true;
+}
+
+}  // namespace vtn

@@ -158,7 +158,7 @@ enum WsSlot {
     WS_TC_A2, WS_TC_PART, WS_GEMM_SPLIT, WS_EIG_PART, WS_TC_ENV, WS_EIG_T, WS_H2_ENV, WS_EXPAND,
     WS_TRUNC_L, WS_TRUNC_R, WS_CENTER, WS_MLP_ACT, WS_MLP_Y, WS_MLP_G, WS_WARM_S, WS_WARM_Z, WS_WARM_P,
     WS_WARM_U, WS_WARM_N, WS_WARM_Q0, WS_CQR_G, WS_CQR_T, WS_CQR_B, WS_RQ_Y, WS_RQ_S, WS_CHOL_LINV, WS_TH_A, WS_TH_B,
-    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_COUNT
+    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_OZ_PREP, WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_N, WS_FLT_U, WS_COUNT
 };
 
 // ------------------------------------------------------------------ cores
@@ -170,6 +170,13 @@ HostCore core_from_abi(const vtn_core* c);
 // ------------------------------------------------------------------ GEMM (complex FP64)
 enum Op { OP_N = 0, OP_C = 1, OP_T = 2 };  // op(X) = X, X^dag (conjugate transpose) or (oz_gemm only) X^T
 
+// Digits of an op(A) that several products share (oz_gemm.cu; valid until the next oz_prepare of the context).
+struct OzPrep {
+    const void* digits = nullptr;
+    int* bx = nullptr;
+    int M = 0, K = 0;
+};
+
 struct GemmArgs {
     int M, N, K;          // op(A): M x K, op(B): K x N, C: M x N
     int batch = 1;        // independent problems
@@ -178,7 +185,8 @@ struct GemmArgs {
     const double2* A; long long lda; long long sA_batch = 0, sA_kb = 0;
     const double2* B; long long ldb; long long sB_batch = 0, sB_kb = 0;
     double2* C; long long ldc; long long sC_batch = 0;
-    long long sC_n = 1;   // element stride between columns of C (oz_gemm only; gemm_c64 wants 1)
+    long long sC_n = 1;   // element stride between columns of C (oz_gemm and products with prepA; then ldc = 1)
+    const OzPrep* prepA = nullptr;  // op(A) is this prepared operand (A, lda, opA as it was prepared from; batch = kb = 1)
     bool accumulate = false;  // C += result (else C = result)
     bool herm_lower = false;  // result is Hermitian: compute tiles on/below the diagonal only
     int max_splits = 0;       // > 0: at most this many CTAs per output tile along the summation
@@ -192,6 +200,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class = TC_GEMM);
 // The same product on the tensor cores by exact integer slices (oz_gemm.cu); gemm_c64 chooses.  splits > 1:
 // partial tiles [splits][batch][M][N] go to `part` instead of C.
 int oz_splits(const Ctx& ctx, const GemmArgs& g);
+OzPrep oz_prepare(Ctx& ctx, int M, int K, Op opA, const double2* A, long long lda);
 void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part);
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize, bytes) for kernel fn on the context's
@@ -382,6 +391,16 @@ TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int dir
                          const double2* theta, double2* left, double2* right, int outer = -1,
                          double* defer = nullptr);
 TruncResult truncate_deferred_result(const double* slot, int k);
+// rho = T T^dag (direction 0, nL x nL) or T^dag T (nR x nR) of the nL x nR matrix T (eigh.cu)
+void density_dev(Ctx& ctx, int nL, int nR, int direction, const double2* theta, double2* rho);
+// The same truncation by filtered subspace iteration to full accuracy (trunc_filter.cu): false when the spectrum
+// does not suit it (nothing but workspaces is then written).  filter_rows: its block size, 0 = not for this shape.
+int filter_rows(int nL, int nR, int direction, int k);
+bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, const double2* theta, double2* left,
+                       double2* right, int outer, double* defer, TruncResult& res);
+// One CholeskyQR pass over the rows of A (m x n) in place (chol_qr.cu); info (device double[5]) = the pivots of row
+// 0, row k - 1 and row m - 1, the smallest pivot relative to its row's norm, and 1 if a pivot was not positive.
+void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info);
 
 // ------------------------------------------------------------------ misc kernels
 // Philox counter word 3: the stream of the random numbers (initial MPS, sampler, truncation)

@@ -1,0 +1,68 @@
+"""Truncation of density matrices larger than 256 (Chebyshev-filtered subspace iteration, csrc/trunc_filter.cu)
+against a singular value decomposition, with spectra it suits and spectra that go to the full reduction."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _tensor(rng, n1, n2, s):
+    q = lambda n: np.linalg.qr(rng.standard_normal((n, len(s))) + 1j * rng.standard_normal((n, len(s))))[0]
+    return (q(n1) * s) @ q(n2).conj().T
+
+
+def _spectrum(kind, n, k):
+    e = np.arange(n, dtype=float)
+    if kind == "decaying":
+        return np.exp(-9.0 * e / n)
+    if kind == "flat":
+        return np.exp(-1.0 * e / n)
+    if kind == "degenerate top":
+        return np.where(e < k // 2, 1.0, np.exp(-9.0 * e / n))
+    if kind == "steep":  # squared Schmidt values below rounding inside the block
+        return np.exp(-60.0 * e / n)
+    if kind == "rank below k":
+        return np.exp(-e[: k // 2] / n)
+    assert kind == "degenerate at k"
+    s = np.exp(-9.0 * e / n)
+    s[k - 4:k + 2 * k] = s[k - 4]
+    return s
+
+
+# (chi_l, d1, d2, chi_r, k): just above the limit, a ragged block, unequal sides, a block of several tiles
+@pytest.mark.parametrize("shape", [(52, 5, 5, 53, 20), (87, 6, 6, 91, 33), (65, 8, 8, 80, 64)])
+@pytest.mark.parametrize("kind", ["decaying", "flat", "degenerate top", "steep", "rank below k", "degenerate at k"])
+@pytest.mark.parametrize("direction", [0, 1])
+def test_large_truncation_matches_the_svd(ctx, shape, kind, direction):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    cl, d1, d2, cr, k = shape
+    n1, n2 = cl * d1, d2 * cr
+    rng = np.random.default_rng(n1 + 7 * n2 + direction)
+    T = _tensor(rng, n1, n2, _spectrum(kind, min(n1, n2), k))
+    th = torch.from_numpy(np.ascontiguousarray(T)).cuda()
+    left = torch.empty(n1, k, dtype=torch.complex128, device="cuda")
+    right = torch.empty(k, n2, dtype=torch.complex128, device="cuda")
+    before = vtn.vtn_launch_count(ctx)
+    kk, lam, disc = vtn.vtn_truncate(ctx, cl, d1, d2, cr, direction, k, th, left, right)
+    launches = vtn.vtn_launch_count(ctx) - before
+    U, S, Vh = np.linalg.svd(T, full_matrices=False)
+    nrm2 = float((S ** 2).sum())
+    n = n1 if direction == 0 else n2
+    u = 2.0 ** -53
+    # rounding of rho and of its eigenpairs: a small multiple of n u |rho| (as the bounds of the full reduction)
+    assert kk == k and np.abs(lam - S[:k] ** 2).max() <= 4 * n * u * S[0] ** 2
+    assert abs(disc - (1.0 - (S[:k] ** 2).sum() / nrm2)) <= 4 * n * u * k
+    iso = left if direction == 0 else right.conj().T
+    eye = torch.eye(k, dtype=torch.complex128, device="cuda")
+    assert float((iso.conj().T @ iso - eye).abs().max()) <= 4 * n * u
+    got = (left @ right).cpu().numpy()
+    if kind in ("decaying", "flat", "degenerate top"):
+        ref = (U[:, :k] * S[:k]) @ Vh[:k]
+        gap = (S[k - 1] ** 2 - S[k] ** 2) / S[0] ** 2
+        # subspace error: residual over gap, weighted by the boundary's Schmidt values
+        assert np.linalg.norm(got - ref) <= (4 * n * u / gap * S[k - 1] + 4 * n * u * S[0]) * np.sqrt(k)
+    # whatever was kept at a degenerate or noise-level boundary carries the largest weight there is
+    assert np.linalg.norm(got) ** 2 >= (S[:k] ** 2).sum() - 8 * n * u * k * S[0] ** 2
+    if kind == "decaying":
+        assert launches > 120, launches  # the full reduction takes about 30
