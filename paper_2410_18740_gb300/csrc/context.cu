@@ -113,6 +113,7 @@ void Ctx::tflush() {
 
 void Ctx::check_dstatus() {
     if (!dstatus) return;
+    dstatus_due = false;
     VTN_CUDA_TRY(cudaMemcpyAsync(pinned + 4095, dstatus, sizeof(int), cudaMemcpyDeviceToHost, stream));
     sync();
     int v = 0;

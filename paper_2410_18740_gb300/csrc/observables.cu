@@ -262,6 +262,114 @@ __global__ void __launch_bounds__(256) sample_kernel(SampleArgs a) {
     }
 }
 
+// One site of the batched sampler, a CTA per sample: X = ell A (d x cr, solver basis), Y = X E.  The mode's
+// conditional density rho[m][m'] = sum_b Y[m][b] conj(X[m'][b]) (d x d), p[n] = sum V[n][m] rho[m][m'] conj(V[n][m'])
+// (V null: the Fock basis, p[n] = rho[n][n]), the draw as in sample_kernel, and the next ell = sum_m V[n][m] X[m] /
+// sqrt(p[n]).  The D levels enter only here, so the two products of a site are D / d times smaller than on
+// rotated tensors and run for all samples at once (64 samples of a 100-mode chi = 96 chain: 78 ms as one CTA per
+// sample over all sites, FP64-pipe bound on 64 SMs).
+__global__ void __launch_bounds__(256) sample_site_kernel(int s, int M, int D, int d, int cr, unsigned k0, unsigned k1, int t0,
+                                                          const double2* __restrict__ X, const double2* __restrict__ Y,
+                                                          const double2* __restrict__ V, double2* __restrict__ ell,
+                                                          int* __restrict__ out) {
+    __shared__ double2 rho[256];  // d <= 16
+    __shared__ double p[1024];    // D in passes of 1024
+    __shared__ int pick;
+    __shared__ double total_sh, p_sh;
+    const int t = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double2* x = X + (long long)t * d * cr;
+    const double2* y = Y + (long long)t * d * cr;
+    for (int e = warp; e < d * d; e += 8) {
+        const double2 *ye = y + (long long)(e / d) * cr, *xe = x + (long long)(e % d) * cr;
+        double re = 0.0, im = 0.0;
+        for (int b = lane; b < cr; b += 32) {
+            const double2 u = ye[b], v = xe[b];
+            re = fma(u.x, v.x, fma(u.y, v.y, re));
+            im = fma(u.y, v.x, fma(-u.x, v.y, im));
+        }
+        re = warp_sum(re);
+        im = warp_sum(im);
+        if (lane == 0) rho[e] = make_double2(re, im);
+    }
+    __syncthreads();
+    auto prob = [&](int n) {
+        double acc = 0.0;
+        if (V == nullptr) {
+            acc = rho[n * d + n].x;
+        } else {
+            for (int m = 0; m < d; ++m) {
+                double re = 0.0, im = 0.0;  // sum_m' rho[m][m'] conj(V[n][m'])
+                for (int q = 0; q < d; ++q) {
+                    const double2 r = rho[m * d + q], v = V[n * d + q];
+                    re = fma(r.x, v.x, fma(r.y, v.y, re));
+                    im = fma(r.y, v.x, fma(-r.x, v.y, im));
+                }
+                const double2 v = V[n * d + m];
+                acc = fma(v.x, re, fma(-v.y, im, acc));
+            }
+        }
+        return fmax(acc, 0.0);
+    };
+    // two passes over the levels (the total, then the draw), 1024 at a time
+    for (int pass = 0; pass < 2; ++pass) {
+        double run = 0.0;
+        bool found = false;
+        for (int n0 = 0; n0 < D; n0 += 1024) {
+            const int cnt = min(1024, D - n0);
+            if (pass == 0 || D > 1024) {
+                for (int n = threadIdx.x; n < cnt; n += 256) p[n] = prob(n0 + n);
+                __syncthreads();
+            }
+            if (threadIdx.x == 0) {
+                if (pass == 0) {
+                    for (int n = 0; n < cnt; ++n) run += p[n];
+                } else if (!found) {
+                    for (int n = 0; n < cnt && !found; ++n) {
+                        run += p[n];
+                        if (run > total_sh) {
+                            found = true;
+                            pick = n0 + n;
+                            p_sh = p[n];
+                        }
+                    }
+                    if (!found && n0 + cnt == D) {
+                        pick = D - 1;
+                        p_sh = p[cnt - 1];
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        if (pass == 0 && threadIdx.x == 0) {
+            unsigned c[4] = {(unsigned)(t0 + t), 0u, (unsigned)s, 2u};
+            philox4x32_10(c, k0, k1);
+            total_sh = uniform53(c[0], c[1]) * run;
+        }
+        __syncthreads();
+    }
+    const int n = pick;
+    if (threadIdx.x == 0) out[(long long)t * M + s] = n;
+    const double inv = 1.0 / sqrt(fmax(p_sh, 1e-300));
+    for (int b = threadIdx.x; b < cr; b += 256) {
+        double2 acc = make_double2(0.0, 0.0);
+        if (V == nullptr) {
+            acc = x[(long long)n * cr + b];
+        } else {
+            for (int m = 0; m < d; ++m) {
+                const double2 v = V[n * d + m], u = x[(long long)m * cr + b];
+                acc.x = fma(v.x, u.x, fma(-v.y, u.y, acc.x));
+                acc.y = fma(v.x, u.y, fma(v.y, u.x, acc.y));
+            }
+        }
+        ell[(long long)t * cr + b] = make_double2(acc.x * inv, acc.y * inv);
+    }
+}
+
+__global__ void fill_one_kernel(double2* p, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) p[i] = make_double2(1.0, 0.0);
+}
+
 // rho[s][t] = sum_{i, c} U[i][s][c] conj(A[i][t][c]) for s, t < d: one CTA per (s, t),
 // fixed-order block sum
 __global__ void __launch_bounds__(256) reduced_density_kernel(int cl, int d, int cr, const double2* __restrict__ U,
@@ -365,6 +473,49 @@ void sample_dev(Ctx& ctx, const double2* const* AF_dev, const double2* const* ER
     sample_kernel<<<n_samples, 256, shm, ctx.stream>>>(a);
     ctx.count_launch();
     ctx.check_launch("sample_kernel");
+}
+
+void sample_limit(Ctx& ctx, int D, int chi_max) {
+    const size_t shm = sizeof(double2) * (size_t)chi_max * (1 + D) + sizeof(double) * D;
+    int optin = 0;
+    VTN_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx.device));
+    cudaFuncAttributes fa;
+    VTN_CUDA_TRY(cudaFuncGetAttributes(&fa, (const void*)sample_kernel));
+    VTN_REQUIRE(shm <= (size_t)optin - fa.sharedSizeBytes,
+                "sampler working set exceeds shared memory (chi_max * (D + 1) too large)");
+}
+
+void sample_batched_dev(Ctx& ctx, const double2* const* sites, const double2* ER, size_t env, const int* dims, const double2* iso,
+                        int M, int D, int d, int chi_max, uint64_t seed, int n_samples, int* out_dev) {
+    const int step = std::min(n_samples, 4096);
+    double2* ell = (double2*)ctx.workspace(WS_SMP, sizeof(double2) * (size_t)step * chi_max * (1 + 2 * (size_t)d));
+    double2* X = ell + (size_t)step * chi_max;
+    double2* Y = X + (size_t)step * chi_max * d;
+    for (int t0 = 0; t0 < n_samples; t0 += step) {
+        const int ns = std::min(step, n_samples - t0);
+        fill_one_kernel<<<(ns + 255) / 256, 256, 0, ctx.stream>>>(ell, ns);
+        ctx.count_launch();
+        for (int s = 0; s < M; ++s) {
+            const int cl = dims[s], cr = dims[s + 1];
+            GemmArgs g1;
+            g1.M = ns; g1.N = d * cr; g1.K = cl;
+            g1.A = ell; g1.lda = cl;
+            g1.B = sites[s]; g1.ldb = (long long)d * cr;
+            g1.C = X; g1.ldc = (long long)d * cr;
+            gemm_c64(ctx, g1);
+            GemmArgs g2;
+            g2.M = ns * d; g2.N = cr; g2.K = cr;
+            g2.A = X; g2.lda = cr;
+            g2.B = ER + env * (s + 1); g2.ldb = cr;
+            g2.C = Y; g2.ldc = cr;
+            gemm_c64(ctx, g2);
+            sample_site_kernel<<<ns, 256, 0, ctx.stream>>>(s, M, D, d, cr, (unsigned)(seed & 0xFFFFFFFFu), (unsigned)(seed >> 32),
+                                                           t0, X, Y, iso ? iso + (size_t)s * D * d : nullptr, ell,
+                                                           out_dev + (size_t)t0 * M);
+            ctx.count_launch();
+        }
+        ctx.check_launch("sample_site_kernel");
+    }
 }
 
 void reduced_density_dev(Ctx& ctx, int cl, int d, int cr, const double2* U, const double2* A, double2* rho) {

@@ -133,6 +133,7 @@ struct Ctx {
     size_t defer_cap = 0;         // doubles
     long long host_syncs = 0;     // stream synchronisations made by sync()
     double* defer_reserve(size_t doubles);  // grows (synchronising first), never shrinks
+    bool dstatus_due = false;  // a kernel with bounded waits was queued since the word was last read
     int* dstatus = nullptr;    // device status word: non-zero after a bounded device wait gave up
     int num_sms = 0;
 
@@ -158,7 +159,7 @@ enum WsSlot {
     WS_TC_A2, WS_TC_PART, WS_GEMM_SPLIT, WS_EIG_PART, WS_TC_ENV, WS_EIG_T, WS_H2_ENV, WS_EXPAND,
     WS_TRUNC_L, WS_TRUNC_R, WS_CENTER, WS_MLP_ACT, WS_MLP_Y, WS_MLP_G, WS_WARM_S, WS_WARM_Z, WS_WARM_P,
     WS_WARM_U, WS_WARM_N, WS_WARM_Q0, WS_CQR_G, WS_CQR_T, WS_CQR_B, WS_RQ_Y, WS_RQ_S, WS_CHOL_LINV, WS_TH_A, WS_TH_B,
-    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_OZ_PREP, WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_N, WS_FLT_U, WS_COUNT
+    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_OZ_PREP, WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_N, WS_FLT_U, WS_SMP, WS_COUNT
 };
 
 // ------------------------------------------------------------------ cores
@@ -421,6 +422,12 @@ void reduced_density_dev(Ctx& ctx, int cl, int d, int cr, const double2* U, cons
 void marginal_reduce_dev(Ctx& ctx, int chi_l, int D, int chi_r, const double2* AF, const double2* U, double* P);
 void sample_dev(Ctx& ctx, const double2* const* AF_dev, const double2* const* ER_dev, const int* dims_dev, int M,
                 int D, int chi_max, uint64_t seed, int n_samples, int* out_dev);
+
+// The same draws by two products per site for all samples at once, in the solver basis; sites, dims: host arrays,
+// ER: [M + 1] right environments env complex apart, iso: isometries (null in the Fock basis)
+void sample_batched_dev(Ctx& ctx, const double2* const* sites, const double2* ER, size_t env, const int* dims, const double2* iso,
+                        int M, int D, int d, int chi_max, uint64_t seed, int n_samples, int* out_dev);
+void sample_limit(Ctx& ctx, int D, int chi_max);  // VTN_EINVAL beyond the sampler's working set
 
 }  // namespace vtn
 
