@@ -220,10 +220,23 @@ void solve_lower_rows(Ctx& ctx, const double2* G, const double2* Linv_all, int m
     }
 }
 
-// before the factorisation: the Gram matrix' diagonal
-__global__ void gram_diagonal(const double2* __restrict__ G, int m, double* __restrict__ d) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < m) d[j] = G[(long long)j * m + j].x;
+// before the factorisation: the Gram matrix' diagonal, after shift * trace is added to it
+__global__ void __launch_bounds__(1024) gram_diagonal(double2* __restrict__ G, int m, double shift, double* __restrict__ d) {
+    __shared__ double sh[32];
+    double tr = 0.0;
+    if (shift > 0.0) {
+        for (int j = threadIdx.x; j < m; j += 1024) tr += G[(long long)j * m + j].x;
+        for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = tr;
+        __syncthreads();
+        tr = 0.0;
+        for (int w = 0; w < 32; ++w) tr += sh[w];
+    }
+    for (int j = threadIdx.x; j < m; j += 1024) {
+        const double g = G[(long long)j * m + j].x + shift * tr;
+        if (shift > 0.0) G[(long long)j * m + j].x = g;
+        d[j] = g;
+    }
 }
 
 // after it: pivots of rows 0, k - 1 and m - 1, the smallest pivot relative to its row's norm, the flag
@@ -249,7 +262,7 @@ __global__ void __launch_bounds__(1024) pivot_info(const double2* __restrict__ G
 
 }  // namespace
 
-void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info) {
+void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info, double shift) {
     const int nblk = (m + NB - 1) / NB;
     double2* G = (double2*)ctx.workspace(WS_CQR_G, sizeof(double2) * ((size_t)m * m + (size_t)nblk * NB * NB + m));
     double2* Linv = G + (size_t)m * m;
@@ -264,7 +277,7 @@ void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info) {
     g.C = G; g.ldc = m;
     g.herm_lower = true;
     gemm_c64(ctx, g);
-    gram_diagonal<<<(m + 255) / 256, 256, 0, ctx.stream>>>(G, m, diag);
+    gram_diagonal<<<1, 1024, 0, ctx.stream>>>(G, m, shift, diag);
     cholesky_blocked(ctx, G, m, Linv, tmp, flag);
     pivot_info<<<1, 1024, 0, ctx.stream>>>(G, m, k, diag, flag, info);
     ctx.count_launch(2);

@@ -168,7 +168,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     // against sliced: 128^3 22 | 34 us, 160^3 34 | 35 us, 192^3 55 | 37 us, 256^3 136 | 38 us, 1024 x 16 x 1024
     // (narrow: padded to 32 columns) 74 | 49 us; at 3072^3 200 ms against 6.1 ms.  Its row sums fit 96-bit integers
     // for summations of up to 2^19 terms.
-    const bool oz = g.prepA != nullptr || ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.5e6 && (long long)g.K * g.kb <= (1LL << 19);
+    const bool oz = g.prepA != nullptr || ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.2e6 && (long long)g.K * g.kb <= (1LL << 19);
     int S = 1;
     if (oz) {
         S = oz_splits(ctx, g);

@@ -421,11 +421,12 @@ void orthonormalize_rows_small(Ctx& ctx, double2* A, int rows, int cols, const i
     ctx.check_launch("orth_rows_kernel");
 }
 
-// Gram-Schmidt of the rows in order.  Small problems run the single-CTA kernel; from 128 rows
-// and 2^25 complex multiply-adds on, CholeskyQR2 on the GEMM (same result, all SMs).
+// Gram-Schmidt of the rows in order.  Small problems run the single-CTA kernel (2 rows^2 cols complex multiply-adds
+// on one SM's FP64 pipe: 2 ms at 40 x 240, 11 ms at 64 x 512, 43 ms at 128 x 768); from 40 rows and 2^18 of them
+// on, CholeskyQR2 on the GEMM (0.7, 0.9 and 1.7 ms; same result, all SMs).
 void orthonormalize_rows(Ctx& ctx, double2* A, int rows, int cols) {
     VTN_REQUIRE(rows <= 4096 && rows <= cols, "row orthonormalisation needs rows <= min(cols, 4096)");
-    if (rows >= 128 && (double)rows * rows * cols >= 33554432.0) orthonormalize_rows_cholqr(ctx, A, rows, cols);
+    if (rows >= 40 && (double)rows * rows * cols >= 262144.0) orthonormalize_rows_cholqr(ctx, A, rows, cols);
     else orthonormalize_rows_small(ctx, A, rows, cols, nullptr);
 }
 

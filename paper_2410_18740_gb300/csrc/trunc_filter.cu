@@ -61,10 +61,14 @@ __global__ void __launch_bounds__(256) row_norm_max(const double2* __restrict__ 
 
 }  // namespace
 
-// Block size 1.5 k + 16 in tiles of 32, from n = 257 on and where the block is at most half of rho.
+// Block size 1.5 k + 16 in tiles of 32, from n = 257 on and where the block is at most half of rho.  Where T's other
+// side r is no larger than that, the block is T's own range (r rows, no iteration): at the ends of a chain, where
+// rho is n x n of rank r = n / d.
 int filter_rows(int nL, int nR, int direction, int k) {
-    const int n = direction == 0 ? nL : nR, m = (3 * k / 2 + 16 + 31) / 32 * 32;
-    return n > 256 && n <= 4096 && 2 * m <= n && m <= std::min(nL, nR) ? m : 0;
+    const int n = direction == 0 ? nL : nR, other = direction == 0 ? nR : nL, m = (3 * k / 2 + 16 + 31) / 32 * 32;
+    if (n <= 256) return 0;
+    if (2 * other <= n && other <= 4096 && (other <= m || n > 4096)) return other;
+    return n <= 4096 && 2 * m <= n && m <= other ? m : 0;
 }
 
 bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, const double2* theta, double2* left,
@@ -82,9 +86,14 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
             if (t >= 0) c.tend(t);
         }
     } guard{ctx, timing, tt};
-    double2* rho = (double2*)ctx.workspace(WS_EIG_A, sizeof(double2) * (size_t)n * n);
-    density_dev(ctx, nL, nR, direction, theta, rho);
-    const OzPrep prep = oz_prepare(ctx, n, n, OP_T, rho, n);
+    const bool range = m == other;
+    double2* rho = nullptr;
+    OzPrep prep;
+    if (!range) {
+        rho = (double2*)ctx.workspace(WS_EIG_A, sizeof(double2) * (size_t)n * n);
+        density_dev(ctx, nL, nR, direction, theta, rho);
+        prep = oz_prepare(ctx, n, n, OP_T, rho, n);
+    }
     double2* S = (double2*)ctx.workspace(WS_FLT_S, sizeof(double2) * (size_t)mn);
     double2* X = (double2*)ctx.workspace(WS_FLT_X, sizeof(double2) * (size_t)mn);
     double2* P = (double2*)ctx.workspace(WS_FLT_P, sizeof(double2) * (size_t)m * std::max(n, other));
@@ -107,75 +116,96 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
         // NaN fails every comparison
         return ctx.pinned[4] == 0.0 && pivot > 1e-7 && lk > 0.0 && l1 < 1e300;
     };
-    // ---- two plain products of a random block: eigenvalue estimates from the second one's pivots
-    fill_random_normal(ctx, S, mn, 0x5eedull, n, PHILOX_STREAM_TRUNC);
-    apply(S, P);
-    if (!orth(P)) return false;
-    apply(P, S);
-    if (!orth(S)) return false;
-    if (!(lm > 1e-12 * l1) || !(lk > lm)) return false;
-    const double b = lm, lam1 = l1;
-    const double g1 = std::acosh(2.0 * 1.6 * lam1 / b - 1.0);  // growth per degree; the largest pivot reads low
-    double gk = std::acosh(2.0 * lk / b - 1.0);
-    // Degrees that cost as much as the reduction: 8.9 ms at n = 512, 30 at 1024 and 86 at 1830, against 5, 8 and
-    // 20 ms of orthonormalisation and Rayleigh-Ritz and 40, 60 and 110 us a degree.
-    const double limit = 40.0 * std::pow(n / 512.0, 1.6);
-    if (!(35.0 / gk <= limit)) return false;
-    double grown = 0.0, degrees = 0.0;
-    bool done = false;
-    for (int cycle = 0; cycle < 32 && !done; ++cycle) {
-        // the first block is not in Schur order yet: its rows may part by 1e5 only; later ones by 1e11
-        int D = (int)(std::log(cycle == 0 ? 1e5 : 1e11) / g1);
-        D = std::max(2, std::min({D, 12, (int)std::ceil((36.0 - grown) / gk)}));
-        degrees += D;
-        if (degrees > 2.0 * limit) return false;
+    auto iterate = [&]() -> bool {
+        // ---- two plain products of a random block: eigenvalue estimates from the second one's pivots
+        fill_random_normal(ctx, S, mn, 0x5eedull, n, PHILOX_STREAM_TRUNC);
         apply(S, P);
-        cheb_step<<<(unsigned)((mn + 255) / 256), 256, 0, ctx.stream>>>(mn, 2.0 / b, P, -1.0, S, 0.0, nullptr, X);
-        double2 *prev = S, *cur = X;
-        for (int i = 1; i < D; ++i) {
-            apply(cur, P);
-            cheb_step<<<(unsigned)((mn + 255) / 256), 256, 0, ctx.stream>>>(mn, 4.0 / b, P, -2.0, cur, -1.0, prev, prev);
-            std::swap(prev, cur);
-        }
-        ctx.count_launch(D);
-        ctx.check_launch("cheb_step");
-        S = cur;
-        X = prev;
+        if (!orth(P)) return false;
+        apply(P, S);
         if (!orth(S)) return false;
-        grown += std::log(lk);
-        gk = std::log(lk) / D;
-        if (!(gk > 0.0)) return false;
-        if (grown < 35.0) {
-            if (!(degrees + (35.0 - grown) / gk <= 2.0 * limit)) return false;
-            continue;
+        if (!(lm > 1e-12 * l1) || !(lk > lm)) return false;
+        const double b = lm, lam1 = l1;
+        const double g1 = std::acosh(2.0 * 1.6 * lam1 / b - 1.0);  // growth per degree; the largest pivot reads low
+        double gk = std::acosh(2.0 * lk / b - 1.0);
+        // Degrees that cost as much as the reduction: 8.9 ms at n = 512, 30 at 1024 and 86 at 1830, against 5, 8 and
+        // 20 ms of orthonormalisation and Rayleigh-Ritz and 40, 60 and 110 us a degree.
+        const double limit = 40.0 * std::pow(n / 512.0, 1.6);
+        if (!(35.0 / gk <= limit)) return false;
+        double grown = 0.0, degrees = 0.0;
+        bool done = false;
+        for (int cycle = 0; cycle < 32 && !done; ++cycle) {
+            // the first block is not in Schur order yet: its rows may part by 1e5 only; later ones by 1e11
+            int D = (int)(std::log(cycle == 0 ? 1e5 : 1e11) / g1);
+            D = std::max(2, std::min({D, 12, (int)std::ceil((36.0 - grown) / gk)}));
+            degrees += D;
+            if (degrees > 2.0 * limit) return false;
+            apply(S, P);
+            cheb_step<<<(unsigned)((mn + 255) / 256), 256, 0, ctx.stream>>>(mn, 2.0 / b, P, -1.0, S, 0.0, nullptr, X);
+            double2 *prev = S, *cur = X;
+            for (int i = 1; i < D; ++i) {
+                apply(cur, P);
+                cheb_step<<<(unsigned)((mn + 255) / 256), 256, 0, ctx.stream>>>(mn, 4.0 / b, P, -2.0, cur, -1.0, prev, prev);
+                std::swap(prev, cur);
+            }
+            ctx.count_launch(D);
+            ctx.check_launch("cheb_step");
+            S = cur;
+            X = prev;
+            if (!orth(S)) return false;
+            grown += std::log(lk);
+            gk = std::log(lk) / D;
+            if (!(gk > 0.0)) return false;
+            if (grown < 35.0) {
+                if (!(degrees + (35.0 - grown) / gk <= 2.0 * limit)) return false;
+                continue;
+            }
+            // the pass lost orthogonality like u / pivot^2
+            if (pivot < 0.2 && !orth(S)) return false;
+            // ---- residual of the first k rows: S rho - (S rho S^dag) S
+            apply(S, P);
+            GemmArgs h;
+            h.M = m; h.N = m; h.K = n;
+            h.A = P; h.lda = n;
+            h.opB = OP_C; h.B = S; h.ldb = n;
+            h.C = H; h.ldc = m;
+            gemm_c64(ctx, h);
+            GemmArgs r;
+            r.M = k; r.N = n; r.K = m;
+            r.A = H; r.lda = m;
+            r.B = S; r.ldb = n;
+            r.C = P; r.ldc = n;
+            r.accumulate = true; r.negate = true;
+            gemm_c64(ctx, r);
+            VTN_CUDA_TRY(cudaMemsetAsync(num + 5, 0, sizeof(double), ctx.stream));
+            row_norm_max<<<k, 256, 0, ctx.stream>>>(P, n, (unsigned long long*)(num + 5));
+            ctx.count_launch();
+            ctx.check_launch("row_norm_max");
+            VTN_CUDA_TRY(cudaMemcpyAsync(ctx.pinned, num + 5, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
+            ctx.sync();
+            done = std::sqrt(ctx.pinned[0]) <= 4e-15 * lam1;
+            if (!done && grown > 60.0) return false;
         }
-        // the pass lost orthogonality like u / pivot^2
-        if (pivot < 0.2 && !orth(S)) return false;
-        // ---- residual of the first k rows: S rho - (S rho S^dag) S
-        apply(S, P);
-        GemmArgs h;
-        h.M = m; h.N = m; h.K = n;
-        h.A = P; h.lda = n;
-        h.opB = OP_C; h.B = S; h.ldb = n;
-        h.C = H; h.ldc = m;
-        gemm_c64(ctx, h);
-        GemmArgs r;
-        r.M = k; r.N = n; r.K = m;
-        r.A = H; r.lda = m;
-        r.B = S; r.ldb = n;
-        r.C = P; r.ldc = n;
-        r.accumulate = true; r.negate = true;
-        gemm_c64(ctx, r);
-        VTN_CUDA_TRY(cudaMemsetAsync(num + 5, 0, sizeof(double), ctx.stream));
-        row_norm_max<<<k, 256, 0, ctx.stream>>>(P, n, (unsigned long long*)(num + 5));
-        ctx.count_launch();
-        ctx.check_launch("row_norm_max");
-        VTN_CUDA_TRY(cudaMemcpyAsync(ctx.pinned, num + 5, sizeof(double), cudaMemcpyDeviceToHost, ctx.stream));
-        ctx.sync();
-        done = std::sqrt(ctx.pinned[0]) <= 4e-15 * lam1;
-        if (!done && grown > 60.0) return false;
+        return done;
+    };
+    if (range) {
+        // the rows of T (or of T^dag) span everything; two passes, as one loses u (|T| / smallest singular value)^2
+        auto load = [&]() {
+            if (direction == 0) conj_transpose_dev(ctx, nL, nR, theta, nR, S, nL);
+            else VTN_CUDA_TRY(cudaMemcpyAsync(S, theta, sizeof(double2) * (size_t)mn, cudaMemcpyDeviceToDevice, ctx.stream));
+        };
+        load();
+        if (!orth(S)) {
+            // ill-conditioned: shifted passes first (Fukaya et al. 2020), each of which takes a factor of about 1e7 off
+            load();
+            const double shift = 11.0 * ((double)mn + (double)m * (m + 1)) * 1.1e-16;
+            cholqr_pass(ctx, S, m, n, k, num, shift);
+            cholqr_pass(ctx, S, m, n, k, num, shift);
+            if (!orth(S)) return false;
+        }
+        if (!orth(S) || !(pivot > 0.5)) return false;
+    } else if (!iterate()) {
+        return false;
     }
-    if (!done) return false;
     // ---- Rayleigh-Ritz: the exact truncation of the projected tensor
     norm2_dev(ctx, theta, (long long)nL * nR, num + 6);
     ctx.timing = false;

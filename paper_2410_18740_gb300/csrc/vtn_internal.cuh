@@ -401,7 +401,8 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
                        double2* right, int outer, double* defer, TruncResult& res);
 // One CholeskyQR pass over the rows of A (m x n) in place (chol_qr.cu); info (device double[5]) = the pivots of row
 // 0, row k - 1 and row m - 1, the smallest pivot relative to its row's norm, and 1 if a pivot was not positive.
-void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info);
+// shift > 0: shift * trace is added to the Gram matrix' diagonal (shifted Cholesky-QR, for ill-conditioned rows).
+void cholqr_pass(Ctx& ctx, double2* A, int m, int n, int k, double* info, double shift = 0.0);
 
 // ------------------------------------------------------------------ misc kernels
 // Philox counter word 3: the stream of the random numbers (initial MPS, sampler, truncation)

@@ -66,3 +66,29 @@ def test_large_truncation_matches_the_svd(ctx, shape, kind, direction):
     assert np.linalg.norm(got) ** 2 >= (S[:k] ** 2).sum() - 8 * n * u * k * S[0] ** 2
     if kind == "decaying":
         assert launches > 120, launches  # the full reduction takes about 30
+
+
+# one side of the tensor at most half of the other: the block is the tensor's own range
+@pytest.mark.parametrize("shape,direction", [((8, 8, 8, 64, 64), 1), ((70, 5, 5, 11, 30), 0), ((1, 6, 6, 61, 6), 1)])
+@pytest.mark.parametrize("decay", [0.0, 9.0, 60.0])  # the last is too ill-conditioned for it
+def test_truncation_of_a_density_matrix_of_low_rank(ctx, shape, direction, decay):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    cl, d1, d2, cr, k = shape
+    n1, n2 = cl * d1, d2 * cr
+    rng = np.random.default_rng(n1 + 3 * n2)
+    r = min(n1, n2)
+    T = _tensor(rng, n1, n2, np.exp(-decay * np.arange(r) / r))
+    th = torch.from_numpy(np.ascontiguousarray(T)).cuda()
+    left = torch.empty(n1, k, dtype=torch.complex128, device="cuda")
+    right = torch.empty(k, n2, dtype=torch.complex128, device="cuda")
+    kk, lam, disc = vtn.vtn_truncate(ctx, cl, d1, d2, cr, direction, k, th, left, right)
+    U, S, Vh = np.linalg.svd(T, full_matrices=False)
+    n, u = max(n1, n2), 2.0 ** -53
+    assert kk == k and np.abs(lam - S[:k] ** 2).max() <= 4 * n * u * S[0] ** 2
+    iso = left if direction == 0 else right.conj().T
+    assert float((iso.conj().T @ iso - torch.eye(k, dtype=torch.complex128, device="cuda")).abs().max()) <= 4 * n * u
+    got = (left @ right).cpu().numpy()
+    assert np.linalg.norm(got) ** 2 >= (S[:k] ** 2).sum() - 8 * n * u * k * S[0] ** 2
+    if k == r:
+        assert np.linalg.norm(got - T) <= 4 * n * u * S[0] * np.sqrt(k)
