@@ -52,6 +52,21 @@ __device__ double block_sum(double v, double* sh) {
     return r;  // valid in every thread
 }
 
+// The same for values of which only those of threads t < m (per stride of the block) can be non-zero: the warps
+// beyond them add nothing and stay off the FP64 pipe.  Two calls in a row need different sh.
+__device__ double block_sum_first(double v, double* sh, int m) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid * 32 < m) v = warp_sum(v);
+    if (lane == 0) sh[wid] = v;
+    __syncthreads();
+    if (wid == 0) {
+        const double r = warp_sum((lane < (int)(blockDim.x >> 5)) ? sh[lane] : 0.0);
+        if (lane == 0) sh[32] = r;
+    }
+    __syncthreads();
+    return sh[32];  // valid in every thread
+}
+
 struct EigSmall {
     double* diag;   // [n]
     double* offd;   // [n]
@@ -292,24 +307,33 @@ __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
+    unsigned o;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(o) : "l"(p), "r"(v) : "memory");
+    return o;
+}
+
 // Grid barrier number `epoch` (0, 1, 2, ... in every CTA): each CTA adds its arrival to a
 // monotonic counter (fire-and-forget reduction) and polls it until it reaches
-// (epoch + 1) * nblocks (about 1.5 us for 152 CTAs on GB300; a CTA that releases the others
-// through a second word takes about 2.5 us).  Waits are bounded (2 s): a CTA that gives up
+// (epoch + 1) * nblocks (a CTA that releases the others through a second word takes a microsecond more).
+// The CTA barrier before the release and after the acquire orders the other threads' accesses
+// (release and acquire are cumulative), so no separate fence is needed: a fence costs
+// about 0.4 us, and a column's chain had five of them.  Waits are bounded (2 s): a CTA that gives up
 // sets bar->error, which the other pollers check every 256 polls; all CTAs then return
-// false and the kernel exits.
-__device__ bool grid_sync(GridBar* bar, unsigned int nblocks, unsigned int epoch) {
+// false and the kernel exits.  `meanwhile` runs in warp 1 while thread 0 polls.
+template <class F>
+__device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned int nblocks, unsigned int epoch, F&& meanwhile) {
     __shared__ int ok_sh;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         red_release_add(&bar->count, 1u);
         const unsigned target = (epoch + 1u) * nblocks;
         bool ok = true;
-        const unsigned long long t0 = global_ns();
         unsigned polls = 0;
+        unsigned long long t0 = 0;
         while (ld_acquire_u32(&bar->count) < target) {
             if ((++polls & 255u) == 0) {
+                if (t0 == 0) t0 = global_ns();
                 if (*(volatile int*)&bar->error != 0 || global_ns() - t0 > 2000000000ull) {
                     atomicExch(&bar->error, 1);
                     ok = false;
@@ -317,11 +341,15 @@ __device__ bool grid_sync(GridBar* bar, unsigned int nblocks, unsigned int epoch
                 }
             }
         }
-        __threadfence();
         ok_sh = ok ? 1 : 0;
+    } else if ((threadIdx.x >> 5) == 1) {
+        meanwhile();
     }
     __syncthreads();
     return ok_sh != 0;
+}
+__device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned int nblocks, unsigned int epoch) {
+    return grid_sync(bar, nblocks, epoch, [] {});
 }
 
 __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {  // a * conj(b)
@@ -371,20 +399,36 @@ __device__ __forceinline__ int tri_pass_cost(int m, int nb, int cpl) {
     return passes * rows * cpl;
 }
 
+// The trailing pass of a column: columns per lane, chunks, row slices, and whether every CTA sums the chunks'
+// partials itself after the barrier.  The last CTA of a chunk to arrive costs an atomic, two round trips to
+// L2 and a CTA barrier, about 1.4 us; the redundant sums cost ceil(m / 128) CS adds of 64 cycles and a real and
+// imaginary part, which is less up to m ~ 256.  Both add the slices in order.
+struct TriPlan {
+    int cpl, C, CS, all_sum;
+};
+__device__ __forceinline__ TriPlan tri_plan(int m, int nb) {
+    TriPlan p;
+    p.cpl = tri_pass_cost(m, nb, 2) < tri_pass_cost(m, nb, 1) ? 2 : 1;
+    tri_layout(m, nb, p.cpl, p.C, p.CS);
+    p.all_sum = (m + 127) / 128 * p.CS <= 16;
+    return p;
+}
+
 // Trailing pass of step k: pending rank-2 update of the trailing block fused with (A v).  Work
 // unit u = (column chunk c = u mod C of 32*CPL columns, row slice cs = u / C of CS); CTA b
 // takes units b, b + nb, ...; warp w walks the rows k+1 + cs*NW + w + t*CS*NW, lane l owns the
 // columns c*32*CPL + q*32 + l (q < CPL).  The CTAs of a chunk each write one partial (A v) per
-// column; the last to arrive sums them in slice order into p = tau A v.
+// column; the last to arrive sums them in slice order into p = tau A v (or every CTA does after the
+// barrier: TriPlan::all_sum).
 template <int CPL>
 __device__ void tri_pass(double2* __restrict__ A, int n, int k, int m, int nb, bool have_prev,
                          const double2* vprev, const double2* wprev, const double2* vcur, double tau,
-                         double2* pk, double2* pfin, unsigned* arrive, double2* colred, int& last_sh) {
+                         double2* pk, double2* pfin, unsigned* arrive, double2* colred, int& last_sh,
+                         const TriPlan& plan) {
     constexpr int U = TRI_UNROLL / CPL;  // rows in flight per warp
     constexpr int LD = TRI_MAX_CPL * 32;  // colred row stride
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int C, CS;
-    tri_layout(m, nb, CPL, C, CS);
+    const int C = plan.C, CS = plan.CS;
     for (int unit = (int)blockIdx.x; unit < C * CS; unit += nb) {
         const int c = unit % C, cs = unit / C;
         int il[CPL], col[CPL];
@@ -467,17 +511,13 @@ __device__ void tri_pass(double2* __restrict__ A, int n, int k, int m, int nb, b
                 const double2 a0 = colred[q * 32 + lane], a1 = colred[LD + q * 32 + lane];
                 if (ok[q]) pk[(long long)cs * n + il[q]] = make_double2(a0.x + a1.x, a0.y + a1.y);
             }
-            __threadfence();
         }
         __syncthreads();
+        if (plan.all_sum) continue;  // (colred is free again; the grid barrier releases the partials)
         // the last CTA of this chunk sums its CS partials in slice order (warp q: columns q*32..)
-        if (threadIdx.x == 0) {
-            __threadfence();
-            last_sh = atomicAdd(&arrive[c], 1u) == (unsigned)(CS - 1);
-        }
+        if (threadIdx.x == 0) last_sh = atom_add_acq_rel(&arrive[c], 1u) == (unsigned)(CS - 1);
         __syncthreads();
         if (last_sh && warp < CPL) {
-            __threadfence();
             const int ilq = c * 32 * CPL + warp * 32 + lane;
             if (ilq < m) {
                 double sx = 0.0, sy = 0.0;
@@ -504,13 +544,15 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_persistent(double2* __res
     double2* vprev = sm;
     double2* wprev = sm + n;
     double2* vcur = sm + 2 * n;
-    __shared__ double red[33];
+    __shared__ double red[2][33];
     __shared__ double tau_sh, dk_sh;
     __shared__ double2 p0_sh;
     __shared__ int last_sh;
+    __shared__ TriPlan plan_sh;
     __shared__ double2 colred[TRI_NW][TRI_MAX_CPL * 32];
     const int nb = (int)gridDim.x;
     bool have_prev = false;
+    if (threadIdx.x == 32) plan_sh = tri_plan(n - 1, nb);
     // row 0 (no pending update): x = conj(A[0][1..n-1])
     double a2 = 0.0;
     for (int t = threadIdx.x; t < n - 1; t += blockDim.x) {
@@ -523,7 +565,7 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_persistent(double2* __res
     for (int k = 0; k + 2 < n; ++k) {
         const int m = n - k - 1;
         // ---- reflector for column k from x = vcur (norm^2 a2)
-        a2 = block_sum(a2, red);
+        a2 = block_sum_first(a2, red[0], m);
         if (threadIdx.x == 0) {
             // alpha = |x|, phi = x0 / |x0|: v0 = x0 + phi alpha, beta = -phi alpha,
             // tau = 1 / (alpha (alpha + |x0|)); with few FP64 instructions (two reciprocal
@@ -568,22 +610,41 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_persistent(double2* __res
         double2* pk = tb.part + (long long)(k & 1) * nb * n;
         double2* pfin = tb.p + (long long)(k & 1) * n;
         unsigned* arrive = tb.arrive + (k & 1) * TRI_MAX_CHUNKS;
-        if (tri_pass_cost(m, nb, 2) < tri_pass_cost(m, nb, 1))
-            tri_pass<2>(A, n, k, m, nb, have_prev, vprev, wprev, vcur, tau, pk, pfin, arrive, &colred[0][0], last_sh);
+        const TriPlan plan = plan_sh;  // (computed while the last barrier was waited for)
+        if (plan.cpl == 2)
+            tri_pass<2>(A, n, k, m, nb, have_prev, vprev, wprev, vcur, tau, pk, pfin, arrive, &colred[0][0], last_sh, plan);
         else
-            tri_pass<1>(A, n, k, m, nb, have_prev, vprev, wprev, vcur, tau, pk, pfin, arrive, &colred[0][0], last_sh);
-        if (!grid_sync(bar, (unsigned)nb, (unsigned)k)) return;
+            tri_pass<1>(A, n, k, m, nb, have_prev, vprev, wprev, vcur, tau, pk, pfin, arrive, &colred[0][0], last_sh, plan);
+        if (!grid_sync(bar, (unsigned)nb, (unsigned)k, [&] {
+                if (threadIdx.x == 32) plan_sh = tri_plan(m - 1, nb);
+            }))
+            return;
         // ---- C(k): K = (tau/2) Re(v^dag p); p parked in wprev (its old content is spent)
         const bool next = k + 3 < n;  // another reflector follows
         double dot = 0.0;
+        // the next diagonal entry, raw (its load is off the chain here)
+        const double dk_raw = threadIdx.x == 0 && next ? __ldcg(&A[(long long)(k + 1) * n + (k + 1)]).x : 0.0;
         for (int t = threadIdx.x; t < m; t += blockDim.x) {
-            const double2 p = __ldcg(&pfin[t]), v = vcur[t];
+            const double2 v = vcur[t];
             if (next && t >= 1) vprev[t - 1] = __ldcg(&A[(long long)(k + 1) * n + (k + 1 + t)]);  // row k+1, raw
+            double2 p;
+            if (plan.all_sum) {
+                double sx = 0.0, sy = 0.0;
+#pragma unroll 4
+                for (int s2 = 0; s2 < plan.CS; ++s2) {
+                    const double2 pp = __ldcg(&pk[(long long)s2 * n + t]);
+                    sx += pp.x;
+                    sy += pp.y;
+                }
+                p = make_double2(tau * sx, tau * sy);
+            } else {
+                p = __ldcg(&pfin[t]);
+            }
             wprev[t] = p;
             if (t == 0) p0_sh = p;
             dot = fma(v.x, p.x, fma(v.y, p.y, dot));
         }
-        dot = block_sum(dot, red);
+        dot = block_sum_first(dot, red[1], m);
         const double K = 0.5 * tau * dot;
         // rotate: the pending pair becomes (v_k, w_k); the free buffer takes row k+1
         double2* vnew = vcur;
@@ -605,7 +666,7 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_persistent(double2* __res
                 a2 = fma(x.x, x.x, fma(x.y, x.y, a2));
             }
         }
-        if (threadIdx.x == 0 && next) dk_sh = __ldcg(&A[(long long)(k + 1) * n + (k + 1)]).x - 2.0 * (v0.x * w0.x + v0.y * w0.y);
+        if (threadIdx.x == 0 && next) dk_sh = dk_raw - 2.0 * (v0.x * w0.x + v0.y * w0.y);
         vprev = vnew;
         wprev = wnew;
         vcur = xnext;
