@@ -163,18 +163,25 @@ void destroy_mps(vtn_mps m) {
     delete m;
 }
 
-// A core uploaded for the duration of one call (kernel-level entry points).
+// A core uploaded for the duration of one call (kernel-level entry points) into a workspace slot.  The calls end
+// with a synchronisation, so the staging memory is free again for the next one; on an exception the destructor waits.
 struct TempCore {
     Ctx* c;
     DevCore dc;
-    TempCore(Ctx& ctx, const HostCore& h, bool fp64 = true) : c(&ctx) { upload_core(ctx, h, dc, fp64); }
+    TempCore(Ctx& ctx, const HostCore& h, int what = CORE_F64, int slot = WS_CORE_A) : c(&ctx) {
+        upload_core(ctx, h, dc, what, slot);
+    }
+    TempCore(const TempCore&) = delete;
     ~TempCore() {
-        if (c) {
-            cudaStreamSynchronize(c->stream);
-            free_core(*c, dc);
-        }
+        if (std::uncaught_exceptions() > 0) cudaStreamSynchronize(c->stream);
     }
 };
+
+// End of a kernel-level call: waits for its work and reports a bounded wait that gave up.
+void finish(Ctx& c) {
+    if (c.dstatus_due) c.check_dstatus();
+    else c.sync();
+}
 
 // The term form of a bond given as two cores, for the duration of one call.
 struct TempTerms {
@@ -363,7 +370,7 @@ vtn_status vtn_create(vtn_ctx* out, int device, void* cuda_stream, const vtn_all
             c.has_alloc = true;
         }
         VTN_CUDA_TRY(cudaDeviceGetAttribute(&c.num_sms, cudaDevAttrMultiProcessorCount, device));
-        VTN_CUDA_TRY(cudaMallocHost((void**)&c.pinned, sizeof(double) * 4096));
+        VTN_CUDA_TRY(cudaMallocHost((void**)&c.pinned, sizeof(double) * (Ctx::PINNED + 2 * Ctx::STAGE)));
         c.ws.resize(WS_COUNT);
         c.dstatus = (int*)c.dalloc(256);
         VTN_CUDA_TRY(cudaMemsetAsync(c.dstatus, 0, 256, c.stream));
@@ -1765,21 +1772,27 @@ vtn_status vtn_heff_apply(vtn_ctx ctx, const vtn_core* Wi, const vtn_core* Wj, i
             throw Error{VTN_EUNSUPPORTED, "VTN_TF32X3 is not available in this build"};
         Ctx& c = ctx->c;
         use_device(c);
-        HostCore hi = core_from_abi(Wi), hj = core_from_abi(Wj);
+        HostCore hi = core_from_abi(Wi, false), hj = core_from_abi(Wj, false);
         VTN_REQUIRE(hi.wr == hj.wl && hi.d == hj.d, "Wi.w_right must equal Wj.w_left and d must agree");
-        TempCore ci(c, hi, prec == VTN_FP64), cj(c, hj, prec == VTN_FP64);
         if (prec == VTN_BF16X3) {
             TempTerms tt(c, hi, hj);
             HeffPacked pk;
-            heff_pack_envs(c, ci.dc, cj.dc, chi_l, chi_r, (const double2*)L, (const double2*)R, pk,
-                           tt.bt.worthwhile ? &tt.bt : nullptr);
+            if (tt.bt.usable && tt.bt.worthwhile) {  // the cores themselves are not needed
+                heff_pack_terms(c, tt.bt, chi_l, chi_r, (const double2*)L, (const double2*)R, pk);
+                heff_apply_terms(c, pk, (const double2*)theta, (double2*)y);
+                finish(c);
+                return VTN_OK;
+            }
+            TempCore ci(c, hi, CORE_F32, WS_CORE_A), cj(c, hj, CORE_F32, WS_CORE_B);
+            heff_pack_envs(c, ci.dc, cj.dc, chi_l, chi_r, (const double2*)L, (const double2*)R, pk, nullptr);
             heff_apply_bf16x3(c, ci.dc, cj.dc, pk, (const double2*)theta, (double2*)y);
+            finish(c);
         } else {
+            TempCore ci(c, hi, CORE_F64, WS_CORE_A), cj(c, hj, CORE_F64, WS_CORE_B);
             heff_apply_dev(c, ci.dc, cj.dc, chi_l, chi_r, (const double2*)L, (const double2*)R,
                            (const double2*)theta, (double2*)y);
+            finish(c);
         }
-        c.sync();
-        c.check_dstatus();
         return VTN_OK;
     });
 }
@@ -1795,8 +1808,8 @@ vtn_status vtn_env_update(vtn_ctx ctx, const vtn_core* W, int side, int chi_l, i
             throw Error{VTN_EUNSUPPORTED, "VTN_TF32X3 is not available in this build"};
         Ctx& c = ctx->c;
         use_device(c);
-        HostCore h = core_from_abi(W);
-        TempCore tc(c, h, prec == VTN_FP64);
+        HostCore h = core_from_abi(W, false);
+        TempCore tc(c, h, prec == VTN_FP64 ? CORE_F64 : CORE_F32);
         const double2* e = (const double2*)env;
         const double2* a = (const double2*)A;
         double2* o = (double2*)out;
@@ -1807,8 +1820,7 @@ vtn_status vtn_env_update(vtn_ctx ctx, const vtn_core* W, int side, int chi_l, i
             if (side == 0) env_left_dev(c, tc.dc, chi_l, chi_r, e, a, o);
             else env_right_dev(c, tc.dc, chi_l, chi_r, e, a, o);
         }
-        c.check_dstatus();
-        c.sync();
+        finish(c);
         return VTN_OK;
     });
 }
@@ -1822,11 +1834,10 @@ vtn_status vtn_heff1_apply(vtn_ctx ctx, const vtn_core* W, int chi_l, int chi_r,
         VTN_REQUIRE(A != y, "y must not alias A");
         Ctx& c = ctx->c;
         use_device(c);
-        HostCore h = core_from_abi(W);
+        HostCore h = core_from_abi(W, false);
         TempCore tc(c, h);
         heff1_apply_dev(c, tc.dc, chi_l, chi_r, (const double2*)L, (const double2*)R, (const double2*)A, (double2*)y);
-        c.sync();
-        c.check_dstatus();
+        finish(c);
         return VTN_OK;
     });
 }
@@ -1842,14 +1853,13 @@ vtn_status vtn_expand(vtn_ctx ctx, const vtn_core* W, int side, int chi_l, int c
         VTN_REQUIRE(A != out && env != out, "out must not alias the inputs");
         Ctx& c = ctx->c;
         use_device(c);
-        HostCore h = core_from_abi(W);
+        HostCore h = core_from_abi(W, false);
         TempCore tc(c, h);
         if (side == 0)
             expand_right_dev(c, tc.dc, chi_l, chi_r, (const double2*)env, (const double2*)A, alpha, (double2*)out);
         else
             expand_left_dev(c, tc.dc, chi_l, chi_r, (const double2*)env, (const double2*)A, alpha, (double2*)out);
-        c.sync();
-        c.check_dstatus();
+        finish(c);
         return VTN_OK;
     });
 }
@@ -1863,9 +1873,9 @@ vtn_status vtn_heff_ground(vtn_ctx ctx, const vtn_core* Wi, const vtn_core* Wj, 
         VTN_REQUIRE(chi_l >= 1 && chi_r >= 1, "bond dimensions must be >= 1");
         Ctx& c = ctx->c;
         use_device(c);
-        HostCore hi = core_from_abi(Wi), hj = core_from_abi(Wj);
+        HostCore hi = core_from_abi(Wi, false), hj = core_from_abi(Wj, false);
         VTN_REQUIRE(hi.wr == hj.wl && hi.d == hj.d, "Wi.w_right must equal Wj.w_left and d must agree");
-        TempCore ci(c, hi), cj(c, hj);
+        TempCore ci(c, hi, CORE_F64, WS_CORE_A), cj(c, hj, CORE_F64, WS_CORE_B);
         const long long n = (long long)chi_l * hi.d * hi.d * chi_r;
         LanczosResult lr = lanczos(c, n, (double2*)theta, tol, krylov_max, max_restarts,
                                    [&](const double2* in, double2* out) {

@@ -131,7 +131,7 @@ void Ctx::check_launch(const char* what) {
 }
 
 // ------------------------------------------------------------------ cores
-HostCore core_from_abi(const vtn_core* c) {
+HostCore core_from_abi(const vtn_core* c, bool copy) {
     VTN_REQUIRE(c != nullptr, "null core");
     VTN_REQUIRE(c->w_left >= 1 && c->w_right >= 1 && c->d >= 1 && c->d <= 16 && c->nnz >= 0,
                 "core shape out of range (need w >= 1, 1 <= d <= 16)");
@@ -140,26 +140,34 @@ HostCore core_from_abi(const vtn_core* c) {
     h.wl = c->w_left;
     h.wr = c->w_right;
     h.d = c->d;
-    const int dd = c->d * c->d;
-    for (int k = 0; k < c->nnz; ++k) {
+    const int dd = c->d * c->d, nnz = c->nnz;
+    for (int k = 0; k < nnz; ++k)
         VTN_REQUIRE(c->rows[k] >= 0 && c->rows[k] < c->w_left && c->cols[k] >= 0 && c->cols[k] < c->w_right,
                     "core entry channel out of range");
-        h.rows.push_back(c->rows[k]);
-        h.cols.push_back(c->cols[k]);
-        bool ident = true;
-        cplx s(c->ops[2 * (size_t)k * dd], c->ops[2 * (size_t)k * dd + 1]);
-        for (int i = 0; i < c->d; ++i)
-            for (int j = 0; j < c->d; ++j) {
-                cplx v(c->ops[2 * ((size_t)k * dd + i * c->d + j)], c->ops[2 * ((size_t)k * dd + i * c->d + j) + 1]);
-                h.ops.push_back(v);
-                if (i == j ? (v != s) : (v != cplx(0, 0))) ident = false;
-            }
-        h.ident.push_back(ident ? 1 : 0);
+    h.rows.assign(c->rows, c->rows + nnz);
+    h.cols.assign(c->cols, c->cols + nnz);
+    const cplx* ops = reinterpret_cast<const cplx*>(c->ops);
+    if (copy) h.ops.assign(ops, ops + (size_t)nnz * dd);
+    else h.ext = ops;
+    h.ident.resize(nnz);
+    for (int k = 0; k < nnz; ++k) {
+        // scaled identity: every entry equals its place in s I (no early exit: the loop vectorises)
+        const double* p = c->ops + 2 * (size_t)k * dd;
+        const double sr = p[0], si = p[1];
+        int bad = 0;
+        for (int i = 0; i < 2 * dd; ++i) bad += p[i] != 0.0;
+        int diag = 0;
+        for (int i = 0; i < c->d; ++i) {
+            const double* q = p + 2 * (size_t)i * (c->d + 1);
+            bad -= (q[0] != 0.0) + (q[1] != 0.0);
+            diag += (q[0] != sr) + (q[1] != si);
+        }
+        h.ident[k] = bad == 0 && diag == 0 ? 1 : 0;
     }
     return h;
 }
 
-void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
+void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, int what, int slot) {
     dc.wl = hc.wl;
     dc.wr = hc.wr;
     dc.d = hc.d;
@@ -202,7 +210,7 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
         dc.cid_real = true;
         for (int k = 0; k < nnz; ++k) {
             if (!hc.ident[k]) continue;
-            const cplx c = hc.ops[(size_t)k * d * d];
+            const cplx c = hc.op(k)[0];
             const size_t at = (size_t)hc.rows[k] * hc.wr + hc.cols[k];
             cid[2 * at] += (float)c.real();
             cid[2 * at + 1] += (float)c.imag();
@@ -211,119 +219,128 @@ void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64) {
         group(true, true, dcp, dcs, dco);
         group(false, true, drp, drs, dro);
     }
-    // spelled-out terms (FP64 mixing): the groups' entries in order, then the operator's row in order
+    // spelled-out terms: the groups' entries in order, then the operator's row in order
     std::vector<int> nzp[4];
     std::vector<unsigned> nzs[4];
     std::vector<cplx> nzc[4], cid64;
-    for (int dir = 0; dir < (fp64 ? (dc.has_cid ? 4 : 2) : 0); ++dir) {
-        const bool by_col = (dir & 1) == 0;
-        const std::vector<int>&ptr = dir == 0 ? col_ptr : dir == 1 ? row_ptr : dir == 2 ? dcp : drp,
-                              &src = dir == 0 ? col_src : dir == 1 ? row_src : dir == 2 ? dcs : drs,
-                              &op = dir == 0 ? col_op : dir == 1 ? row_op : dir == 2 ? dco : dro;
+    const int n_lists = !(what & CORE_F64) ? 0 : dc.has_cid ? 4 : 2;
+    for (int l = 0; l < n_lists; ++l) {
+        const bool by_col = (l & 1) == 0;
+        const std::vector<int>&ptr = l == 0 ? col_ptr : l == 1 ? row_ptr : l == 2 ? dcp : drp,
+                              &src = l == 0 ? col_src : l == 1 ? row_src : l == 2 ? dcs : drs,
+                              &op = l == 0 ? col_op : l == 1 ? row_op : l == 2 ? dco : dro;
         const int w_out = by_col ? hc.wr : hc.wl;
-        nzp[dir].push_back(0);
+        nzp[l].reserve((size_t)w_out * d + 1);
+        nzs[l].reserve(op.size() * (size_t)d);
+        nzc[l].reserve(op.size() * (size_t)d);
+        nzp[l].push_back(0);
+        auto add = [&](int e, int t, const cplx& c) {
+            if (c == cplx(0, 0)) return;
+            const unsigned kind = c == cplx(1, 0) ? MIX_ONE : c.imag() == 0.0 ? MIX_REAL : c.real() == 0.0 ? MIX_IMAG : MIX_CPLX;
+            nzs[l].push_back((unsigned)(src[e] * d + t) | (kind << 30));
+            nzc[l].push_back(c);
+        };
         for (int b = 0; b < w_out; ++b)
             for (int sp = 0; sp < d; ++sp) {
-                for (int e = ptr[b]; e < ptr[b + 1]; ++e)
-                    for (int t = 0; t < d; ++t) {
-                        const cplx c = hc.ops[(size_t)op[e] * d * d + sp * d + t];
-                        if (c == cplx(0, 0)) continue;
-                        const unsigned kind = c == cplx(1, 0) ? MIX_ONE : c.imag() == 0.0 ? MIX_REAL : c.real() == 0.0 ? MIX_IMAG : MIX_CPLX;
-                        nzs[dir].push_back((unsigned)(src[e] * d + t) | (kind << 30));
-                        nzc[dir].push_back(c);
-                    }
-                nzp[dir].push_back((int)nzs[dir].size());
+                for (int e = ptr[b]; e < ptr[b + 1]; ++e) {
+                    const cplx* o = hc.op(op[e]) + (size_t)sp * d;
+                    if (hc.ident[op[e]]) add(e, sp, hc.op(op[e])[0]);
+                    else
+                        for (int t = 0; t < d; ++t) add(e, t, o[t]);
+                }
+                nzp[l].push_back((int)nzs[l].size());
             }
     }
-    if (fp64 && dc.has_cid) {
+    if ((what & CORE_F64) && dc.has_cid) {
         cid64.assign((size_t)hc.wl * hc.wr, cplx(0, 0));
         for (int k = 0; k < nnz; ++k)
-            if (hc.ident[k]) cid64[(size_t)hc.rows[k] * hc.wr + hc.cols[k]] += hc.ops[(size_t)k * d * d];
+            if (hc.ident[k]) cid64[(size_t)hc.rows[k] * hc.wr + hc.cols[k]] += hc.op(k)[0];
     }
-    // one allocation holding everything
-    size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
-    auto ibytes = [](const std::vector<int>& v) { return sizeof(int) * std::max(v.size(), size_t(1)); };
-    const size_t o_cp = take(ibytes(col_ptr)), o_cs = take(ibytes(col_src)), o_co = take(ibytes(col_op)),
-                 o_rp = take(ibytes(row_ptr)), o_rs = take(ibytes(row_src)), o_ro = take(ibytes(row_op)),
-                 o_ops = take(sizeof(double2) * std::max((size_t)nnz * d * d, size_t(1))),
-                 o_id = take(std::max(nnz, 1)),
-                 o_f32 = take(sizeof(float) * 2 * std::max((size_t)nnz * d * d, size_t(1))),
-                 o_cid = take(sizeof(float) * std::max(cid.size(), size_t(1))), o_dcp = take(ibytes(dcp)),
-                 o_dcs = take(ibytes(dcs)), o_dco = take(ibytes(dco)), o_drp = take(ibytes(drp)),
-                 o_drs = take(ibytes(drs)), o_dro = take(ibytes(dro));
-    const size_t o_cid64 = take(sizeof(double2) * std::max(cid64.size(), size_t(1)));
-    size_t o_nzp[4], o_nzs[4], o_nzc[4];
-    for (int i = 0; i < 4; ++i) {
-        o_nzp[i] = take(ibytes(nzp[i]));
-        o_nzs[i] = take(sizeof(unsigned) * std::max(nzs[i].size(), size_t(1)));
-        o_nzc[i] = take(sizeof(double2) * std::max(nzc[i].size(), size_t(1)));
-    }
-    std::vector<unsigned char> blob(off, 0);
-    auto put = [&](size_t o, const void* p, size_t bytes) {
-        if (bytes) std::memcpy(&blob[o], p, bytes);
-    };
-    auto puti = [&](size_t o, const std::vector<int>& v) { put(o, v.data(), sizeof(int) * v.size()); };
-    puti(o_cp, col_ptr);
-    puti(o_cs, col_src);
-    puti(o_co, col_op);
-    puti(o_rp, row_ptr);
-    puti(o_rs, row_src);
-    puti(o_ro, row_op);
-    if (nnz) {
-        put(o_ops, hc.ops.data(), sizeof(double2) * (size_t)nnz * d * d);
-        put(o_id, hc.ident.data(), nnz);
-        std::vector<float> f32((size_t)nnz * d * d * 2);
-        for (size_t i = 0; i < (size_t)nnz * d * d; ++i) {
-            f32[2 * i] = (float)hc.ops[i].real();
-            f32[2 * i + 1] = (float)hc.ops[i].imag();
+    // FP32 operators, one scalar for a scaled identity
+    const int n_mix = !(what & CORE_F32) ? 0 : dc.has_cid ? 3 : 2;
+    std::vector<float> f32;
+    std::vector<int> code(n_mix ? nnz : 0);
+    for (int k = 0; k < (n_mix ? nnz : 0); ++k) {
+        code[k] = (int)f32.size() + (hc.ident[k] ? 1 : 0);  // (floats so far = 2 x complex offset)
+        const cplx* o = hc.op(k);
+        for (int i = 0; i < (hc.ident[k] ? 1 : d * d); ++i) {
+            f32.push_back((float)o[i].real());
+            f32.push_back((float)o[i].imag());
         }
-        put(o_f32, f32.data(), sizeof(float) * f32.size());
     }
+    const std::vector<int>* mix[3][2] = {{&col_ptr, &col_src}, {&row_ptr, &row_src}, {&dcp, &dcs}};
+    std::vector<int> mix_op[3];
+    for (int l = 0; l < n_mix; ++l) {
+        const std::vector<int>& op = l == 0 ? col_op : l == 1 ? row_op : dco;
+        mix_op[l].resize(op.size());
+        for (size_t i = 0; i < op.size(); ++i) mix_op[l][i] = code[op[i]];
+    }
+    // one block holding everything
+    size_t off = 0;
+    auto take = [&](size_t bytes) { size_t o = off; off += (std::max(bytes, size_t(1)) + 255) & ~size_t(255); return o; };
+    const size_t o_cid = take(sizeof(float) * cid.size()), o_cid64 = take(sizeof(double2) * cid64.size());
+    const size_t o_f32 = take(sizeof(float) * f32.size());
+    size_t o_p[4], o_s[4], o_c[4], o_m[3][3];
+    for (int l = 0; l < n_mix; ++l) {
+        o_m[l][0] = take(sizeof(int) * mix[l][0]->size());
+        o_m[l][1] = take(sizeof(int) * mix[l][1]->size());
+        o_m[l][2] = take(sizeof(int) * mix_op[l].size());
+    }
+    for (int l = 0; l < n_lists; ++l) {
+        o_p[l] = take(sizeof(int) * nzp[l].size());
+        o_s[l] = take(sizeof(unsigned) * nzs[l].size());
+        o_c[l] = take(sizeof(double2) * nzc[l].size());
+    }
+    const bool staged = slot >= 0 && off <= Ctx::STAGE * sizeof(double);
+    std::vector<unsigned char> owned;
+    unsigned char* blob;
+    if (staged) {
+        blob = (unsigned char*)(ctx.pinned + Ctx::PINNED + (slot == WS_CORE_B ? Ctx::STAGE : 0));
+    } else {
+        owned.resize(off);
+        blob = owned.data();
+    }
+    auto put = [&](size_t o, const void* p, size_t bytes) {
+        if (bytes) std::memcpy(blob + o, p, bytes);
+    };
     put(o_cid, cid.data(), sizeof(float) * cid.size());
-    puti(o_dcp, dcp);
-    puti(o_dcs, dcs);
-    puti(o_dco, dco);
-    puti(o_drp, drp);
-    puti(o_drs, drs);
-    puti(o_dro, dro);
     put(o_cid64, cid64.data(), sizeof(double2) * cid64.size());
-    for (int i = 0; i < 4; ++i) {
-        puti(o_nzp[i], nzp[i]);
-        put(o_nzs[i], nzs[i].data(), sizeof(unsigned) * nzs[i].size());
-        put(o_nzc[i], nzc[i].data(), sizeof(double2) * nzc[i].size());
+    for (int l = 0; l < n_lists; ++l) {
+        put(o_p[l], nzp[l].data(), sizeof(int) * nzp[l].size());
+        put(o_s[l], nzs[l].data(), sizeof(unsigned) * nzs[l].size());
+        put(o_c[l], nzc[l].data(), sizeof(double2) * nzc[l].size());
     }
-    DevBuf b;
-    b.bytes = off;
-    b.p = ctx.dalloc(off);
-    VTN_CUDA_TRY(cudaMemcpyAsync(b.p, blob.data(), off, cudaMemcpyHostToDevice, ctx.stream));
-    ctx.sync();  // blob is a stack-local host buffer
-    unsigned char* base = (unsigned char*)b.p;
-    dc.col_ptr = (int*)(base + o_cp);
-    dc.col_src = (int*)(base + o_cs);
-    dc.col_op = (int*)(base + o_co);
-    dc.row_ptr = (int*)(base + o_rp);
-    dc.row_src = (int*)(base + o_rs);
-    dc.row_op = (int*)(base + o_ro);
-    dc.ops = (double2*)(base + o_ops);
-    dc.ident = base + o_id;
-    dc.ops_f32 = (float2*)(base + o_f32);
-    if (fp64 && dc.has_cid) dc.cid64 = (double2*)(base + o_cid64);
-    for (int i = 0; i < (fp64 ? (dc.has_cid ? 4 : 2) : 0); ++i) {
-        dc.nz_ptr[i] = (int*)(base + o_nzp[i]);
-        dc.nz_src[i] = (unsigned*)(base + o_nzs[i]);
-        dc.nz_c[i] = (double2*)(base + o_nzc[i]);
+    put(o_f32, f32.data(), sizeof(float) * f32.size());
+    for (int l = 0; l < n_mix; ++l) {
+        put(o_m[l][0], mix[l][0]->data(), sizeof(int) * mix[l][0]->size());
+        put(o_m[l][1], mix[l][1]->data(), sizeof(int) * mix[l][1]->size());
+        put(o_m[l][2], mix_op[l].data(), sizeof(int) * mix_op[l].size());
     }
-    if (dc.has_cid) {
-        dc.cid = (float2*)(base + o_cid);
-        dc.dcol_ptr = (int*)(base + o_dcp);
-        dc.dcol_src = (int*)(base + o_dcs);
-        dc.dcol_op = (int*)(base + o_dco);
-        dc.drow_ptr = (int*)(base + o_drp);
-        dc.drow_src = (int*)(base + o_drs);
-        dc.drow_op = (int*)(base + o_dro);
+    unsigned char* base;
+    if (slot >= 0) {
+        base = (unsigned char*)ctx.workspace(slot, off);
+    } else {
+        DevBuf b;
+        b.bytes = off;
+        b.p = ctx.dalloc(off);
+        base = (unsigned char*)b.p;
+        dc.bufs.push_back(b);
     }
-    dc.bufs.push_back(b);
+    VTN_CUDA_TRY(cudaMemcpyAsync(base, blob, off, cudaMemcpyHostToDevice, ctx.stream));
+    if (!staged) ctx.sync();  // blob is a local host buffer
+    if (dc.has_cid) dc.cid = (float2*)(base + o_cid);
+    if (!cid64.empty()) dc.cid64 = (double2*)(base + o_cid64);
+    for (int l = 0; l < n_lists; ++l) {
+        dc.nz_ptr[l] = (int*)(base + o_p[l]);
+        dc.nz_src[l] = (unsigned*)(base + o_s[l]);
+        dc.nz_c[l] = (double2*)(base + o_c[l]);
+    }
+    if (n_mix) dc.ops_f32 = (float2*)(base + o_f32);
+    for (int l = 0; l < n_mix; ++l) {
+        dc.mix_ptr[l] = (int*)(base + o_m[l][0]);
+        dc.mix_src[l] = (int*)(base + o_m[l][1]);
+        dc.mix_op[l] = (int*)(base + o_m[l][2]);
+    }
 }
 
 void free_core(Ctx& ctx, DevCore& dc) {

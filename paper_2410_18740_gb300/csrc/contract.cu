@@ -73,13 +73,13 @@ __global__ void __launch_bounds__(256) mix_kernel(int P, int d, int Q, const int
 // block; their inputs come from L2 (each is used by a few outputs).
 // ACC: added to the output instead of replacing it (outputs without a term keep what they hold).
 template <bool ACC>
-__global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int Q, const int* __restrict__ ptr,
+__global__ void __launch_bounds__(256) mix_terms_kernel(long long PQ, int d, int Q, int n_out, const int* __restrict__ ptr,
                                                         const unsigned* __restrict__ src,
                                                         const double2* __restrict__ coef,
                                                         const double2* __restrict__ in, double2* __restrict__ out) {
     const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
-    const int o = blockIdx.y;
-    if (t >= PQ) return;
+    const int o = blockIdx.y + blockIdx.z * 65535;
+    if (t >= PQ || o >= n_out) return;
     const long long p = t / Q, q = t % Q;
     const long long blk = PQ * d, at = p * d * Q + q;
     const int e0 = ptr[o], e1 = ptr[o + 1];
@@ -124,8 +124,9 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
     double fl = 8.0 * PQ * ((double)core.n_ident * d + (double)core.n_dense * d * d);
     int t = ctx.tbegin(TC_MIX, fl);
     const int dir = by_col ? 0 : 1;
-    const bool terms = core.nz_ptr[dir] != nullptr && (long long)w_out * d <= 65535;
-    const dim3 tgrid((unsigned)((PQ + 255) / 256), w_out * d);
+    const bool terms = core.nz_c[dir] != nullptr;
+    VTN_REQUIRE(terms || core.ops != nullptr, "FP64 mixing needs the core's FP64 operators");
+    const dim3 tgrid((unsigned)((PQ + 255) / 256), (unsigned)std::min(w_out * d, 65535), (w_out * d + 65534) / 65535);
     const long long E = PQ * d;
     // A collapse core couples all channels to all: its scaled identities are a channel product
     // out[b][e] = sum_a C[a][b] in[a][e], which the FP64 pipe does at two operations a coupling and element (0.49e12
@@ -140,10 +141,10 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
         g.opB = by_col ? OP_N : OP_T; g.B = core.cid64; g.ldb = core.wr;
         g.C = out; g.ldc = 1; g.sC_n = E;
         oz_gemm(ctx, g, 1, nullptr);
-        mix_terms_kernel<true><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, core.nz_ptr[2 + dir], core.nz_src[2 + dir],
+        mix_terms_kernel<true><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, w_out * d, core.nz_ptr[2 + dir], core.nz_src[2 + dir],
                                                               core.nz_c[2 + dir], in, out);
     } else if (terms)
-        mix_terms_kernel<false><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, core.nz_ptr[dir], core.nz_src[dir],
+        mix_terms_kernel<false><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, w_out * d, core.nz_ptr[dir], core.nz_src[dir],
                                                                core.nz_c[dir], in, out);
     else if (d <= 4)
         mix_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, ptr, src, opi, core.ops, core.ident, in, out);

@@ -63,7 +63,7 @@ Expanded expand_core(const HostCore& h, int max_basis) {
     std::vector<std::vector<cplx>> Q;  // orthonormal, orthogonal to I: the basis elements 1..r-1
     std::vector<cplx> res(dd);
     for (int k = 0; k < h.nnz(); ++k) {
-        const cplx* op = &h.ops[(size_t)k * dd];
+        const cplx* op = h.op(k);
         const int a = h.rows[k], b = h.cols[k];
         if (h.ident[k]) {
             if (op[0] != 0.0) e.coef[0].push_back({a, b, op[0]});
@@ -183,16 +183,18 @@ bool bond_terms_host(const HostCore& Wi, const HostCore& Wj, int& n_id, std::vec
             const int nr = (int)B.rows.size(), nc = (int)B.cols.size();
             const std::vector<cplx>& k = B.k;
             std::vector<int> nzr, nzc;  // positions in the block
+            std::vector<double> cmax(nc, 0.0);
             for (int a = 0; a < nr; ++a) {
                 double m = 0.0;
-                for (int c = 0; c < nc; ++c) m = std::max(m, std::norm(k[(size_t)a * nc + c]));
+                for (int c = 0; c < nc; ++c) {
+                    const double v = std::norm(k[(size_t)a * nc + c]);
+                    m = v > m ? v : m;
+                    cmax[c] = v > cmax[c] ? v : cmax[c];
+                }
                 if (m > tol2) nzr.push_back(a);
             }
-            for (int c = 0; c < nc; ++c) {
-                double m = 0.0;
-                for (int a = 0; a < nr; ++a) m = std::max(m, std::norm(k[(size_t)a * nc + c]));
-                if (m > tol2) nzc.push_back(c);
-            }
+            for (int c = 0; c < nc; ++c)
+                if (cmax[c] > tol2) nzc.push_back(c);
             if (nzr.empty()) continue;
             const size_t trivial = std::min(nzr.size(), nzc.size());
             std::vector<HostTerm> got;

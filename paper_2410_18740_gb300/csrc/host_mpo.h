@@ -15,6 +15,8 @@ struct HostCore {
     int wl = 0, wr = 0, d = 0;
     std::vector<int> rows, cols;
     std::vector<cplx> ops;          // nnz * d * d, ops[k][s'][s]
+    const cplx* ext = nullptr;      // when set: the same array in the caller's memory (ops is empty)
+    const cplx* op(int k) const { return (ext ? ext : ops.data()) + (size_t)k * d * d; }
     std::vector<unsigned char> ident;  // 1 if ops[k] = s * I (scalar in ops[k][0][0])
     int nnz() const { return (int)rows.size(); }
 };

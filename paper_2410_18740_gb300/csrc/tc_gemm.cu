@@ -380,6 +380,7 @@ void tc_gemm_bf16(Ctx& ctx, const TcGemmArgs& a, int timing_class, double useful
     int t1 = timing_class >= 0 ? ctx.tbegin(timing_class, useful_flops) : -1;
     tc_gemm_kernel<<<n_cta, TC_THREADS, SMEM_BYTES, ctx.stream>>>(ma, mb, p);
     ctx.count_launch();
+    ctx.dstatus_due = true;
     ctx.check_launch("tc_gemm_kernel");
     if (splits > 1) {
         const long long cnt = (long long)a.M * a.N;

@@ -190,7 +190,9 @@ __global__ void zero_pad_kernel(__nv_bfloat16* out, long long ldo, int rows, int
 
 // out[b][p][s'][q] = sum_e op_e[s'][s] in[src_e][p][s][q] in FP32 (ops rounded to float).
 // All threads of a CTA share the output channel b, so the channel's operators are staged
-// in shared memory (as float2) in chunks, instead of being re-read by every thread.
+// in shared memory (as float2) in chunks, instead of being re-read by every thread.  Memory bound (each input read
+// once per operator for all d levels: 388 us for the 1.4 GB of the large workload's environment update at chi = 384;
+// one output level per thread from spelled-out terms, as in FP64, re-reads them and took twice as long).
 constexpr int MIX_SH = 4096;  // float2 operator entries per chunk (32 KiB)
 
 // element (channel c, p, s, q) of the mixing input sits at c * cs + p * ps + s * ss + q
@@ -201,9 +203,7 @@ struct MixIn {
 template <int DM>
 __global__ void __launch_bounds__(256) mix_f32_kernel(int P, int d, int Q, MixIn st, const int* __restrict__ ptr,
                                                       const int* __restrict__ src, const int* __restrict__ opi,
-                                                      const float2* __restrict__ ops,
-                                                      const unsigned char* __restrict__ ident,
-                                                      const float2* __restrict__ in, float2* __restrict__ out,
+                                                      const float2* __restrict__ ops, const float2* __restrict__ in, float2* __restrict__ out,
                                                       int accumulate) {
     __shared__ float2 op_sh[MIX_SH];
     __shared__ int src_sh[MIX_SH / 4];
@@ -226,11 +226,12 @@ __global__ void __launch_bounds__(256) mix_f32_kernel(int P, int d, int Q, MixIn
         __syncthreads();
         for (int i = threadIdx.x; i < ne * dd; i += blockDim.x) {
             const int e = i / dd, j = i - e * dd;
-            op_sh[i] = ops[(long long)opi[e0 + e] * dd + j];
+            const int k = opi[e0 + e];  // offset of the operator * 2 + (1: a scaled identity, its scalar only)
+            if (j == 0 || !(k & 1)) op_sh[i] = ops[(k >> 1) + j];
         }
         for (int e = threadIdx.x; e < ne; e += blockDim.x) {
             src_sh[e] = src[e0 + e];
-            id_sh[e] = ident[opi[e0 + e]];
+            id_sh[e] = opi[e0 + e] & 1;
         }
         __syncthreads();
         if (!active) continue;
@@ -526,10 +527,7 @@ void mix_apply_f32(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, con
     const long long PQ = (long long)P * Q;
     if (PQ == 0) return;
     VTN_REQUIRE(w_out <= 65535, "too many MPO channels");
-    dim3 grid((unsigned)((PQ + 255) / 256), w_out);
-    const int* ptr = by_col ? core.col_ptr : core.row_ptr;  // reassigned to the dense-only lists of a collapse core
-    const int* src = by_col ? core.col_src : core.row_src;
-    const int* opi = by_col ? core.col_op : core.row_op;
+    int list = by_col ? 0 : 1;
     double fl = 8.0 * PQ * ((double)core.n_ident * d + (double)core.n_dense * d * d);
     MixIn st;
     st.cs = PQ * d;
@@ -541,7 +539,7 @@ void mix_apply_f32(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, con
         st.ss = in_strides[2];
     }
     int t = ctx.tbegin(TC_MIX, fl);
-    VTN_REQUIRE(core.ops_f32 != nullptr, "FP32 mixing needs the core's FP32 operators");
+    VTN_REQUIRE(core.mix_ptr[list] != nullptr, "FP32 mixing needs the core's FP32 operators");
     const int w_in = by_col ? core.wl : core.wr;
     const long long E = PQ * d;
     bool accumulate = false;
@@ -559,21 +557,18 @@ void mix_apply_f32(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, con
             const unsigned grid_c = (unsigned)std::min<long long>(tiles, std::max(ctx.num_sms, 1));
             launch_mix_cid(ctx, JB, EI, core.cid_real, (int)bytes, grid_c, w_in, w_out, E, core.cid, w_out, in, out);
             ctx.check_launch("mix_cid_kernel");
-            ptr = core.dcol_ptr;
-            src = core.dcol_src;
-            opi = core.dcol_op;
+            list = 2;  // the entries that are no identities
             accumulate = true;
         }
     }
+    const dim3 grid((unsigned)((PQ + 255) / 256), w_out);
+    const int *ptr = core.mix_ptr[list], *src = core.mix_src[list], *opi = core.mix_op[list];
     if (d <= 4)
-        mix_f32_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, core.ident, in, out,
-                                                        accumulate ? 1 : 0);
+        mix_f32_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, in, out, accumulate ? 1 : 0);
     else if (d <= 8)
-        mix_f32_kernel<8><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, core.ident, in, out,
-                                                        accumulate ? 1 : 0);
+        mix_f32_kernel<8><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, in, out, accumulate ? 1 : 0);
     else
-        mix_f32_kernel<16><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, core.ident, in, out,
-                                                         accumulate ? 1 : 0);
+        mix_f32_kernel<16><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, in, out, accumulate ? 1 : 0);
     ctx.count_launch();
     ctx.check_launch("mix_f32_kernel");
     ctx.tend(t);

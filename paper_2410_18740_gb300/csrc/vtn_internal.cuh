@@ -75,10 +75,7 @@ struct DevCore {
     int* row_ptr = nullptr;   // [wl + 1]
     int* row_src = nullptr;   // [nnz]
     int* row_op = nullptr;    // [nnz]
-    double2* ops = nullptr;   // [nnz][d][d]
-    float2* ops_f32 = nullptr;  // the same operators rounded to FP32 once at upload (the FP32 mixing
-                                // of the split-precision mode reads these: a double -> float
-                                // conversion runs on GB300's narrow FP64 pipe)
+    double2* ops = nullptr;   // [nnz][d][d] (with ident: only for cores without spelled-out terms)
     unsigned char* ident = nullptr;  // [nnz]
     double flops_ident = 0, flops_dense = 0;  // counts for the flop model
     int n_ident = 0, n_dense = 0;
@@ -87,8 +84,6 @@ struct DevCore {
     // remaining (dense) entries by column and by row
     bool has_cid = false, cid_real = false;
     float2* cid = nullptr;
-    int *dcol_ptr = nullptr, *dcol_src = nullptr, *dcol_op = nullptr;
-    int *drow_ptr = nullptr, *drow_src = nullptr, *drow_op = nullptr;
     // the same entries spelled out per output element (channel, level) in the order of the lists above, zero
     // coefficients dropped: term t of output o adds nz_c[t] * in[nz_src[t]], nz_src = channel * d + level with
     // the coefficient's kind (MixTerm) in the two topmost bits; [0] by column, [1] by row
@@ -96,6 +91,13 @@ struct DevCore {
     int* nz_ptr[4] = {};       // [w_out * d + 1]
     unsigned* nz_src[4] = {};
     double2* nz_c[4] = {};
+    // FP32 mixing: entries grouped by output channel ([0] by column, [1] by row, [2] by column without the scaled
+    // identities of a collapse core); mix_op = offset into ops_f32 * 2 + 1 for a scaled identity (its scalar), + 0 for
+    // a d x d operator; rounded to FP32 once here (a conversion on the device would run on the narrow FP64 pipe)
+    int* mix_ptr[3] = {};
+    int* mix_src[3] = {};
+    int* mix_op[3] = {};
+    float2* ops_f32 = nullptr;
     double2* cid64 = nullptr;  // C[a][b] in FP64
     std::vector<DevBuf> bufs;
 };
@@ -128,7 +130,8 @@ struct Ctx {
     std::vector<cudaEvent_t> event_pool;
     // named workspace slots
     std::vector<DevBuf> ws;
-    double* pinned = nullptr;  // pinned host scratch (4096 doubles)
+    double* pinned = nullptr;  // pinned host scratch (4096 doubles), then the staging of two cores
+    static constexpr size_t PINNED = 4096, STAGE = 8192;  // doubles
     double* defer_buf = nullptr;  // pinned staging of results read back once per sweep
     size_t defer_cap = 0;         // doubles
     long long host_syncs = 0;     // stream synchronisations made by sync()
@@ -163,10 +166,14 @@ enum WsSlot {
 };
 
 // ------------------------------------------------------------------ cores
-// fp64 = false leaves out the spelled-out terms of the FP64 mixing
-void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, bool fp64 = true);
+// what: which coefficients go up (FP64 mixing, FP32 mixing of the split-precision mode).  slot < 0: the core owns its
+// device memory; else it lies in that workspace slot, staged through the context's pinned memory when
+// it is small (nothing is allocated or waited for)
+enum CoreWhat { CORE_F64 = 1, CORE_F32 = 2, CORE_BOTH = 3 };
+void upload_core(Ctx& ctx, const HostCore& hc, DevCore& dc, int what = CORE_BOTH, int slot = -1);
 void free_core(Ctx& ctx, DevCore& dc);
-HostCore core_from_abi(const vtn_core* c);
+// copy = false: the operators stay in the caller's array (valid for the call)
+HostCore core_from_abi(const vtn_core* c, bool copy = true);
 
 // ------------------------------------------------------------------ GEMM (complex FP64)
 enum Op { OP_N = 0, OP_C = 1, OP_T = 2 };  // op(X) = X, X^dag (conjugate transpose) or (oz_gemm only) X^T
