@@ -44,8 +44,8 @@ __device__ __forceinline__ double rsqrt_newton(double x) {
 // One CTA, b <= NB.  flag[0] = 1 on a pivot that is not positive.
 // FP64-issue bound (about 2 x 170 warp-wide element updates of 6 instructions), so the elements left of each step are
 // dealt out densely to the lanes: L D L^dag with unit L, the update of column j and the same row operations on
-// the growing inverse in one pass with one barrier, the square roots taken once at the end.  168 -> 59 us
-// for a block of 32 (one column per step with three barriers and the inverse as 32 serial dot products before).
+// the growing inverse in one pass with one barrier, the square roots taken once at the end, the next pivot while the others still work.  168 -> 50 us
+// for a block of 32 (three barriers a column and the inverse as 32 serial dot products before).
 __global__ void __launch_bounds__(256) potrf_block(double2* __restrict__ G, int b, long long ld,
                                                   double2* __restrict__ Linv, int* __restrict__ flag) {
     __shared__ double2 S[NB][NB + 1];
@@ -79,27 +79,37 @@ __global__ void __launch_bounds__(256) potrf_block(double2* __restrict__ G, int 
         }
     }
     __shared__ int row_exp[NB];
-    __shared__ double piv[NB];
+    __shared__ double piv[NB], pinv[NB];
     __syncthreads();
     if (tid < NB) row_exp[tid] = (int)D[tid];
-    for (int j = 0; j < b; ++j) {
-        double d = S[j][j].x;
+    // (row, column) of the t-th element of a lower triangle counted by rows: the same for every size
+    __shared__ unsigned char ti[NB * (NB + 1) / 2], tl[NB * (NB + 1) / 2];
+    for (int t = tid; t < NB * NB; t += 256) {
+        const int i = t / NB, l = t - (t / NB) * NB;
+        if (l <= i) {
+            ti[i * (i + 1) / 2 + l] = (unsigned char)i;
+            tl[i * (i + 1) / 2 + l] = (unsigned char)l;
+        }
+    }
+    // pivot j and its reciprocal; the thread that updates S[j + 1][j + 1] takes the next one while the others work
+    auto take_pivot = [&](int j, double d) {
         if (!(d > 1e-30)) {  // pivots are relative to their row's norm; the caller's fallback replaces the result
-            if (tid == 0) bad = 1;
+            bad = 1;
             d = 1.0;
         }
-        if (tid == 0) piv[j] = d;
-        const double inv = recip_newton(d);
+        piv[j] = d;
+        pinv[j] = recip_newton(d);
+    };
+    if (tid == 0) take_pivot(0, S[0][0].x);
+    __syncthreads();
+    for (int j = 0; j < b; ++j) {
+        const double inv = pinv[j];
         const int r = b - 1 - j;
         const int n_s = r * (r + 1) / 2, n_x = r * (j + 1);
+        const float wi = 1.0f / (float)(j + 1);
         for (int t = tid; t < n_s + n_x; t += 256) {
-            int i, l;
             if (t < n_s) {  // S[i][l] -= S[i][j] conj(S[l][j]) / d, j < l <= i
-                i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-                while (i * (i + 1) / 2 > t) --i;
-                while ((i + 1) * (i + 2) / 2 <= t) ++i;
-                l = t - i * (i + 1) / 2 + j + 1;
-                i += j + 1;
+                const int i = ti[t] + j + 1, l = tl[t] + j + 1;
                 double2 a = S[i][j];
                 const double2 c = S[l][j];
                 a.x *= inv;
@@ -108,10 +118,13 @@ __global__ void __launch_bounds__(256) potrf_block(double2* __restrict__ G, int 
                 s.x = fma(-a.x, c.x, fma(-a.y, c.y, s.x));
                 s.y = fma(-a.y, c.x, fma(a.x, c.y, s.y));
                 S[i][l] = s;
+                if (t == 0) take_pivot(j + 1, s.x);
             } else {  // X[i][l] -= S[i][j] / d X[j][l], i > j, l <= j
                 const int u = t - n_s;
-                i = j + 1 + u / (j + 1);
-                l = u % (j + 1);
+                int q = (int)((float)u * wi);
+                q += (q + 1) * (j + 1) <= u;
+                q -= q * (j + 1) > u;
+                const int i = j + 1 + q, l = u - q * (j + 1);
                 double2 a = S[i][j];
                 const double2 x = X[j][l];
                 a.x *= inv;
@@ -191,6 +204,7 @@ void cholesky_blocked(Ctx& ctx, double2* G, int m, double2* Linv_all, double2* t
         u.C = L21 + b; u.ldc = m;
         u.accumulate = true;
         u.negate = true;
+        u.herm_lower = true;  // (the strict upper tiles are never read)
         gemm_c64(ctx, u);
     }
 }

@@ -159,7 +159,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     p.herm_lower = g.herm_lower ? 1 : 0;
     p.negate = g.negate ? 1 : 0;
     VTN_REQUIRE(g.sC_n == 1 || (g.prepA != nullptr && g.ldc == 1 && !g.herm_lower), "column strides need a prepared operand");
-    VTN_REQUIRE(!g.herm_lower || (g.M == g.N && !g.accumulate), "Hermitian GEMM needs a square, non-accumulating C");
+    VTN_REQUIRE(!g.herm_lower || g.M == g.N, "Hermitian GEMM needs a square C");
     p.batch = g.batch;
     const long long gx = (g.N + BT - 1) / BT, gy = (g.M + BT - 1) / BT;
     VTN_REQUIRE(gy <= 4 * 65535LL, "gemm M too large");
