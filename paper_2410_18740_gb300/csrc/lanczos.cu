@@ -200,15 +200,42 @@ __device__ int sturm_count(const double* a, const double* b, int m, double x, do
     return cnt;
 }
 
+// Whether an eigenvalue lies below x, from the leading minors (p_i = (a_i - x) p_{i-1} - b_{i-1}^2 p_{i-2}; scaled
+// by s = 1 / |T|): two dependent operations a step where the quotients of sturm_count take a division.  Its
+// rounding moves the answer by a few ulps of |T| like theirs, so it serves while the section's points are far
+// apart.
+__device__ bool below_minors(const double* a, const double* b, int m, double x, double s) {
+    double p0 = 1.0, p1 = (a[0] - x) * s;
+    bool neg = p1 <= 0.0;
+    for (int i = 1; i < m; ++i) {
+        const double bs = b[i - 1] * s;
+        const double p2 = fma((a[i] - x) * s, p1, -(bs * bs) * p0);
+        neg = neg || p2 <= 0.0;  // the first sign change: p_{i-1} was positive
+        p0 = p1;
+        p1 = p2;
+    }
+    return neg;
+}
+
 // One warp.  Lowest eigenpair of the m x m symmetric tridiagonal (alpha, beta), Ritz
-// residual beta_j |y_{m-1}|, and the decision for the host.
-__global__ void ritz_kernel(LzState* st, int m, double tol, double breakdown, int last) {
-    __shared__ double lo_s, hi_s;
-    const int lane = threadIdx.x;
-    if (st->stop) return;  // an earlier iteration ended the recursion (device-driven loop)
-    const double* a = st->alpha;
-    const double* b = st->beta;
+// residual beta_j |y_{m-1}|, and the decision for the host.  A serial chain of divisions (about 0.4 us each),
+// so the matrix and the factors are kept in shared memory.
+struct RitzScratch {
+    double a[KMAX_DEV], b[KMAX_DEV], dd[KMAX_DEV], du[KMAX_DEV], du2[KMAX_DEV], dl[KMAX_DEV], x[KMAX_DEV];
+    int piv[KMAX_DEV];
+    double lo, hi;
+};
+
+__device__ void ritz_step(LzState* st, int m, double tol, double breakdown, int last, RitzScratch& sc) {
+    const int lane = threadIdx.x & 31;
+    double &lo_s = sc.lo, &hi_s = sc.hi;
+    double *a = sc.a, *b = sc.b;
     if (lane == 0) st->alpha[m - 1] = st->c1[m - 1].x;
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) {
+        a[i] = st->alpha[i];
+        b[i] = st->beta[i];
+    }
     __syncwarp();
     double gl = 1e308, gu = -1e308, tnrm = 0.0;
     for (int i = 0; i < m; ++i) {
@@ -219,6 +246,7 @@ __global__ void ritz_kernel(LzState* st, int m, double tol, double breakdown, in
     }
     const double eps = 2.220446049250313e-16;
     const double pivmin = fmax(1e-300, eps * eps * fmax(tnrm, 1e-300));
+    const double inv_tnrm = 1.0 / fmax(tnrm, 1e-300);
     if (lane == 0) {
         lo_s = gl - eps * tnrm - pivmin;
         hi_s = gu + eps * tnrm + pivmin;
@@ -230,8 +258,8 @@ __global__ void ritz_kernel(LzState* st, int m, double tol, double breakdown, in
         if (hi - lo <= 2.0 * eps * fmax(fabs(lo), fabs(hi)) + 4.0 * pivmin) break;
         const double step = (hi - lo) / 33.0;
         const double x = lo + step * (lane + 1);
-        const int c = sturm_count(a, b, m, x, pivmin);
-        const unsigned ballot = __ballot_sync(0xffffffffu, c >= 1);
+        const bool below = step > 1e-7 * tnrm ? below_minors(a, b, m, x, inv_tnrm) : sturm_count(a, b, m, x, pivmin) >= 1;
+        const unsigned ballot = __ballot_sync(0xffffffffu, below);
         __syncwarp();
         if (lane == 0) {
             if (ballot == 0) {
@@ -247,8 +275,8 @@ __global__ void ritz_kernel(LzState* st, int m, double tol, double breakdown, in
     if (lane != 0) return;
     const double th = 0.5 * (lo_s + hi_s);
     // inverse iteration with the pivoted LU of (T - th I)
-    double dd[KMAX_DEV], du[KMAX_DEV], du2[KMAX_DEV], dl[KMAX_DEV], x[KMAX_DEV];
-    int piv[KMAX_DEV];
+    double *dd = sc.dd, *du = sc.du, *du2 = sc.du2, *dl = sc.dl, *x = sc.x;
+    int* piv = sc.piv;
     const double tiny = eps * fmax(tnrm, 1e-300);
     for (int i = 0; i < m; ++i) {
         dd[i] = a[i] - th;
@@ -312,6 +340,117 @@ __global__ void ritz_kernel(LzState* st, int m, double tol, double breakdown, in
     else {
         st->stop = 1;
         st->m_stop = m;
+    }
+}
+
+__global__ void __launch_bounds__(32) ritz_kernel(LzState* st, int m, double tol, double breakdown, int last) {
+    __shared__ RitzScratch sc;
+    if (st->stop) return;  // an earlier iteration ended the recursion (device-driven loop)
+    ritz_step(st, m, tol, breakdown, last, sc);
+}
+
+// The vector work of one Krylov step in one CTA, for vectors of up to SMALL_BLOCKS * 4 * RB elements: the two
+// orthogonalisation passes, the norm, the Ritz pair and the next vector, ten or more launches of about 3 us otherwise
+// (the smallest workload spends most of a solve in them).  The CTA stands for the `nblk` blocks of the separate
+// kernels: the same elements per thread, the same butterflies and the same order of partial sums, so the results are
+// the same bit for bit.  Up to 2048 elements: at 4096 one SM's FP64 pipe makes it 190 us against about 150 us of separate
+// launches, at 1440 it is 89 against 110, at 256 45 against 75.
+constexpr int SMALL_BLOCKS = 2;
+
+// sum of up to SMALL_BLOCKS partials in the order of a warp's butterfly
+__device__ __forceinline__ double small_tree(const double* p, int stride, int nblk) {
+    return p[0] + (nblk > 1 ? p[stride] : 0.0);
+}
+
+__global__ void __launch_bounds__(SMALL_BLOCKS * RB) lanczos_small_kernel(double2* __restrict__ V, int n, int j,
+                                                                          double2* __restrict__ w, LzState* st, double tol,
+                                                                          double breakdown, int last, int nblk) {
+    __shared__ double sh[SMALL_BLOCKS][RB / 32][32];
+    __shared__ double2 part[SMALL_BLOCKS][KMAX_DEV];
+    __shared__ double2 cs[KMAX_DEV];
+    __shared__ double npart[SMALL_BLOCKS];
+    __shared__ double beta2_sh;
+    __shared__ int flag_sh;
+    __shared__ RitzScratch sc;
+    if (st->stop) return;
+    const int blk = threadIdx.x / RB, t = threadIdx.x % RB, lane = t & 31, wid = t >> 5, nv = j + 1;
+    const int e0 = blk * RB + t, step = nblk * RB;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int g0 = 0; g0 < nv; g0 += DOT_GROUP) {
+            const int cnt = min(DOT_GROUP, nv - g0);
+            double v[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = 0.0;
+            for (int e = e0; e < n; e += step) {
+                const double2 we = w[e];
+#pragma unroll
+                for (int i = 0; i < DOT_GROUP; ++i) {
+                    if (i < cnt) {
+                        const double2 a = V[(long long)(g0 + i) * n + e];
+                        v[2 * i] = fma(a.x, we.x, fma(a.y, we.y, v[2 * i]));
+                        v[2 * i + 1] = fma(a.x, we.y, fma(-a.y, we.x, v[2 * i + 1]));
+                    }
+                }
+            }
+            sh[blk][wid][lane] = warp_reduce32(v);
+            __syncthreads();
+            if (wid == 0) {
+                double r = 0.0;
+#pragma unroll
+                for (int w2 = 0; w2 < RB / 32; ++w2) r += sh[blk][w2][lane];
+                const double im = __shfl_down_sync(0xffffffffu, r, 1);
+                if ((lane & 1) == 0 && lane / 2 < cnt) part[blk][g0 + lane / 2] = make_double2(r, im);
+            }
+            __syncthreads();
+        }
+        if ((int)threadIdx.x < nv) {
+            const int i = threadIdx.x;
+            const double2 c = make_double2(small_tree(&part[0][i].x, 2 * KMAX_DEV, nblk), small_tree(&part[0][i].y, 2 * KMAX_DEV, nblk));
+            cs[i] = c;
+            (pass == 0 ? st->c1 : st->c2)[i] = c;
+        }
+        __syncthreads();
+        for (int e = e0; e < n; e += step) {
+            double2 acc = w[e];
+            for (int i = 0; i < nv; ++i) {
+                const double2 v = V[(long long)i * n + e];
+                const double2 ci = cs[i];
+                acc.x = fma(-v.x, ci.x, fma(v.y, ci.y, acc.x));
+                acc.y = fma(-v.x, ci.y, fma(-v.y, ci.x, acc.y));
+            }
+            w[e] = acc;
+        }
+    }
+    double acc = 0.0;
+    for (int e = e0; e < n; e += step) {
+        const double2 v = w[e];
+        acc += v.x * v.x + v.y * v.y;
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) sh[blk][0][wid] = acc;
+    __syncthreads();
+    if (wid == 0) {
+        const double r = warp_sum(lane < RB / 32 ? sh[blk][0][lane] : 0.0);
+        if (lane == 0) npart[blk] = r;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) {
+            beta2_sh = small_tree(npart, 1, nblk);
+            st->beta2 = beta2_sh;
+        }
+        __syncwarp();
+        ritz_step(st, nv, tol, breakdown, last, sc);
+        __syncwarp();
+        if (threadIdx.x == 0) flag_sh = st->flag;
+    }
+    __syncthreads();
+    if (flag_sh) return;
+    const double s = 1.0 / sqrt(beta2_sh);
+    double2* next = V + (long long)(j + 1) * n;
+    for (int e = e0; e < n; e += step) {
+        const double2 v = w[e];
+        next[e] = make_double2(v.x * s, v.y * s);
     }
 }
 
@@ -392,24 +531,34 @@ LanczosResult lanczos(Ctx& ctx, long long n, double2* x, double tol, int kmax, i
     ctx.count_launch();
     LanczosResult res{0.0, 0, false};
     const double breakdown = 1e-14;
+    // the vector work after matvec j: v_{j+1} = w / beta_j unless the iteration stops there
+    auto step = [&](int j, const int* stop) {
+        const int last = j == kmax - 1 ? 1 : 0;
+        if (nblk <= SMALL_BLOCKS) {
+            lanczos_small_kernel<<<1, nblk * RB, 0, ctx.stream>>>(V, (int)n, j, W, st, tol, breakdown, last, nblk);
+            ctx.count_launch();
+            return;
+        }
+        multi_dot(ctx, V, n, j + 1, W, n, st->c1, stop);
+        multi_axpy(ctx, V, n, j + 1, st->c1, W, n, stop);
+        multi_dot(ctx, V, n, j + 1, W, n, st->c2, stop);
+        multi_axpy(ctx, V, n, j + 1, st->c2, W, n, stop);
+        norm2_dev(ctx, W, n, &st->beta2, stop);
+        ritz_kernel<<<1, 32, 0, ctx.stream>>>(st, j + 1, tol, breakdown, last);
+        ctx.count_launch();
+        if (!last) {
+            scale_kernel<<<nblk, RB, 0, ctx.stream>>>(V + (size_t)(j + 1) * n, n, &st->beta2, &st->flag, W);
+            ctx.count_launch();
+        }
+    };
     if (defer != nullptr && restarts == 0) {
         // device-driven: all kmax steps queued; the stop flag set by ritz_kernel ends the
         // recursion on the device, and the Ritz vector is built from the first m_stop vectors
-        const int* stop = &st->stop;
+        const int* stop = &st->stop;  // (every vector kernel returns once it is set)
         for (int j = 0; j < kmax; ++j) {
             matvec(V + (size_t)j * n, W);
             int tl = ctx.tbegin(TC_LANCZOS, 0.0);
-            multi_dot(ctx, V, n, j + 1, W, n, st->c1, stop);
-            multi_axpy(ctx, V, n, j + 1, st->c1, W, n, stop);
-            multi_dot(ctx, V, n, j + 1, W, n, st->c2, stop);
-            multi_axpy(ctx, V, n, j + 1, st->c2, W, n, stop);
-            norm2_dev(ctx, W, n, &st->beta2, stop);
-            ritz_kernel<<<1, 32, 0, ctx.stream>>>(st, j + 1, tol, breakdown, j == kmax - 1 ? 1 : 0);
-            ctx.count_launch();
-            if (j + 1 < kmax) {
-                scale_kernel<<<nblk, RB, 0, ctx.stream>>>(V + (size_t)(j + 1) * n, n, &st->beta2, &st->flag, W);
-                ctx.count_launch();
-            }
+            step(j, stop);
             ctx.tend(tl);
             ctx.check_launch("lanczos iteration");
         }
@@ -431,18 +580,7 @@ LanczosResult lanczos(Ctx& ctx, long long n, double2* x, double tol, int kmax, i
             matvec(vj, W);
             res.n_matvec++;
             int tl = ctx.tbegin(TC_LANCZOS, 0.0);
-            multi_dot(ctx, V, n, j + 1, W, n, st->c1);
-            multi_axpy(ctx, V, n, j + 1, st->c1, W, n);
-            multi_dot(ctx, V, n, j + 1, W, n, st->c2);
-            multi_axpy(ctx, V, n, j + 1, st->c2, W, n);
-            norm2_dev(ctx, W, n, &st->beta2);
-            ritz_kernel<<<1, 32, 0, ctx.stream>>>(st, j + 1, tol, breakdown, j == kmax - 1 ? 1 : 0);
-            ctx.count_launch();
-            if (j + 1 < kmax) {
-                // v_{j+1} = w / beta_j unless the iteration stops here
-                scale_kernel<<<nblk, RB, 0, ctx.stream>>>(V + (size_t)(j + 1) * n, n, &st->beta2, &st->flag, W);
-                ctx.count_launch();
-            }
+            step(j, nullptr);
             ctx.tend(tl);
             ctx.check_launch("lanczos iteration");
             VTN_CUDA_TRY(cudaMemcpyAsync(ctx.pinned, &st->theta, 3 * sizeof(double) + sizeof(int),
