@@ -200,8 +200,14 @@ struct MixIn {
     long long cs, ps, ss;
 };
 
+// where the mixed tensor goes as the split A operand of the next product instead (row (b, p), inner index (s', q))
+struct MixPack {
+    __nv_bfloat16* out;  // null: plain FP32 output
+    long long ldo, half;
+};
+
 template <int DM>
-__global__ void __launch_bounds__(256) mix_f32_kernel(int P, int d, int Q, MixIn st, const int* __restrict__ ptr,
+__global__ void __launch_bounds__(256) mix_f32_kernel(int P, int d, int Q, MixIn st, MixPack pk, const int* __restrict__ ptr,
                                                       const int* __restrict__ src, const int* __restrict__ opi,
                                                       const float2* __restrict__ ops, const float2* __restrict__ in, float2* __restrict__ out,
                                                       int accumulate) {
@@ -268,6 +274,24 @@ __global__ void __launch_bounds__(256) mix_f32_kernel(int P, int d, int Q, MixIn
         }
     }
     if (!active) return;
+    if (pk.out != nullptr) {
+        __nv_bfloat16* o = pk.out + ((long long)b * P + pp) * pk.ldo + q;
+        const long long Kt = (long long)d * Q;
+#pragma unroll
+        for (int sp = 0; sp < DM; ++sp) {
+            if (sp < d) {
+                __nv_bfloat16 rh, rl, ih, il;
+                CplxTraits<float2>::split(acc[sp].x, rh, rl);
+                CplxTraits<float2>::split(acc[sp].y, ih, il);
+                __nv_bfloat16* r = o + (long long)sp * Q;
+                r[0] = rh;
+                r[Kt] = ih;
+                r[pk.half] = rl;
+                r[pk.half + Kt] = il;
+            }
+        }
+        return;
+    }
     float2* y = out + (long long)b * blk + pp * d * Q + q;
 #pragma unroll
     for (int sp = 0; sp < DM; ++sp) {
@@ -444,6 +468,16 @@ void launch_mix_cid(Ctx& ctx, int JB, int EI, bool real_c, int bytes, unsigned g
 // row width of a split operand: two halves of 2 Kt columns, each padded to a multiple of 64
 long long ksplit(long long Kt) { return 2 * (((2 * Kt + 63) / 64) * 64); }
 
+// zeroes the padding columns of both halves of a split operand
+void pad_halves(Ctx& ctx, __nv_bfloat16* out, long long ldo, int rows, long long Kt) {
+    const int from = (int)(2 * Kt), to = (int)(ldo / 2);
+    if (to <= from) return;
+    const long long cnt = (long long)rows * (to - from);
+    zero_pad_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx.stream>>>(out, ldo, rows, from, to);
+    zero_pad_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx.stream>>>(out, ldo, rows, to + from, 2 * to);
+    ctx.count_launch(2);
+}
+
 template <typename T>
 void pack_impl(Ctx& ctx, const T* X, int rows, int K, int kb, long long ld, long long s_kb, bool conj_t, bool is_b,
                __nv_bfloat16* out, int rq, long long s_rq) {
@@ -472,15 +506,7 @@ void pack_impl(Ctx& ctx, const T* X, int rows, int K, int kb, long long ld, long
         VTN_REQUIRE(grid.y <= 65535, "pack: too many rows");
         pack_kernel<T><<<grid, dim3(32, 8), 0, ctx.stream>>>(X, p);
     }
-    const int orows = is_b ? 2 * rows : rows;
-    const int from = (int)(2 * Kt), to = (int)(ldo / 2);
-    if (to > from) {
-        // the padding of both halves
-        const long long cnt = (long long)orows * (to - from);
-        zero_pad_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx.stream>>>(out, ldo, orows, from, to);
-        zero_pad_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx.stream>>>(out, ldo, orows, to + from, 2 * to);
-        ctx.count_launch(2);
-    }
+    pad_halves(ctx, out, ldo, is_b ? 2 * rows : rows, Kt);
     ctx.count_launch();
     ctx.check_launch(rows4 ? "pack_rows4_kernel" : "pack_kernel");
 }
@@ -521,7 +547,7 @@ bool channel_gemm_f32(Ctx& ctx, int w_in, int w_out, long long E, const float2* 
 }
 
 void mix_apply_f32(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const float2* in, float2* out,
-                   const long long* in_strides) {
+                   const long long* in_strides, __nv_bfloat16* packed) {
     const int w_out = by_col ? core.wr : core.wl;
     const int d = core.d;
     const long long PQ = (long long)P * Q;
@@ -562,13 +588,24 @@ void mix_apply_f32(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, con
         }
     }
     const dim3 grid((unsigned)((PQ + 255) / 256), w_out);
+    MixPack pk{nullptr, 0, 0};
+    if (packed != nullptr) {
+        VTN_REQUIRE(!accumulate, "a packed mixing output cannot be accumulated");
+        pk.out = packed;
+        pk.ldo = ksplit((long long)d * Q);
+        pk.half = pk.ldo / 2;
+        pad_halves(ctx, packed, pk.ldo, w_out * P, (long long)d * Q);
+    }
     const int *ptr = core.mix_ptr[list], *src = core.mix_src[list], *opi = core.mix_op[list];
     if (d <= 4)
-        mix_f32_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, in, out, accumulate ? 1 : 0);
+        mix_f32_kernel<4><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, pk, ptr, src, opi, core.ops_f32, in, out,
+                                                        accumulate ? 1 : 0);
     else if (d <= 8)
-        mix_f32_kernel<8><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, in, out, accumulate ? 1 : 0);
+        mix_f32_kernel<8><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, pk, ptr, src, opi, core.ops_f32, in, out,
+                                                        accumulate ? 1 : 0);
     else
-        mix_f32_kernel<16><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, ptr, src, opi, core.ops_f32, in, out, accumulate ? 1 : 0);
+        mix_f32_kernel<16><<<grid, 256, 0, ctx.stream>>>(P, d, Q, st, pk, ptr, src, opi, core.ops_f32, in, out,
+                                                        accumulate ? 1 : 0);
     ctx.count_launch();
     ctx.check_launch("mix_f32_kernel");
     ctx.tend(t);
@@ -750,7 +787,6 @@ void env_right_bf16x3(Ctx& ctx, const DevCore& W, int chi_l, int chi_r, const do
     __nv_bfloat16* PA = (__nv_bfloat16*)ctx.workspace(WS_TC_L, sizeof(__nv_bfloat16) * (size_t)chi_l * d * ld1);
     __nv_bfloat16* PB = (__nv_bfloat16*)ctx.workspace(WS_TC_R, sizeof(__nv_bfloat16) * (size_t)2 * wr * chi_r * ld1);
     float2* X = (float2*)ctx.workspace(WS_X, sizeof(float2) * (size_t)wmax * nA);
-    float2* Yb = (float2*)ctx.workspace(WS_Y, sizeof(float2) * (size_t)wmax * nA);
     tc_pack(ctx, A, chi_l * d, chi_r, 1, chi_r, 0, false, false, PA);
     tc_pack(ctx, R, wr * chi_r, chi_r, 1, chi_r, 0, false, true, PB, chi_r, (long long)chi_r * chi_r);
     TcGemmArgs g1;
@@ -770,12 +806,13 @@ void env_right_bf16x3(Ctx& ctx, const DevCore& W, int chi_l, int chi_r, const do
     // 2. U[b][j][t][p] = sum W[b,c,t,s] T[c][j][s][p]; T element (c, j, s, p) sits at
     //    ((j d + s) wr + c) chi_r + p
     const long long st[3] = {chi_r, (long long)d * wr * chi_r, (long long)wr * chi_r};
-    mix_apply_f32(ctx, W, false, chi_l, chi_r, X, Yb, st);
-    // 3. out[(b,j)][i] = sum_{(t,p)} U[(b,j)][(t,p)] conj(A[i][(t,p)])
+    //    Written as the split A operand of the third product right away (rows (b, j), inner (t, p)): an FP32 tensor and
+    //    a pass over it less (the large workload's update at chi = 384: mixing and packing 585 -> 442 us).
     const long long ld3 = ksplit((long long)d * chi_r);
     __nv_bfloat16* PA3 = (__nv_bfloat16*)ctx.workspace(WS_TC_A2, sizeof(__nv_bfloat16) * (size_t)wl * chi_l * ld3);
     __nv_bfloat16* PB3 = (__nv_bfloat16*)ctx.workspace(WS_TC_B1, sizeof(__nv_bfloat16) * (size_t)2 * chi_l * ld3);
-    tc_pack(ctx, (const float2*)Yb, wl * chi_l, d * chi_r, 1, (long long)d * chi_r, 0, false, false, PA3);
+    mix_apply_f32(ctx, W, false, chi_l, chi_r, X, nullptr, st, PA3);
+    // 3. out[(b,j)][i] = sum_{(t,p)} U[(b,j)][(t,p)] conj(A[i][(t,p)])
     tc_pack(ctx, A, chi_l, d * chi_r, 1, (long long)d * chi_r, 0, true, true, PB3);
     TcGemmArgs g3;
     g3.M = wl * chi_l;

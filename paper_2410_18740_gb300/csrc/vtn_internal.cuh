@@ -247,8 +247,10 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
                double2* out);
 
 // in_strides (optional): channel, p and s strides of the input (default: standard layout)
+// packed (optional, not for a collapse core by column): the result as a split A operand of w_out P rows and inner
+// index (s', q) instead of `out`
 void mix_apply_f32(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const float2* in, float2* out,
-                   const long long* in_strides = nullptr);
+                   const long long* in_strides = nullptr, __nv_bfloat16* packed = nullptr);
 
 // ------------------------------------------------------------------ contractions
 void heff_apply_dev(Ctx& ctx, const DevCore& Wi, const DevCore& Wj, int chi_l, int chi_r,
