@@ -134,8 +134,8 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
         double grown = 0.0, degrees = 0.0;
         bool done = false;
         for (int cycle = 0; cycle < 32 && !done; ++cycle) {
-            // the first block is not in Schur order yet: its rows may part by 1e5 only; later ones by 1e11
-            int D = (int)(std::log(cycle == 0 ? 1e5 : 1e11) / g1);
+            // the first block is not in Schur order yet: its rows may part by 1e6 only; later ones by 1e13
+            int D = (int)(std::log(cycle == 0 ? 1e6 : 1e13) / g1);
             D = std::max(2, std::min({D, 12, (int)std::ceil((36.0 - grown) / gk)}));
             degrees += D;
             if (degrees > 2.0 * limit) return false;
