@@ -110,38 +110,49 @@ __device__ __forceinline__ int k_shift(const OzShift* sh, const int* kxa, const 
 
 constexpr int MAX_KS = 64;
 
-// Largest exponent of each row: 32 rows x 64 summation indices per block, 8 warps (eight independent loads a
-// thread: one memory latency).  PASS 0 takes the
+// Largest exponent of each row: tiles of 32 rows x 64 summation indices, 8 warps (eight independent loads a
+// thread: one memory latency), `reps` tiles of the same indices one after the other per block: as many as make
+// the grid about eight blocks an SM, so that a large operand's blocks do not queue for the same 64 index
+// maxima and the one counter.  PASS 0 takes the
 // unscaled rows and the exponents kx of the summation indices; its last block decides whether the summation
 // index needs scaling (OzShift::on) and clears the row exponents if it does.  PASS 1 then takes the
 // scaled rows (and returns at once where no scaling is needed).
+// Bound by its loads: comparisons of doubles cost more than a load on the FP64 pipe, and loads that wait behind
+// an atomic come two at a time.  Without both, mean of the three products of an H_eff application at chi 256, d 4:
+// 132 -> 71 us; of the products of a readout at chi 96 (mostly latency): 10.4 -> 6.2 us.
 template <int PASS>
 __global__ void __launch_bounds__(256) oz_max_kernel(OzOperand a, OzOperand b, OzShift* shift, int nblk_a, int kseg,
-                                                     int n_bx) {
+                                                     int reps, int n_bx) {
     if (PASS == 1 && !shift->on) return;
     const bool is_b = (int)blockIdx.x >= nblk_a;
     const OzOperand& o = is_b ? b : a;
     const int id = is_b ? (int)blockIdx.x - nblk_a : (int)blockIdx.x;
-    const int rb = (o.rows + 31) / 32;
-    const int seg = id % kseg, rt = (id / kseg) % rb, bt = id / (kseg * rb);
+    const int rb = (o.rows + 31) / 32, rg = (rb + reps - 1) / reps;
+    const int seg = id % kseg, rt0 = (id / kseg) % rg * reps, rt1 = min(rb, rt0 + reps), bt = id / (kseg * rg);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int Kt = o.K * o.kbn;
     const int k0 = seg * MAX_KS, k1 = min(Kt, k0 + MAX_KS);
     const long long base = (long long)bt * o.s_batch;
     int* bx = o.bx + (long long)bt * o.tiles * (is_b ? TNC : TM);
     __shared__ int kmax[MAX_KS];
-    __shared__ int sh[8][32];
+    __shared__ int sh[2][8][32];
     if (PASS == 0) {
         if (threadIdx.x < MAX_KS) kmax[threadIdx.x] = 0;
         __syncthreads();
     }
-    auto exp_of = [&](int row, int kk, int& raw) {
-        const int kb = kk / o.K;
-        const double2 v = oz_load(o, base, row, kb, kk - kb * o.K);
+    auto load = [&](int row, int kk) {
+        if (row >= o.rows || kk >= k1) return make_double2(0.0, 0.0);
+        const int kb = o.kbn > 1 ? kk / o.K : 0;
+        const double2* p = o.X + base + kb * o.s_kb;
+        const long long k = kk - kb * o.K;
+        return __ldg(o.kc ? p + row * o.ld + k : p + k * o.ld + row);
+    };
+    auto exp_of = [&](double2 v, int kk, int& raw) {
         raw = max(biased_exp(v.x), biased_exp(v.y));
-        const bool zero = v.x == 0.0 && v.y == 0.0;
         if (raw == 0x7ff) return NONFINITE;
-        if (zero) return 0;
+        // by bits: two comparisons of doubles an element are longer than its load on the narrow FP64 pipe
+        if (raw == 0 && ((unsigned)(__double2hiint(v.x) | __double2hiint(v.y)) << 1 | (unsigned)__double2loint(v.x) |
+                         (unsigned)__double2loint(v.y)) == 0u) return 0;
         int e = max(raw, 1);
         if (PASS == 1) {
             const int sk = k_shift(shift, a.kx, b.kx, kk);
@@ -149,50 +160,62 @@ __global__ void __launch_bounds__(256) oz_max_kernel(OzOperand a, OzOperand b, O
         }
         return e + EXP0;
     };
+    // (all loads of a tile before the first maximum: none moves up over an atomic)
+    constexpr int NL = MAX_KS / 8;
     if (o.kc) {
-        // a warp per row, its lanes along the summation index
-        int km[MAX_KS / 32];
+        // a warp per four rows, its lanes along the summation index
+        int km[2] = {0, 0};
+        for (int rt = rt0; rt < rt1; ++rt) {
+            const int row = rt * 32 + warp * 4;
+            double2 v[NL];
 #pragma unroll
-        for (int j = 0; j < MAX_KS / 32; ++j) km[j] = 0;
+            for (int j = 0; j < NL; ++j) v[j] = load(row + j / 2, k0 + (j & 1) * 32 + lane);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int row = rt * 32 + warp * 4 + r;
+            for (int r = 0; r < 4; ++r) {
+                int raw0, raw1;
+                int m = max(exp_of(v[2 * r], k0 + lane, raw0), exp_of(v[2 * r + 1], k0 + 32 + lane, raw1));
+                km[0] = max(km[0], raw0);
+                km[1] = max(km[1], raw1);
+                m = __reduce_max_sync(0xffffffffu, m);
+                if (lane == 0 && row + r < o.rows) atomicMax(&bx[row + r], m);
+            }
+        }
+        if (PASS == 0) {
+            atomicMax(&kmax[lane], km[0]);
+            atomicMax(&kmax[32 + lane], km[1]);
+        }
+    } else {
+        int km[NL];
+#pragma unroll
+        for (int j = 0; j < NL; ++j) km[j] = 0;
+        for (int rt = rt0; rt < rt1; ++rt) {
+            const int row = rt * 32 + lane;
+            double2 v[NL];
+#pragma unroll
+            for (int j = 0; j < NL; ++j) v[j] = load(row, k0 + warp * NL + j);
             int m = 0;
 #pragma unroll
-            for (int j = 0; j < MAX_KS / 32; ++j) {
-                const int kk = k0 + j * 32 + lane;
-                if (row < o.rows && kk < k1) {
-                    int raw;
-                    m = max(m, exp_of(row, kk, raw));
-                    km[j] = max(km[j], raw);
-                }
+            for (int j = 0; j < NL; ++j) {
+                int raw;
+                m = max(m, exp_of(v[j], k0 + warp * NL + j, raw));
+                km[j] = max(km[j], raw);
             }
-            m = __reduce_max_sync(0xffffffffu, m);
-            if (lane == 0 && row < o.rows) atomicMax(&bx[row], m);
+            // two buffers: a warp is at most one tile ahead of the one that reads
+            int(*part)[32] = sh[rt & 1];
+            part[warp][lane] = m;
+            __syncthreads();
+            if (warp == (rt & 7) && row < o.rows) {
+#pragma unroll
+                for (int w = 0; w < 8; ++w) m = max(m, part[w][lane]);
+                atomicMax(&bx[row], m);
+            }
         }
         if (PASS == 0)
 #pragma unroll
-            for (int j = 0; j < MAX_KS / 32; ++j) atomicMax(&kmax[j * 32 + lane], km[j]);
-    } else {
-        const int row = rt * 32 + lane;
-        int m = 0;
-#pragma unroll
-        for (int j = 0; j < MAX_KS / 8; ++j) {
-            const int kk = k0 + warp * (MAX_KS / 8) + j;
-            int raw = 0;
-            if (row < o.rows && kk < k1) m = max(m, exp_of(row, kk, raw));
-            if (PASS == 0) {
-                raw = __reduce_max_sync(0xffffffffu, raw);
-                if (lane == 0) kmax[kk - k0] = raw;  // this warp alone has index kk in this block
+            for (int j = 0; j < NL; ++j) {
+                const int kk = warp * NL + j, raw = __reduce_max_sync(0xffffffffu, km[j]);
+                if (lane == 0) kmax[kk] = raw;  // this warp alone has index kk in this block
             }
-        }
-        sh[warp][lane] = m;
-        __syncthreads();
-        if (warp == 0 && row < o.rows) {
-#pragma unroll
-            for (int w = 1; w < 8; ++w) m = max(m, sh[w][lane]);
-            atomicMax(&bx[row], m);
-        }
     }
     if (PASS == 1 || n_bx < 0) return;  // a prepared operand leaves no choice
     __syncthreads();
@@ -206,26 +229,35 @@ __global__ void __launch_bounds__(256) oz_max_kernel(OzOperand a, OzOperand b, O
     if (!last_sh) return;
     __threadfence();
     int ma = 0, mb = 0, mt = 0;
-    for (int kk = threadIdx.x; kk < Kt; kk += 256) {
-        const int x = __ldcg(&a.kx[kk]), y = __ldcg(&b.kx[kk]);
-        if (x == 0x7ff || y == 0x7ff) continue;  // those rows and columns are summed directly
-        ma = max(ma, x);
-        mb = max(mb, y);
-        if (x > 0 && y > 0) mt = max(mt, x + y);
+    for (int kk0 = threadIdx.x; kk0 < Kt; kk0 += 8 * 256) {
+        int x[8], y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int kk = kk0 + j * 256;
+            x[j] = kk < Kt ? __ldcg(&a.kx[kk]) : 0;
+            y[j] = kk < Kt ? __ldcg(&b.kx[kk]) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (x[j] == 0x7ff || y[j] == 0x7ff) continue;  // those rows and columns are summed directly
+            ma = max(ma, x[j]);
+            mb = max(mb, y[j]);
+            if (x[j] > 0 && y[j] > 0) mt = max(mt, x[j] + y[j]);
+        }
     }
     ma = __reduce_max_sync(0xffffffffu, ma);
     mb = __reduce_max_sync(0xffffffffu, mb);
     mt = __reduce_max_sync(0xffffffffu, mt);
     if (lane == 0) {
-        sh[0][warp] = ma;
-        sh[1][warp] = mb;
-        sh[2][warp] = mt;
+        sh[0][0][warp] = ma;
+        sh[0][1][warp] = mb;
+        sh[0][2][warp] = mt;
     }
     __syncthreads();
     for (int w = 0; w < 8; ++w) {
-        ma = max(ma, sh[0][w]);
-        mb = max(mb, sh[1][w]);
-        mt = max(mt, sh[2][w]);
+        ma = max(ma, sh[0][0][w]);
+        mb = max(mb, sh[0][1][w]);
+        mt = max(mt, sh[0][2][w]);
     }
     if (mt > 0 && ma + mb - mt > LOSS_BITS) {
         for (int i = threadIdx.x; i < n_bx; i += 256) a.bx[i] = 0;  // bx of A and B are contiguous
@@ -615,6 +647,9 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
 
 long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
 
+// tiles per block of the exponent kernel
+int max_reps(const Ctx& ctx, long long tiles) { return (int)cdiv(tiles, 8ll * std::max(ctx.num_sms, 1)); }
+
 }  // namespace
 
 // Splits of the summation over the CTAs: the smallest number (<= 16) whose waves of equal items come within a
@@ -663,9 +698,9 @@ OzPrep oz_prepare(Ctx& ctx, int M, int K, Op opA, const double2* A, long long ld
     OzShift* shift = (OzShift*)(a.bx + n_bx);
     a.kx = nullptr;
     VTN_CUDA_TRY(cudaMemsetAsync(a.bx, 0, sizeof(int) * n_bx + sizeof(OzShift), ctx.stream));
-    const int kseg = (int)cdiv(K, MAX_KS);
-    const long long ma = cdiv(M, 32) * kseg, sa = (long long)tiles * nkb;
-    oz_max_kernel<0><<<(unsigned)ma, 256, 0, ctx.stream>>>(a, a, shift, (int)ma, kseg, -1);
+    const int kseg = (int)cdiv(K, MAX_KS), reps = max_reps(ctx, cdiv(M, 32) * kseg);
+    const long long ma = cdiv(cdiv(M, 32), reps) * kseg, sa = (long long)tiles * nkb;
+    oz_max_kernel<0><<<(unsigned)ma, 256, 0, ctx.stream>>>(a, a, shift, (int)ma, kseg, reps, -1);
     oz_slice_kernel<<<(unsigned)sa, 256, 0, ctx.stream>>>(a, a, shift, (int)sa, nkb);
     ctx.count_launch(2);
     ctx.check_launch("oz_prepare");
@@ -727,10 +762,12 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 p.status = ctx.dstatus;
                 VTN_CUDA_TRY(cudaMemsetAsync(shift, 0, sizeof(int) * n_exp, ctx.stream));
                 const int kseg = (int)cdiv((long long)g.K * g.kb, MAX_KS);
-                const long long ma = prep ? 0 : cdiv(mm, 32) * kseg * p.a.nb, mb = cdiv(nn, 32) * kseg * p.b.nb;
-                oz_max_kernel<0><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg,
+                const long long ra = prep ? 0 : cdiv(mm, 32), rb = cdiv(nn, 32);
+                const int reps = max_reps(ctx, (ra * p.a.nb + rb * p.b.nb) * kseg);
+                const long long ma = cdiv(ra, reps) * kseg * p.a.nb, mb = cdiv(rb, reps) * kseg * p.b.nb;
+                oz_max_kernel<0><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg, reps,
                                                                               prep ? -1 : (int)(na + nbx));
-                if (!prep) oz_max_kernel<1><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg, 0);
+                if (!prep) oz_max_kernel<1><<<(unsigned)(ma + mb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)ma, kseg, reps, 0);
                 const long long sa = prep ? 0 : (long long)p.a.nb * p.tiles_m * nkb, sb = (long long)p.b.nb * p.tiles_n * nkb;
                 oz_slice_kernel<<<(unsigned)(sa + sb), 256, 0, ctx.stream>>>(p.a, p.b, shift, (int)sa, nkb);
                 const long long items = (long long)p.tiles_m * p.tiles_n * nb * splits;

@@ -76,6 +76,17 @@ def test_sliced_product_of_opposed_gradings(ctx):
     assert _worst(L, th, _product(ctx, L, th), rng) <= 1.0
 
 
+@pytest.mark.parametrize("m,n,decades", [(64, 2300, 0), (33, 2275, 28)])
+def test_sliced_product_with_several_row_tiles_a_block(ctx, m, n, decades):
+    """The right operand's exponents taken by blocks of more than one tile of columns, with and without the
+    scaling of the summation index: theta R, with L = I the exact product."""
+    import torch
+    rng = np.random.default_rng(n)
+    g = torch.logspace(0, -decades, n, dtype=torch.float64, device="cuda")
+    th, R = _randn(rng, m, n) * g[None, :], _randn(rng, n, n) * g.flip(0)[:, None]
+    assert _worst(th, R, _product(ctx, torch.eye(m, dtype=torch.complex128, device="cuda"), th, R), rng) <= 1.0
+
+
 def test_sliced_product_with_non_finite_rows_and_extreme_scales(ctx):
     import torch
     rng = np.random.default_rng(9)
