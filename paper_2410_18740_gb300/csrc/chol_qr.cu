@@ -44,8 +44,8 @@ __device__ __forceinline__ double rsqrt_newton(double x) {
 // One CTA, b <= NB.  flag[0] = 1 on a pivot that is not positive.
 // FP64-issue bound (about 2 x 170 warp-wide element updates of 6 instructions), so the elements left of each step are
 // dealt out densely to the lanes: L D L^dag with unit L, the update of column j and the same row operations on
-// the growing inverse in one pass with one barrier, the square roots taken once at the end, the next pivot while the others still work.  168 -> 50 us
-// for a block of 32 (three barriers a column and the inverse as 32 serial dot products before).
+// the growing inverse in one pass with one barrier, the square roots taken once at the end, the next pivot while
+// the others still work.  168 -> 50 us for a block of 32 (three barriers a column and the inverse as 32 serial dot products before).
 __global__ void __launch_bounds__(256) potrf_block(double2* __restrict__ G, int b, long long ld,
                                                   double2* __restrict__ Linv, int* __restrict__ flag) {
     __shared__ double2 S[NB][NB + 1];

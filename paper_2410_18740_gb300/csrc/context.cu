@@ -17,9 +17,14 @@ void* Ctx::dalloc(size_t bytes) {
     void* p = nullptr;
     if (has_alloc) {
         p = alloc.alloc(bytes, alloc.user);
+        if (!p && drop_digits()) p = alloc.alloc(bytes, alloc.user);
         if (!p) throw Error{VTN_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed"};
     } else {
         cudaError_t e = cudaMalloc(&p, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (drop_digits()) e = cudaMalloc(&p, bytes);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             throw Error{VTN_ENOMEM, "cudaMalloc(" + std::to_string(bytes) + "): " + cudaGetErrorString(e)};
@@ -58,6 +63,24 @@ void* Ctx::workspace(int slot, size_t bytes) {
         b.bytes = want;
     }
     return b.p;
+}
+
+void Ctx::drop(int slot) {
+    if (slot >= (int)ws.size() || ws[slot].p == nullptr) return;
+    sync();
+    dfree(ws[slot].p);
+    ws[slot].p = nullptr;
+    ws[slot].bytes = 0;
+}
+
+bool Ctx::drop_digits() {
+    if (digits_busy) return false;
+    size_t held = 0;
+    for (int s : {WS_OZ_EXP, WS_OZ_A, WS_OZ_B}) {
+        if (s < (int)ws.size()) held += ws[s].bytes;
+        drop(s);
+    }
+    return held > 0;
 }
 
 double* Ctx::defer_reserve(size_t doubles) {

@@ -132,6 +132,7 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
     // out[b][e] = sum_a C[a][b] in[a][e], which the FP64 pipe does at two operations a coupling and element (0.49e12
     // a second) and the sliced GEMM (rows e, padded to 16 channels a stage) at 0.13 us per 128 elements and
     // stage plus 35 us: the split workload's centre core at chi = 128 takes 2.6 against 1.1 ms.
+    bool collapsed = false;
     const double stages = ((by_col ? core.wl : core.wr) + 15) / 16;
     if (terms && core.cid64 != nullptr && ctx.dstatus != nullptr && E < (1LL << 30) && w_out <= 1024 &&
         2.0 * core.n_ident * E / 0.49e12 > 1.2 * (35e-6 + E / 128.0 * (stages * 0.05e-6 + 0.03e-6))) {
@@ -140,10 +141,12 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
         g.opA = OP_T; g.A = in; g.lda = E;
         g.opB = by_col ? OP_N : OP_T; g.B = core.cid64; g.ldb = core.wr;
         g.C = out; g.ldc = 1; g.sC_n = E;
-        oz_gemm(ctx, g, 1, nullptr);
+        collapsed = oz_gemm(ctx, g, 1, nullptr);
+    }
+    if (collapsed)
         mix_terms_kernel<true><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, w_out * d, core.nz_ptr[2 + dir], core.nz_src[2 + dir],
                                                               core.nz_c[2 + dir], in, out);
-    } else if (terms)
+    else if (terms)
         mix_terms_kernel<false><<<tgrid, 256, 0, ctx.stream>>>(PQ, d, Q, w_out * d, core.nz_ptr[dir], core.nz_src[dir],
                                                                core.nz_c[dir], in, out);
     else if (d <= 4)

@@ -1,6 +1,8 @@
 // FP64 truncation eigensolver: the reduced density matrix rho of a two-site tensor,
 // its largest k eigenpairs, and the split of the tensor into a canonical site and the
-// new centre.  Every step runs on the GPU:
+// new centre.  From n = 257 on the filtered subspace iteration of trunc_filter.cu comes first (truncate_dev) and leaves
+// a smaller problem of the same form to these steps; where it gives up they take all of rho.  Every step runs
+// on the GPU:
 //
 //  1. rho = T T^dag (or T^dag T) by the complex GEMM.
 //  2. Householder tridiagonalisation of the Hermitian rho (Golub & Van Loan, Sec. 8.3.1):
@@ -1729,7 +1731,13 @@ TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int dir
     VTN_REQUIRE(n <= 12288, "reduced density matrix larger than 12288 is not supported");
     if (const int m = filter_rows(nL, nR, direction, k)) {
         TruncResult r;
-        if (truncate_filtered(ctx, nL, nR, direction, k, m, theta, left, right, outer, defer, r)) return r;
+        try {
+            if (truncate_filtered(ctx, nL, nR, direction, k, m, theta, left, right, outer, defer, r)) return r;
+        } catch (const Error& e) {
+            // the reduction below needs less memory
+            if (e.status != VTN_ENOMEM) throw;
+            for (int s : {WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_U, WS_OZ_PREP}) ctx.drop(s);
+        }
     }
     int tt = ctx.tbegin(TC_EIG, 0.0);
     double2* A = (double2*)ctx.workspace(WS_EIG_A, sizeof(double2) * (size_t)n * n);

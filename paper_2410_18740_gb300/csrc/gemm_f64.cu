@@ -168,7 +168,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     // against sliced: 128^3 22 | 34 us, 160^3 34 | 35 us, 192^3 55 | 37 us, 256^3 136 | 38 us, 1024 x 16 x 1024
     // (narrow: padded to 32 columns) 74 | 49 us; at 3072^3 200 ms against 6.1 ms.  Its row sums fit 96-bit integers
     // for summations of up to 2^19 terms.
-    const bool oz = g.prepA != nullptr || ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.2e6 && (long long)g.K * g.kb <= (1LL << 19);
+    bool oz = g.prepA != nullptr || ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.2e6 && (long long)g.K * g.kb <= (1LL << 19);
     int S = 1;
     if (oz) {
         S = oz_splits(ctx, g);
@@ -181,18 +181,24 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     }
     if (g.max_splits > 0) S = std::min(S, g.max_splits);
     S = std::max(S, 1);
-    p.splits = S;
     p.part = nullptr;
-    if (S > 1)
-        p.part = (double2*)ctx.workspace(WS_GEMM_SPLIT, sizeof(double2) * (size_t)S * g.batch * g.M * g.N);
+    if (S > 1) {
+        try {
+            p.part = (double2*)ctx.workspace(WS_GEMM_SPLIT, sizeof(double2) * (size_t)S * g.batch * g.M * g.N);
+        } catch (const Error& e) {  // no memory for the sliced product's partial sums: the FP64 kernel, unsplit
+            if (e.status != VTN_ENOMEM || !oz || g.prepA != nullptr) throw;
+            oz = false;
+            S = 1;
+        }
+    }
+    p.splits = S;
     const long long ctas = gx * gy * g.batch * S;
-    VTN_REQUIRE(oz || ctas < (1LL << 31), "gemm too large");
     double flops = 8.0 * g.M * (double)g.N * g.K * g.kb * g.batch * (g.herm_lower ? 0.5 : 1.0);
     int t0 = ctx.tbegin(TC_GEMM, flops);
     int t1 = (timing_class != TC_GEMM) ? ctx.tbegin(timing_class, flops) : -1;
-    if (oz) {
-        oz_gemm(ctx, g, S, p.part);
-    } else {
+    if (!oz || !oz_gemm(ctx, g, S, p.part)) {
+        if (g.prepA != nullptr) throw Error{VTN_ENOMEM, "no device memory for the digits of a prepared product"};
+        VTN_REQUIRE(ctas < (1LL << 31), "gemm too large");
         gemm_c64_kernel<<<(unsigned)ctas, NT, 0, ctx.stream>>>(p);
         ctx.count_launch();
         ctx.check_launch("gemm_c64_kernel");

@@ -712,7 +712,9 @@ OzPrep oz_prepare(Ctx& ctx, int M, int K, Op opA, const double2* A, long long ld
     return p;
 }
 
-void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
+// Returns false, with nothing launched, when there is no device memory for the digits (the first piece needs the
+// most): the caller then takes the FP64 kernel, which needs none.
+bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
     VTN_REQUIRE(ctx.dstatus != nullptr, "context has no device status word");
     VTN_REQUIRE(g.prepA == nullptr || (g.prepA->M == g.M && g.prepA->K == g.K && g.batch == 1 && g.kb == 1),
                 "prepared operand of another shape");
@@ -746,14 +748,24 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 fill_operand(p.b, g, true, b0, n0, nn, p.tiles_n, b_shared ? 1 : nb);
                 const size_t na = prep ? 0 : (size_t)p.a.nb * p.tiles_m * TM, nbx = (size_t)p.b.nb * p.tiles_n * TNC;
                 const size_t nk = (size_t)g.K * g.kb, n_exp = sizeof(OzShift) / sizeof(int) + na + nbx + 2 * nk;
-                OzShift* shift = (OzShift*)ctx.workspace(WS_OZ_EXP, sizeof(int) * n_exp);
+                OzShift* shift;
+                ctx.digits_busy = true;
+                try {
+                    shift = (OzShift*)ctx.workspace(WS_OZ_EXP, sizeof(int) * n_exp);
+                    p.a.out = prep ? (uint4*)prep->digits
+                                   : (uint4*)ctx.workspace(WS_OZ_A, (size_t)p.a.nb * p.tiles_m * nkb * A_BYTES);
+                    p.b.out = (uint4*)ctx.workspace(WS_OZ_B, (size_t)p.b.nb * p.tiles_n * nkb * B_BYTES);
+                } catch (const Error& e) {
+                    ctx.digits_busy = false;
+                    if (e.status != VTN_ENOMEM || b0 + n0 + m0 > 0) throw;
+                    ctx.drop_digits();
+                    return false;
+                }
+                ctx.digits_busy = false;
                 p.a.bx = prep ? prep->bx : (int*)(shift + 1);
                 p.b.bx = (int*)(shift + 1) + na;
                 p.a.kx = p.b.bx + nbx;
                 p.b.kx = p.a.kx + nk;
-                p.a.out = prep ? (uint4*)prep->digits
-                               : (uint4*)ctx.workspace(WS_OZ_A, (size_t)p.a.nb * p.tiles_m * nkb * A_BYTES);
-                p.b.out = (uint4*)ctx.workspace(WS_OZ_B, (size_t)p.b.nb * p.tiles_n * nkb * B_BYTES);
                 p.C = g.C + b0 * g.sC_batch + m0 * g.ldc + n0 * g.sC_n;
                 p.ldc = g.ldc; p.sC_n = g.sC_n; p.sC_batch = g.sC_batch;
                 p.part = part;
@@ -779,6 +791,7 @@ void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
             }
         }
     }
+    return true;
 }
 
 }  // namespace vtn

@@ -13,10 +13,11 @@
 // Rows: S holds the conjugates of the vectors (m x n), so rho acts from the right; (S rho)^T = rho^T S^T is one
 // product with the digits of rho^T, which all products share.
 //
-// Measured (whole truncation, full reduction -> here): n = 512, k = 64 8.9 -> 7.2 ms; n = 1024, k = 128 29.8 -> 13.7 ms;
-// n = 1830, k = 300 86 -> 40 ms (Schmidt values decaying by e^-9); flat random spectra 8.9 -> 9.0, 29.8 -> 27.3,
-// 86 -> 71 ms.  What is left is latency: the Cholesky chains (1.8 us a row and pass), the m x m tridiagonalisation
-// (12 to 15 us a column) and about 50 us a product.
+// Measured (whole truncation; full reduction with sliced products -> here, when the step was made): n = 512, k = 64
+// 8.9 -> 7.2 ms; n = 1024, k = 128 29.8 -> 13.7 ms; n = 1830, k = 300 86 -> 40 ms (Schmidt values decaying by e^-9);
+// flat random spectra 8.9 -> 9.0, 29.8 -> 27.3, 86 -> 71 ms.  With the shorter Cholesky and tridiagonalisation chains
+// the middle two are 12.7 and 37.7 ms.  What is left is latency: the Cholesky chains (50 us per 32 rows and pass), the
+// m x m tridiagonalisation (10 us a column) and about 50 us a product.
 //
 // The host reads five numbers after each pass.  It gives up (false: the full eigendecomposition runs) when the
 // spectrum at k is so flat that the predicted polynomial degree costs more than the reduction, when the block is
@@ -159,8 +160,8 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
                 if (!(degrees + (35.0 - grown) / gk <= 2.0 * limit)) return false;
                 continue;
             }
-            // the pass lost orthogonality like u / pivot^2
-            if (pivot < 0.2 && !orth(S)) return false;
+            // the pass lost orthogonality like u / pivot^2 (a second pass costs 0.5 ms at m = 224)
+            if (pivot < 0.5 && !orth(S)) return false;
             // ---- residual of the first k rows: S rho - (S rho S^dag) S
             apply(S, P);
             GemmArgs h;

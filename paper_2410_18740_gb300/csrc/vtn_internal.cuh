@@ -142,7 +142,10 @@ struct Ctx {
 
     void* dalloc(size_t bytes);
     void dfree(void* p);
-    void* workspace(int slot, size_t bytes);  // grows, never shrinks
+    void* workspace(int slot, size_t bytes);  // grows; given back by drop() only
+    void drop(int slot);
+    bool drop_digits();  // gives back the digit buffers of the FP64 product unless one is being prepared
+    bool digits_busy = false;
     void count_launch(int n = 1) { launches += n; }
     // timing: begin() returns an index (or -1 when timing is off); end() closes it
     int tbegin(int cls, double flops);
@@ -209,7 +212,7 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class = TC_GEMM);
 // partial tiles [splits][batch][M][N] go to `part` instead of C.
 int oz_splits(const Ctx& ctx, const GemmArgs& g);
 OzPrep oz_prepare(Ctx& ctx, int M, int K, Op opA, const double2* A, long long lda);
-void oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part);
+bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part);
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize, bytes) for kernel fn on the context's
 // device, once per (kernel, device) (the attribute is per device); thread-safe.

@@ -119,3 +119,37 @@ def test_sliced_products_of_the_environment_updates(ctx):
         ref = torch.einsum("itl,aij,jtk->alk", A.conj(), E, A) if side == 0 else torch.einsum("jtg,agp,itp->aji", A, E, A.conj())
         # two products of lengths ci and d * (the other): the reference's own rounding, u sqrt(K) each, with room
         assert float(torch.linalg.norm(out - ref) / torch.linalg.norm(ref)) <= 1e-14
+
+
+def test_products_without_memory_for_the_digits(monkeypatch):
+    """An allocator that refuses what the digits need: the FP64 kernel computes the product, the full reduction the
+    truncation, and what the allocator gave is all given back."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(3)
+    n, k, held, refused = 512, 64, {}, []
+
+    def alloc(nbytes, user):
+        if nbytes > 6 << 20:  # n x n complex numbers are 4 MiB, the digits of the two operands 8 and 16
+            refused.append(nbytes)
+            return None
+        t = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    fields = vtn.vtn_allocator._fields_
+    a = vtn.vtn_allocator(fields[0][1](alloc), fields[1][1](lambda p, user: (held.pop(p), None)[1]), None)
+    monkeypatch.setattr(vtn, "_torch_allocator", lambda device: a)
+    ctx = vtn.vtn_create(0)
+    L, th = _randn(rng, n, n), _randn(rng, n, n)
+    y = _product(ctx, L, th)
+    # a sum of n products and the reference's: u sqrt(n) each, with room
+    assert float(torch.linalg.norm(y - L @ th) / torch.linalg.norm(L @ th)) <= 1e-14
+    left, right = _randn(rng, n, k), _randn(rng, k, n)
+    _, lam, _ = vtn.vtn_truncate(ctx, n // 8, 8, 8, n // 8, 0, k, th, left, right)
+    s = np.linalg.svd(th.cpu().numpy(), compute_uv=False)[:k] ** 2
+    # n roundings of the largest eigenvalue
+    assert np.abs(np.asarray(lam) - s).max() <= n * 2.0 ** -52 * s[0]
+    assert refused and held
+    vtn.vtn_destroy(ctx)
+    assert not held
