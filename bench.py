@@ -70,9 +70,6 @@ TRI_LOWER_TRAFFIC = (1.152237 + 19.671560) * 1e9
 # DRAM bytes (read + write) per launch of the term-form H_eff GEMM pair at the large workload's centre
 # bond (ncu, bench.py --case heff --workload large): 15.51 + 8.58 GB and 10.90 + 1.64 GB; their mean.
 TC_GEMM_TRAFFIC_LARGE = 0.5 * ((15.508355 + 8.579924) + (10.900055 + 1.643347)) * 1e9
-# DRAM bytes (read + write) per launch of the FP64 complex GEMM pair of H_eff psi at the middle
-# bond of the split workload (ncu), mean of the two launches.
-GEMM_F64_TRAFFIC = 0.5 * ((30.710272 + 345.032960) + (416.077056 + 13.165824)) * 1e6
 # large workload: window of bonds [LO, HI) at the middle of the chain
 LARGE = "large"
 LARGE_SEED = 200
@@ -508,10 +505,13 @@ def run_native_large(args):
     n_gemm, fl_gemm, s_gemm = tm["gemm"]
     n_heff, fl_heff, s_heff = tm["heff"]
     K = args.steps
+    # a real FP64 product is 36 bf16 products of digits where it runs on the tensor cores
+    oz_peak = tc_peak / 36.0
     cands = {
         "tridiag": (s_tri, _roof("alu", fl_tri / s_tri / 1e12 if s_tri else None, fpeak, fpeak_src,
                                  "tridiag_lower (FP64 Householder tridiagonalisation of rho keeping the lower "
-                                 "triangle, one cooperative launch per truncation, n = 3072)",
+                                 "triangle, one cooperative launch per truncation whose spectrum is too flat for "
+                                 "the filtered subspace iteration, n = 3072)",
                                  "16/3 n^3 real flops per launch", n_tri, s_tri, K, TRI_LOWER_TRAFFIC,
                                  "ncu dram read+write of one launch at n = 3072 (the same kernel and shape)")),
         "tc_gemm": (s_tc, _roof("tensor", fl_tc / s_tc / 1e12 if s_tc else None, tc_peak,
@@ -523,10 +523,12 @@ def run_native_large(args):
                                 n_tc, s_tc, K, TC_GEMM_TRAFFIC_LARGE,
                                 "ncu dram read+write per launch, mean of the centre-bond H_eff GEMM pair of the "
                                 "term form (the step's launches also include smaller environment GEMMs)")),
-        "fp64_gemm": (s_gemm, _roof("alu", fl_gemm / s_gemm / 1e12 if s_gemm else None, fpeak, fpeak_src,
-                                    "gemm_c64_kernel (complex FP64 GEMM: rho, the truncation's products, "
-                                    "the Rayleigh quotient)", "8 M N K (Hermitian rho: half) real flops per launch",
-                                    n_gemm, s_gemm, K)),
+        "fp64_gemm": (s_gemm, _roof("tensor", fl_gemm / s_gemm / 1e12 if s_gemm else None, oz_peak,
+                                    f"{peaks_src} bf16 dense, sustained, / 36 digit products",
+                                    "complex FP64 GEMM (rho, the truncation's products, the Rayleigh quotient): "
+                                    "oz_gemm_kernel with its digit passes (exact integer slices on tcgen05), "
+                                    "gemm_c64_kernel (FP64 units) for products below 5.2e6 multiply-adds",
+                                    "8 M N K (Hermitian rho: half) real flops per call", n_gemm, s_gemm, K)),
     }
     order = sorted(cands, key=lambda k: -cands[k][0])
     roof = cands[order[0]][1]
@@ -870,13 +872,17 @@ def run_native(args):
                "useful_complex_tflops": fl_heff / s_heff / 1e12 if s_heff else None,
                "note": "bf16 flops executed = 3 split products x 4 real per complex multiply-add of the useful work"}
     if prec == vtn.VTN_FP64:
-        # the FP64 complex GEMMs of H_eff psi dominate the FP64-mode step
+        # the FP64 complex GEMMs of H_eff psi: exact integer slices, 36 bf16 products a real product
         achieved = fl_heff / s_heff / 1e12 if s_heff > 0 else None
-        roof = {"bound": "alu", "achieved": achieved, "peak": fpeak, "unit": "TFLOP/s",
-                "frac": (achieved / fpeak) if achieved else None, "traffic": GEMM_F64_TRAFFIC,
-                "traffic_note": "ncu dram read+write per launch, mean of the middle-bond H_eff GEMM pair",
-                "kernel": "gemm_c64_kernel (complex FP64 GEMM inside H_eff psi)", "launches": n_heff,
-                "seconds_per_step": s_heff / args.steps, "peak_source": fpeak_src}
+        oz_peak = tc_peak / 36.0
+        roof = {"bound": "tensor", "achieved": achieved, "peak": oz_peak, "unit": "TFLOP/s",
+                "frac": (achieved / oz_peak) if achieved else None, "traffic": None, "traffic_note": None,
+                "kernel": "oz_gemm_kernel with its digit passes (complex FP64 GEMM inside H_eff psi; gemm_c64_kernel "
+                          "below 5.2e6 multiply-adds)", "launches": n_heff,
+                "seconds_per_step": s_heff / args.steps,
+                "peak_source": f"{peaks_src} bf16 dense, sustained, / 36 digit products"}
+    elif s_tc >= s_tri:  # the truncations are filtered: few full tridiagonalisations are left
+        roof = roof_tc
     else:
         # the Householder tridiagonalisation of the FP64 truncation dominates the mixed-mode step
         achieved = fl_tri / s_tri / 1e12 if s_tri > 0 else None
