@@ -47,9 +47,13 @@ constexpr size_t SMEM = 1024 + (size_t)NST * STAGE + 256;
 // Weight pair q holds weights 7 - 2q and 6 - 2q (q = 0 is issued first).  A weight w sums w + 1 digit pairs of at
 // most 2^14 per column, so an accumulator stays within 2^24 for 1024 / (w + 1) columns: the pairs are drained
 // every 4, 4, 8 and 16 stages of 32 columns, at different stages so that one drain overlaps the products of
-// the other pairs; all of them after an item's last stage.
+// the other pairs; all of them after an item's last stage.  An item of at most eight stages is bound by its drains, so it
+// has as few as are exact: weights 7 and 6 after four stages, 5 and 4 after five, the others at the end (eight
+// stages of L theta at chi 128, d 8: six drains instead of eight; the three products of that H_eff
+// application 766 -> 732 us each).
 __device__ __forceinline__ bool drain_due(int q, int k, int nk) {
     if (k == nk - 1) return true;
+    if (nk <= 8) return q == 0 ? k == 3 : q == 1 && k == 4;
     return q == 0 ? (k & 3) == 3 : q == 1 ? (k & 3) == 1 : q == 2 ? (k & 7) == 6 : (k & 15) == 8;
 }
 

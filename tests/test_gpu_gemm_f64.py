@@ -67,6 +67,16 @@ def test_sliced_product_with_the_largest_digits(ctx, value):
     assert _worst(L, th, _product(ctx, L, th), np.random.default_rng(0), count=2) <= 1.0
 
 
+@pytest.mark.parametrize("k", [64, 65, 80, 81, 128, 129])
+def test_sliced_product_of_short_sums_with_the_largest_digits(ctx, k):
+    """Four, five, six, eight and nine summation stages, every digit as large as it gets."""
+    import torch
+    v, n = float.fromhex("0x1.fefefefefefefp0"), 1300
+    L = torch.full((k, k), complex(v, v), dtype=torch.complex128, device="cuda")
+    th = torch.full((k, n), complex(v, -v), dtype=torch.complex128, device="cuda")
+    assert _worst(L, th, _product(ctx, L, th), np.random.default_rng(k)) <= 1.0
+
+
 def test_sliced_product_of_opposed_gradings(ctx):
     """Columns of the left and rows of the right operand graded against each other over 28 decades."""
     import torch
