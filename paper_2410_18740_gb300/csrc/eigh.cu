@@ -1721,7 +1721,8 @@ void density_dev(Ctx& ctx, int nL, int nR, int direction, const double2* theta, 
 }
 
 TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int direction, int k_max,
-                         const double2* theta, double2* left, double2* right, int outer, double* defer) {
+                         const double2* theta, double2* left, double2* right, int outer, double* defer,
+                         bool filter) {
     const int nL = chi_l * d1, nR = d2 * chi_r;
     const int n = direction == 0 ? nL : nR;
     const int k = std::min(k_max, std::min(nL, nR));
@@ -1729,7 +1730,7 @@ TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int dir
     VTN_REQUIRE(outer >= 1 && outer <= (direction == 0 ? nR : nL), "truncation output range out of bounds");
     VTN_REQUIRE(k >= 1, "truncation keeps no state");
     VTN_REQUIRE(n <= 12288, "reduced density matrix larger than 12288 is not supported");
-    if (const int m = filter_rows(nL, nR, direction, k)) {
+    if (const int m = filter ? filter_rows(nL, nR, direction, k) : 0) {
         TruncResult r;
         try {
             if (truncate_filtered(ctx, nL, nR, direction, k, m, theta, left, right, outer, defer, r)) return r;

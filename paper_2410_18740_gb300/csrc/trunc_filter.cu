@@ -207,7 +207,8 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
     } else if (!iterate()) {
         return false;
     }
-    // ---- Rayleigh-Ritz: the exact truncation of the projected tensor
+    // ---- Rayleigh-Ritz: the exact truncation of the projected tensor, by the full reduction: P, U1 and S are this
+    // function's workspaces, and the range of a tensor larger than 4096 is itself of a size that suits the filter
     norm2_dev(ctx, theta, (long long)nL * nR, num + 6);
     ctx.timing = false;
     double2* U1 = (double2*)ctx.workspace(WS_FLT_U, sizeof(double2) * (size_t)m * k);
@@ -218,7 +219,7 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
         g.B = theta; g.ldb = nR;
         g.C = P; g.ldc = nR;
         gemm_c64(ctx, g);
-        res = truncate_dev(ctx, m, 1, 1, nR, 0, k, P, U1, right, outer, defer);
+        res = truncate_dev(ctx, m, 1, 1, nR, 0, k, P, U1, right, outer, defer, false);
         GemmArgs l;
         l.M = n; l.N = k; l.K = m;
         l.opA = OP_C; l.A = S; l.lda = n;
@@ -231,7 +232,7 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
         g.opB = OP_C; g.B = S; g.ldb = n;
         g.C = P; g.ldc = m;
         gemm_c64(ctx, g);
-        res = truncate_dev(ctx, nL, 1, 1, m, 1, k, P, left, U1, outer, defer);
+        res = truncate_dev(ctx, nL, 1, 1, m, 1, k, P, left, U1, outer, defer, false);
         GemmArgs l;
         l.M = k; l.N = n; l.K = m;
         l.A = U1; l.lda = m;

@@ -400,9 +400,10 @@ void conj_transpose_dev(Ctx& ctx, int rows, int cols, const double2* A, long lon
 // defer != nullptr: nothing is read back; the k eigenvalues, tr(rho) and the status words are
 // copied asynchronously to defer (k + 1 + 4 doubles) and the result's lam is empty until
 // truncate_deferred_result reads them after a synchronisation.
+// filter = false: by the full reduction, whatever the shape (for a theta that lies in truncate_filtered's workspaces).
 TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int direction, int k_max,
                          const double2* theta, double2* left, double2* right, int outer = -1,
-                         double* defer = nullptr);
+                         double* defer = nullptr, bool filter = true);
 TruncResult truncate_deferred_result(const double* slot, int k);
 // rho = T T^dag (direction 0, nL x nL) or T^dag T (nR x nR) of the nL x nR matrix T (eigh.cu)
 void density_dev(Ctx& ctx, int nL, int nR, int direction, const double2* theta, double2* rho);

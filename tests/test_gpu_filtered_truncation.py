@@ -92,3 +92,29 @@ def test_truncation_of_a_density_matrix_of_low_rank(ctx, shape, direction, decay
     assert np.linalg.norm(got) ** 2 >= (S[:k] ** 2).sum() - 8 * n * u * k * S[0] ** 2
     if k == r:
         assert np.linalg.norm(got - T) <= 4 * n * u * S[0] * np.sqrt(k)
+
+
+# a density matrix larger than 4096 whose range is itself of a size that the filter takes (half of it, or nearly)
+@pytest.mark.parametrize("shape,direction", [((300, 16, 8, 64, 32), 0), ((64, 8, 16, 300, 32), 1), ((260, 16, 13, 160, 90), 0)])
+def test_truncation_whose_range_suits_the_filter(ctx, shape, direction):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    cl, d1, d2, cr, k = shape
+    n1, n2 = cl * d1, d2 * cr
+    rng = np.random.default_rng(n1 + 5 * n2)
+    r = min(n1, n2)
+    S = np.exp(-9.0 * np.arange(r) / r)
+    U, V = (np.linalg.qr(rng.standard_normal((n, r)) + 1j * rng.standard_normal((n, r)))[0] for n in (n1, n2))
+    T = (U * S) @ V.conj().T
+    left = torch.empty(n1, k, dtype=torch.complex128, device="cuda")
+    right = torch.empty(k, n2, dtype=torch.complex128, device="cuda")
+    kk, lam, disc = vtn.vtn_truncate(ctx, cl, d1, d2, cr, direction, k, torch.from_numpy(np.ascontiguousarray(T)).cuda(), left, right)
+    n, u = max(n1, n2), 2.0 ** -53
+    # the bounds of the tests above; T itself is the product of its factors to a rounding of r terms
+    assert kk == k and np.abs(lam - S[:k] ** 2).max() <= 4 * n * u * S[0] ** 2
+    assert abs(disc - (1.0 - (S[:k] ** 2).sum() / (S ** 2).sum())) <= 4 * n * u * k
+    iso = left if direction == 0 else right.conj().T
+    assert float((iso.conj().T @ iso - torch.eye(k, dtype=torch.complex128, device="cuda")).abs().max()) <= 4 * n * u
+    ref = (U[:, :k] * S[:k]) @ V[:, :k].conj().T
+    gap = (S[k - 1] ** 2 - S[k] ** 2) / S[0] ** 2
+    assert np.linalg.norm((left @ right).cpu().numpy() - ref) <= (4 * n * u / gap * S[k - 1] + 4 * n * u * S[0]) * np.sqrt(k)
