@@ -1737,7 +1737,7 @@ TruncResult truncate_dev(Ctx& ctx, int chi_l, int d1, int d2, int chi_r, int dir
         } catch (const Error& e) {
             // the reduction below needs less memory
             if (e.status != VTN_ENOMEM) throw;
-            for (int s : {WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_U, WS_OZ_PREP}) ctx.drop(s);
+            for (int s : {WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_U, WS_FLT_Y, WS_OZ_PREP}) ctx.drop(s);
         }
     }
     int tt = ctx.tbegin(TC_EIG, 0.0);

@@ -165,7 +165,7 @@ enum WsSlot {
     WS_TC_A2, WS_TC_PART, WS_GEMM_SPLIT, WS_EIG_PART, WS_TC_ENV, WS_EIG_T, WS_H2_ENV, WS_EXPAND,
     WS_TRUNC_L, WS_TRUNC_R, WS_CENTER, WS_MLP_ACT, WS_MLP_Y, WS_MLP_G, WS_WARM_S, WS_WARM_Z, WS_WARM_P,
     WS_WARM_U, WS_WARM_N, WS_WARM_Q0, WS_CQR_G, WS_CQR_T, WS_CQR_B, WS_RQ_Y, WS_RQ_S, WS_CHOL_LINV, WS_TH_A, WS_TH_B,
-    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_OZ_PREP, WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_N, WS_FLT_U, WS_SMP, WS_COUNT
+    WS_OZ_EXP, WS_OZ_A, WS_OZ_B, WS_OZ_PREP, WS_FLT_S, WS_FLT_X, WS_FLT_P, WS_FLT_H, WS_FLT_N, WS_FLT_U, WS_FLT_Y, WS_SMP, WS_COUNT
 };
 
 // ------------------------------------------------------------------ cores

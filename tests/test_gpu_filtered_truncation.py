@@ -118,3 +118,49 @@ def test_truncation_whose_range_suits_the_filter(ctx, shape, direction):
     ref = (U[:, :k] * S[:k]) @ V[:, :k].conj().T
     gap = (S[k - 1] ** 2 - S[k] ** 2) / S[0] ** 2
     assert np.linalg.norm((left @ right).cpu().numpy() - ref) <= (4 * n * u / gap * S[k - 1] + 4 * n * u * S[0]) * np.sqrt(k)
+
+
+def _slices(a, axis):
+    """Three parts of 19 bits below the largest entry along the axis: products of parts of two of them and their
+    sums of up to 2^12 terms are exact in FP64."""
+    import torch
+    r = torch.view_as_real(a)
+    e = torch.ceil(torch.log2(r.abs().amax((axis, 2), keepdim=True).clamp_min(1e-300))) + 1
+    out = []
+    for i in range(3):
+        u = torch.exp2(e - 19 * (i + 1))
+        s = torch.round(r / u) * u
+        r = r - s
+        out.append(torch.view_as_complex(s.contiguous()))
+    return out
+
+
+@pytest.mark.parametrize("n,d,k", [(512, 8, 64), (1024, 8, 128), (1024, 4, 100)])
+@pytest.mark.parametrize("direction", [0, 1])
+def test_large_truncation_is_as_accurate_as_its_roundings(ctx, n, d, k, direction):
+    """A tensor whose entries and singular vectors are exact: permuted Hadamard matrices with phases 1, i, -1, -i
+    and Schmidt values of 30 bits."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(n + k + direction)
+    H = np.ones((1, 1))
+    while len(H) < n:
+        H = np.block([[H, H], [H, -H]])
+    basis = lambda: (np.array([1, 1j, -1, -1j])[rng.integers(4, size=n)][:, None] * H)[rng.permutation(n)][:, rng.permutation(n)]
+    U, V = basis(), basis()
+    S = np.round(np.exp(-9.0 * np.arange(n) / n) * 2 ** 30) / 2 ** 30
+    T, ref = (U * S) @ V.conj().T / n, (U[:, :k] * S[:k]) @ V[:, :k].conj().T / n
+    left = torch.empty(n, k, dtype=torch.complex128, device="cuda")
+    right = torch.empty(k, n, dtype=torch.complex128, device="cuda")
+    _, lam, disc = vtn.vtn_truncate(ctx, n // d, d, d, n // d, direction, k, torch.from_numpy(T).cuda(), left, right)
+    a, b, err = _slices(left, 1), _slices(right, 0), -torch.from_numpy(ref).cuda()
+    for w in range(3):  # left right - ref, largest parts first: what is left after them is at rounding level
+        for i in range(w + 1):
+            err = err + a[i] @ b[w - i]
+    u = 2.0 ** -53
+    # theta: the basis, the projected tensor, the Ritz vectors on both sides and the two factors are rounded, at
+    # most u of their norm each; as much again for what the products' sums and the first order leave out
+    assert float(torch.linalg.norm(err)) <= 12 * u * np.linalg.norm(ref)
+    # lam: a quotient of two sums whose roundings are below u each (a tree of a few levels), and one rounding
+    assert np.linalg.norm(np.asarray(lam) - S[:k] ** 2) <= 2 * u * np.linalg.norm(S[:k] ** 2)
+    assert abs(disc - (S[k:] ** 2).sum() / (S ** 2).sum()) <= 8 * u
