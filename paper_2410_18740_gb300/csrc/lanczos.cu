@@ -203,11 +203,18 @@ __device__ int sturm_count(const double* a, const double* b, int m, double x, do
 // Whether an eigenvalue lies below x, from the leading minors (p_i = (a_i - x) p_{i-1} - b_{i-1}^2 p_{i-2}; scaled
 // by s = 1 / |T|): two dependent operations a step where the quotients of sturm_count take a division.  Its
 // rounding moves the answer by a few ulps of |T| like theirs, so it serves while the section's points are far
-// apart.
+// apart.  The minors shrink by up to 1e-17 a step against |T| (a spectrum that is narrow against its offset), so
+// every eighth step takes a power of two off them: an underflow to zero would pass for a sign change.
 __device__ bool below_minors(const double* a, const double* b, int m, double x, double s) {
     double p0 = 1.0, p1 = (a[0] - x) * s;
     bool neg = p1 <= 0.0;
     for (int i = 1; i < m; ++i) {
+        if ((i & 7) == 0) {
+            const int e = max((__double2hiint(p0) >> 20) & 0x7ff, (__double2hiint(p1) >> 20) & 0x7ff);
+            const double r = __hiloint2double((2046 - min(max(e, 1), 2045)) << 20, 0);
+            p0 *= r;
+            p1 *= r;
+        }
         const double bs = b[i - 1] * s;
         const double p2 = fma((a[i] - x) * s, p1, -(bs * bs) * p0);
         neg = neg || p2 <= 0.0;  // the first sign change: p_{i-1} was positive

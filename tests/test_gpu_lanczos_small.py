@@ -44,3 +44,28 @@ def test_ritz_pair_after_a_fixed_number_of_steps(ctx, cl, cr, K):
     assert n_mv == K and abs(E - E0) <= 1e-12
     v = th.cpu().numpy().reshape(-1)
     assert abs(abs(np.vdot(v0, v)) - 1.0) <= 1e-10 and abs(np.linalg.norm(v) - 1.0) <= 1e-13
+
+
+@pytest.mark.parametrize("cl,cr", [(30, 40), (64, 64)])  # both forms of the vector work
+@pytest.mark.parametrize("spread", [3e-5, 1e-5, 6e-6])
+def test_long_runs_on_a_spectrum_narrow_against_its_shift(ctx, cl, cr, spread):
+    """64 Krylov vectors of 1 + spread H, H's spectrum thin at its ends: a little below the lowest eigenvalue all 64
+    pivots of the tridiagonal matrix are far below its norm, and their product is below the smallest double."""
+    import torch
+    from statistics import NormalDist
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(cl)
+    quantiles = lambda n: np.array([0.5 + 0.12 * NormalDist().inv_cdf((i + 0.5) / n) for i in range(n)])
+    h, g = 1.0 + spread * quantiles(cl), 1.0 + spread / cl * quantiles(cr)
+    q = lambda n: np.linalg.qr(rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))[0]
+    U, V = q(cl), q(cr)
+    L, R = (U * h) @ U.conj().T, (V * g) @ V.conj().T
+    x = rng.standard_normal((cl, cr)) + 1j * rng.standard_normal((cl, cr))
+    one = vtn.make_core(1, 1, 1, [0], [0], np.ones((1, 1, 1), complex))
+    th = torch.from_numpy(x).cuda()
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    _, E, n_mv = vtn.vtn_heff_ground(ctx, one, one, cl, cr, t(L), t(R), th, tol=1e-300, krylov_max=64, max_restarts=0)
+    v = th.cpu().numpy()
+    rq = np.vdot(v, L @ v @ R).real / np.vdot(v, v).real
+    # a Ritz value lies within the spectrum and is its vector's Rayleigh quotient: 64 steps of roundings of |H| = 1
+    assert n_mv == 64 and E >= (h[:, None] * g).min() - 64 * 2.0 ** -52 and abs(E - rq) <= 64 * 2.0 ** -52
