@@ -67,7 +67,7 @@ struct OzOperand {
     int K, kbn;      // summation range: kbn blocks of K
     int tiles;       // row tiles per batch
     int* bx;         // [nb][tiles * tile rows] largest exponent of a row (offset EXP0; 0 = zero row; NONFINITE)
-    int* kx;         // [kbn * K] largest biased exponent of a column of op(A) or row of op(B)
+    int* kx;         // [kbn * K] largest biased exponent of the finite entries of a column of op(A) or row of op(B)
     uint4* out;      // tiles
 };
 
@@ -153,7 +153,10 @@ __global__ void __launch_bounds__(256) oz_max_kernel(OzOperand a, OzOperand b, O
     };
     auto exp_of = [&](double2 v, int kk, int& raw) {
         raw = max(biased_exp(v.x), biased_exp(v.y));
-        if (raw == 0x7ff) return NONFINITE;
+        if (raw == 0x7ff) {  // flags its row; the other rows' scaling of the index is that without it
+            raw = 0;
+            return NONFINITE;
+        }
         // by bits: two comparisons of doubles an element are longer than its load on the narrow FP64 pipe
         if (raw == 0 && ((unsigned)(__double2hiint(v.x) | __double2hiint(v.y)) << 1 | (unsigned)__double2loint(v.x) |
                          (unsigned)__double2loint(v.y)) == 0u) return 0;
@@ -243,7 +246,6 @@ __global__ void __launch_bounds__(256) oz_max_kernel(OzOperand a, OzOperand b, O
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            if (x[j] == 0x7ff || y[j] == 0x7ff) continue;  // those rows and columns are summed directly
             ma = max(ma, x[j]);
             mb = max(mb, y[j]);
             if (x[j] > 0 && y[j] > 0) mt = max(mt, x[j] + y[j]);

@@ -163,3 +163,31 @@ def test_products_without_memory_for_the_digits(monkeypatch):
     assert refused and held
     vtn.vtn_destroy(ctx)
     assert not held
+
+
+@pytest.mark.parametrize("decades", [6, 28])
+def test_sliced_product_with_non_finite_entries_in_opposed_gradings(ctx, decades):
+    """Non-finite entries beside operands whose summation index is scaled: they take no part in the scaling, so
+    the outputs of the other rows and columns are those of the sum without them."""
+    import torch
+    rng = np.random.default_rng(decades)
+    g = torch.logspace(0, -decades, 400, dtype=torch.float64, device="cuda")
+    L, th = _randn(rng, 400, 400) * g[None, :], _randn(rng, 400, 64) * g.flip(0)[:, None]
+    bad = L.clone()
+    bad[3, 5] = float("inf")
+    bad[399, 398] = complex(0.0, float("nan"))
+    got = _product(ctx, bad, th)
+    rows = torch.ones(400, dtype=torch.bool, device="cuda")
+    rows[[3, 399]] = False
+    assert _worst(L[rows], th, got[rows], rng) <= 1.0
+    assert not bool(torch.isfinite(torch.view_as_real(got[~rows])).all(-1).any())
+    # columns: theta R, with L = I the exact product
+    th, R = _randn(rng, 64, 400) * g[None, :], _randn(rng, 400, 400) * g.flip(0)[:, None]
+    bad = R.clone()
+    bad[200, 63] = complex(float("nan"), 1.0)
+    bad[5, 399] = float("-inf")
+    got = _product(ctx, torch.eye(64, dtype=torch.complex128, device="cuda"), th, bad)
+    cols = torch.ones(400, dtype=torch.bool, device="cuda")
+    cols[[63, 399]] = False
+    assert _worst(th, R[:, cols], got[:, cols], rng) <= 1.0
+    assert not bool(torch.isfinite(torch.view_as_real(got[:, ~cols])).all(-1).any())
