@@ -105,11 +105,15 @@ struct OzShift {
 };
 
 // Power-of-two scaling of summation index k: A's column by 2^-shift, B's row by 2^+shift, so that both have
-// the same largest exponent.  It cancels in the product and costs an addition per exponent.
+// the same largest exponent.  It cancels in the product and costs an addition per exponent.  An index that is
+// zero in one operand adds nothing, so the other operand's entries go below all digits, and no row's or column's largest
+// exponent is theirs.
+constexpr int DEAD = 4096;
 __device__ __forceinline__ int k_shift(const OzShift* sh, const int* kxa, const int* kxb, int kk) {
     if (!sh->on) return 0;
     const int x = kxa[kk], y = kxb[kk];
-    return x == 0 || y == 0 ? 0 : (x - y) / 2;  // a zero column or row scales nothing
+    if (x == 0 || y == 0) return x == y ? 0 : x == 0 ? -DEAD : DEAD;
+    return (x - y) / 2;
 }
 
 constexpr int MAX_KS = 64;

@@ -191,3 +191,14 @@ def test_sliced_product_with_non_finite_entries_in_opposed_gradings(ctx, decades
     cols[[63, 399]] = False
     assert _worst(th, R[:, cols], got[:, cols], rng) <= 1.0
     assert not bool(torch.isfinite(torch.view_as_real(got[:, ~cols])).all(-1).any())
+
+
+@pytest.mark.parametrize("side", [0, 1])
+def test_sliced_product_with_indices_that_meet_only_zeros(ctx, side):
+    """Summation indices whose entries are all zero in one operand and far above the rest in the other."""
+    import torch
+    rng = np.random.default_rng(side)
+    L, th = _randn(rng, 400, 400), _randn(rng, 400, 64)
+    L[:, 100:200] *= 0.0 if side == 0 else 1e30
+    th[100:200] *= 1e30 if side == 0 else 0.0
+    assert _worst(L, th, _product(ctx, L, th), rng) <= 1.0
