@@ -441,11 +441,15 @@ __device__ __forceinline__ double oz_value(long long H, long long L, int x) {
     return w2 == 0u ? 0.0 : __hiloint2double((int)rh, (int)rl);
 }
 
-// the output of a row or column with a non-finite entry, term by term in FP64
-__device__ __noinline__ double2 oz_direct(const OzParams& p, int ba, int bb, int m, int n) {
+// The output of a row or column with a non-finite entry, term by term in FP64: an infinity or a NaN, whatever the
+// order of the terms.  By the whole warp, a term per lane (one lane alone takes 0.5 us a term, and a sum of 2^19 of them
+// is longer than the other warps' bounded wait; `beat` tells them that this one is at work).
+__device__ __noinline__ double2 oz_direct(const OzParams& p, int ba, int bb, int m, int n, unsigned* beat) {
     double2 acc = make_double2(0.0, 0.0);
-    for (int kb = 0; kb < p.a.kbn; ++kb)
-        for (int k = 0; k < p.a.K; ++k) {
+    const int lane = threadIdx.x & 31, Kt = p.a.K * p.a.kbn;
+    for (int k0 = 0; k0 < Kt; k0 += 32) {
+        const int kk = k0 + lane, kb = kk / p.a.K, k = kk - kb * p.a.K;
+        if (kk < Kt) {
             const double2 x = oz_load(p.a, (long long)ba * p.a.s_batch, m, kb, k);
             const double2 y = oz_load(p.b, (long long)bb * p.b.s_batch, n, kb, k);
             acc.x = fma(x.x, y.x, acc.x);
@@ -453,6 +457,16 @@ __device__ __noinline__ double2 oz_direct(const OzParams& p, int ba, int bb, int
             acc.y = fma(x.x, y.y, acc.y);
             acc.y = fma(x.y, y.x, acc.y);
         }
+        if ((k0 & 1023) == 0) {
+            if (lane == 0) atomicAdd(beat, 1u);
+            // NaN in both parts stays
+            if (__any_sync(0xffffffffu, acc.x != acc.x) && __any_sync(0xffffffffu, acc.y != acc.y)) break;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    }
     return acc;
 }
 
@@ -466,6 +480,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
     uint64_t* acc_full = empty + NST;     // [NP]
     uint64_t* acc_empty = acc_full + NP;  // [SL]
     uint32_t* tmem_slot = (uint32_t*)(acc_empty + SL);
+    unsigned* beat = (unsigned*)(tmem_slot + 1);  // counts of oz_direct
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int per_split = p.batch * p.tiles_m * p.tiles_n;
     const int items = per_split * p.splits;
@@ -476,6 +491,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
         }
         for (int s = 0; s < NP; ++s) mbar_init(&acc_full[s], 1);
         for (int s = 0; s < SL; ++s) mbar_init(&acc_empty[s], 8);
+        *beat = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -515,7 +531,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 for (int k = 0; k < nk; ++k, ++g) {
                     const int s = g % NST;
                     const uint32_t round = g / NST;
-                    if (g >= NST && !(ok = mbar_wait(&empty[s], (round & 1) ^ 1, p.status))) break;
+                    if (g >= NST && !(ok = mbar_wait(&empty[s], (round & 1) ^ 1, p.status, beat))) break;
                     uint8_t* dst = smem + (size_t)s * STAGE;
                     mbar_expect_tx(&full[s], STAGE);
                     bulk_load(dst, ga + (long long)k * A_BYTES, A_BYTES, &full[s]);
@@ -534,7 +550,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 const int k0 = z * p.kb_per, nk = min(p.nkb - k0, p.kb_per);
                 for (int k = 0; k < nk && ok; ++k, ++g) {
                     const int s = g % NST;
-                    if (!(ok = mbar_wait(&full[s], (g / NST) & 1, p.status))) break;
+                    if (!(ok = mbar_wait(&full[s], (g / NST) & 1, p.status, beat))) break;
                     fence_after();
                     const uint32_t sa = smem_u32(smem + (size_t)s * STAGE), sb = sa + A_BYTES;
                     const uint64_t ad = oz_desc(sa, TM * 16), bd = oz_desc(sb, TN * 16);
@@ -543,8 +559,8 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                         const int w0 = SL - 1 - 2 * q, w1 = w0 - 1;
                         const bool is_fresh = (fresh >> q) & 1u;
                         if (is_fresh && drains[q] > 0) {
-                            if (ok) ok = mbar_wait(&acc_empty[w0], (drains[q] & 1) ^ 1, p.status);
-                            if (ok) ok = mbar_wait(&acc_empty[w1], (drains[q] & 1) ^ 1, p.status);
+                            if (ok) ok = mbar_wait(&acc_empty[w0], (drains[q] & 1) ^ 1, p.status, beat);
+                            if (ok) ok = mbar_wait(&acc_empty[w1], (drains[q] & 1) ^ 1, p.status, beat);
                             fence_after();
                         }
                         const bool due = drain_due(q, k, nk);
@@ -598,7 +614,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 // weights 7..4 into L, then 3..0 into H (rolled: the kernel's code is a large part of a small call)
                 auto drain = [&](int pr, long long (&acc)[32]) {
                     if (!ok || !drain_due(pr, k, nk)) return;
-                    ok = mbar_wait(&acc_full[pr], (drains >> pr) & 1u, p.status);
+                    ok = mbar_wait(&acc_full[pr], (drains >> pr) & 1u, p.status, beat);
                     drains ^= 1u << pr;
                     if (!ok) return;
                     fence_after();
@@ -627,14 +643,21 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             double2* C = to_part ? p.part + ((long long)z * p.batch + bz) * p.M * p.N : p.C + (long long)bz * p.sC_batch;
             const long long cn = to_part ? (p.part_t ? p.M : 1) : p.sC_n;
             double2* dst = C + (long long)m * (to_part ? (p.part_t ? 1 : p.N) : p.ldc) + n0 * cn;
+            const bool flagged = __any_sync(0xffffffffu, ea == NONFINITE || eb == NONFINITE);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int en = __shfl_sync(0xffffffffu, eb, j);
-                if (m >= p.M || n0 + j >= p.N) continue;
-                double2 r;
-                if (ea == NONFINITE || en == NONFINITE) {
-                    r = z == 0 ? oz_direct(p, ba, bb, m, n0 + j) : make_double2(0.0, 0.0);
-                } else {
+                const bool in = m < p.M && n0 + j < p.N, direct = ea == NONFINITE || en == NONFINITE;
+                double2 r = make_double2(0.0, 0.0);
+                if (flagged && z == 0) {
+                    for (unsigned todo = __ballot_sync(0xffffffffu, in && direct); todo != 0u; todo &= todo - 1u) {
+                        const int l = __ffs(todo) - 1;
+                        const double2 v = oz_direct(p, ba, bb, mt * TM + q * 32 + l, n0 + j, beat);
+                        if (lane == l) r = v;
+                    }
+                }
+                if (!in) continue;
+                if (!direct) {
                     const int x = ea + en - 2 * EXP0;  // of zero rows: the sums are zero
                     r = make_double2(oz_value(H[2 * j], L[2 * j], x), oz_value(H[2 * j + 1], L[2 * j + 1], x));
                 }

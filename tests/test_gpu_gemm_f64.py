@@ -202,3 +202,22 @@ def test_sliced_product_with_indices_that_meet_only_zeros(ctx, side):
     L[:, 100:200] *= 0.0 if side == 0 else 1e30
     th[100:200] *= 1e30 if side == 0 else 0.0
     assert _worst(L, th, _product(ctx, L, th), rng) <= 1.0
+
+
+@pytest.mark.parametrize("last", [float("inf"), float("-inf"), float("nan")])
+def test_sliced_product_whose_last_term_is_not_finite(ctx, last):
+    """Sums of 16384 terms whose last one is infinite or NaN in every column: more tiles than SMs, each summed term
+    by term in its epilogue."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(2)
+    w, m, n = 32, 2048, 512
+    one = vtn.make_core(1, 1, 1, [0], [0], np.ones((1, 1, 1), complex))
+    row = vtn.make_core(1, w, 1, [0] * w, range(w), np.ones((w, 1, 1), complex))
+    L, th, R = torch.eye(m, dtype=torch.complex128, device="cuda"), _randn(rng, m, n), _randn(rng, w, n, n)
+    R[w - 1, n - 1] = last
+    y = torch.empty(m, n, dtype=torch.complex128, device="cuda")
+    vtn.vtn_heff_apply(ctx, one, row, m, n, L, R, th, y)
+    # (a + i b) (inf + 0 i) = a inf + i b inf beside finite terms
+    want = torch.view_as_real(th[:, n - 1:]) * last
+    assert torch.equal(torch.nan_to_num(torch.view_as_real(y)), torch.nan_to_num(want.expand(m, n, 2)))
