@@ -141,6 +141,7 @@ void mix_apply(Ctx& ctx, const DevCore& core, bool by_col, int P, int Q, const d
         g.opA = OP_T; g.A = in; g.lda = E;
         g.opB = by_col ? OP_N : OP_T; g.B = core.cid64; g.ldb = core.wr;
         g.C = out; g.ldc = 1; g.sC_n = E;
+        g.sparse_b = true;  // channels that are not coupled
         collapsed = oz_gemm(ctx, g, 1, nullptr);
     }
     if (collapsed)

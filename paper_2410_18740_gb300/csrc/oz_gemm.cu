@@ -21,7 +21,7 @@
 // no-swizzle K-major core matrices), so a stage is two plain bulk copies with no tensor map.
 //
 // A row or column that holds an infinity or NaN is left out of the digits; its outputs are summed
-// term by term in FP64 in the epilogue, with the results the FP64 kernel gives.
+// term by term in FP64 in the epilogue, with the results the FP64 kernel gives (sparse_b: zeros of B are no terms).
 #include <algorithm>
 
 #include "tc_ptx.cuh"
@@ -79,7 +79,7 @@ struct OzParams {
     long long ldc, sC_n, sC_batch;
     double2* part;
     int part_t;          // partials column by column
-    int accumulate, negate, herm_lower;
+    int accumulate, negate, herm_lower, sparse_b;
     int* status;
 };
 
@@ -452,10 +452,12 @@ __device__ __noinline__ double2 oz_direct(const OzParams& p, int ba, int bb, int
         if (kk < Kt) {
             const double2 x = oz_load(p.a, (long long)ba * p.a.s_batch, m, kb, k);
             const double2 y = oz_load(p.b, (long long)bb * p.b.s_batch, n, kb, k);
-            acc.x = fma(x.x, y.x, acc.x);
-            acc.x = fma(-x.y, y.y, acc.x);
-            acc.y = fma(x.x, y.y, acc.y);
-            acc.y = fma(x.y, y.x, acc.y);
+            if (!p.sparse_b || y.x != 0.0 || y.y != 0.0) {
+                acc.x = fma(x.x, y.x, acc.x);
+                acc.x = fma(-x.y, y.y, acc.x);
+                acc.y = fma(x.x, y.y, acc.y);
+                acc.y = fma(x.y, y.x, acc.y);
+            }
         }
         if ((k0 & 1023) == 0) {
             if (lane == 0) atomicAdd(beat, 1u);
@@ -803,7 +805,7 @@ bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 p.ldc = g.ldc; p.sC_n = g.sC_n; p.sC_batch = g.sC_batch;
                 p.part = part;
                 p.part_t = g.sC_n != 1;
-                p.accumulate = g.accumulate; p.negate = g.negate; p.herm_lower = g.herm_lower;
+                p.accumulate = g.accumulate; p.negate = g.negate; p.herm_lower = g.herm_lower; p.sparse_b = g.sparse_b;
                 p.status = ctx.dstatus;
                 VTN_CUDA_TRY(cudaMemsetAsync(shift, 0, sizeof(int) * n_exp, ctx.stream));
                 const int kseg = (int)cdiv((long long)g.K * g.kb, MAX_KS);

@@ -202,6 +202,7 @@ struct GemmArgs {
     bool herm_lower = false;  // result is Hermitian: compute tiles on/below the diagonal only
     int max_splits = 0;       // > 0: at most this many CTAs per output tile along the summation
                               // (1 = never split, so no split-K workspace is touched); 0 = automatic
+    bool sparse_b = false;    // oz_gemm only: zeros of op(B) are absent terms (0 inf is then not NaN)
     bool negate = false;      // C (=|+=) -op(A) op(B)
 };
 // C[i][j] = conj(C[j][i]) for j > i (n x n, leading dimension ldc)

@@ -52,3 +52,26 @@ def test_spelled_out_terms_match_the_dense_core(ctx, d, cl, cr):
             ref = torch.einsum("ajtp,itp->aji", U, A.conj())
             assert bool((out[-1] == 0).all())
         assert float(torch.linalg.norm(out - ref)) <= 1e-14 * float(torch.linalg.norm(ref)) + 1e-300
+
+
+def test_channels_of_a_collapse_core_stay_apart_from_non_finite_ones(ctx):
+    """Scaled identities between many channels, as one product on the tensor cores: an infinity in one channel reaches
+    the channels that are coupled to it and no others, as term by term."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(8)
+    w, d, cl, cr = 48, 4, 96, 96
+    C = rng.standard_normal((w, w)) * (rng.random((w, w)) < 0.5)
+    a, b = np.nonzero(C)
+    core = vtn.make_core(w, w, d, a, b, C[a, b][:, None, None] * np.eye(d, dtype=complex))
+    A = torch.from_numpy(rng.standard_normal((cl, d, cr)) + 1j * rng.standard_normal((cl, d, cr))).cuda()
+    for side, ci, co in ((0, cl, cr), (1, cr, cl)):
+        E = torch.from_numpy(rng.standard_normal((w, ci, ci)) + 1j * rng.standard_normal((w, ci, ci))).cuda()
+        out, bad = (torch.empty(w, co, co, dtype=torch.complex128, device="cuda") for _ in range(2))
+        vtn.vtn_env_update(ctx, core, side, cl, cr, E, A, out)
+        E[7, 3, 5] = float("inf")
+        vtn.vtn_env_update(ctx, core, side, cl, cr, E, A, bad)
+        free = torch.from_numpy((C[7] if side == 0 else C[:, 7]) == 0).cuda()
+        # the flagged elements are summed in FP64 instead of exactly: u sqrt(w) of a norm, with room
+        assert float(torch.linalg.norm((bad - out)[free])) <= 1e-14 * float(torch.linalg.norm(out[free]))
+        assert not bool(torch.isfinite(torch.view_as_real(bad[~free])).all((1, 2, 3)).any())
