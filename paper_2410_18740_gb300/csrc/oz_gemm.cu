@@ -78,7 +78,7 @@ struct OzParams {
     double2* C;
     long long ldc, sC_n, sC_batch;
     double2* part;
-    int part_t;          // partials column by column
+    long long part_m, part_n, part_batch, part_split;  // strides of the partials
     int accumulate, negate, herm_lower, sparse_b;
     int* status;
 };
@@ -642,9 +642,9 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             }
             if (!ok) break;
             const bool to_part = p.splits > 1;
-            double2* C = to_part ? p.part + ((long long)z * p.batch + bz) * p.M * p.N : p.C + (long long)bz * p.sC_batch;
-            const long long cn = to_part ? (p.part_t ? p.M : 1) : p.sC_n;
-            double2* dst = C + (long long)m * (to_part ? (p.part_t ? 1 : p.N) : p.ldc) + n0 * cn;
+            double2* C = to_part ? p.part + z * p.part_split + bz * p.part_batch : p.C + (long long)bz * p.sC_batch;
+            const long long cn = to_part ? p.part_n : p.sC_n;
+            double2* dst = C + (long long)m * (to_part ? p.part_m : p.ldc) + n0 * cn;
             const bool flagged = __any_sync(0xffffffffu, ea == NONFINITE || eb == NONFINITE);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
@@ -755,7 +755,9 @@ bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 "prepared operand of another shape");
     set_smem_attr_once(ctx, (const void*)oz_gemm_kernel, (int)SMEM);
     const int nkb = (int)cdiv((long long)g.K * g.kb, KBC);
-    // at most 1 GiB of digit tiles per operand (one tile row at least): larger problems run in pieces
+    // At most 1 GiB of digit tiles per operand (one tile row at least, 128 rows and columns of a Hermitian result): larger
+    // problems run in pieces, a Hermitian one in square ones of which those above the diagonal are left out.  A
+    // prepared operand is the caller's; it comes whole.
     const long long cap = 1ll << 30;
     const bool a_shared = g.sA_batch == 0 || g.batch == 1, b_shared = g.sB_batch == 0 || g.batch == 1;
     const long long a_batch = cdiv(g.M, TM) * nkb * A_BYTES, b_batch = cdiv(g.N, TNC) * nkb * B_BYTES;
@@ -765,13 +767,15 @@ bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
     long long ms = g.M, ns = g.N;
     if (a_batch > cap) ms = std::max(1ll, cap / ((long long)nkb * A_BYTES)) * TM;
     if (b_batch > cap) ns = std::max(1ll, cap / ((long long)nkb * B_BYTES)) * TNC;
-    // a Hermitian or split result is computed in one piece (the partials' layout and the diagonal refer to all of it)
-    if (g.herm_lower || splits > 1 || g.prepA) { bs = g.batch; ms = g.M; ns = g.N; }
+    if (g.prepA) ms = g.M;
+    if (g.herm_lower && (ms < g.M || ns < g.N)) ms = ns = std::max(1ll, std::min(ms, ns) / TM) * TM;
+    const bool part_t = g.sC_n != 1;  // partials column by column
+    const long long part_m = part_t ? 1 : g.N, part_n = part_t ? g.M : 1, part_batch = (long long)g.M * g.N;
     for (long long b0 = 0; b0 < g.batch; b0 += bs) {
         const int nb = (int)std::min(bs, g.batch - b0);
         for (long long n0 = 0; n0 < g.N; n0 += ns) {
             const int nn = (int)std::min(ns, g.N - n0);
-            for (long long m0 = 0; m0 < g.M; m0 += ms) {
+            for (long long m0 = g.herm_lower ? n0 : 0; m0 < g.M; m0 += ms) {
                 const int mm = (int)std::min(ms, g.M - m0);
                 OzParams p;
                 p.M = mm; p.N = nn; p.nkb = nkb;
@@ -803,9 +807,10 @@ bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 p.b.kx = p.a.kx + nk;
                 p.C = g.C + b0 * g.sC_batch + m0 * g.ldc + n0 * g.sC_n;
                 p.ldc = g.ldc; p.sC_n = g.sC_n; p.sC_batch = g.sC_batch;
-                p.part = part;
-                p.part_t = g.sC_n != 1;
-                p.accumulate = g.accumulate; p.negate = g.negate; p.herm_lower = g.herm_lower; p.sparse_b = g.sparse_b;
+                p.part = part + b0 * part_batch + m0 * part_m + n0 * part_n;
+                p.part_m = part_m; p.part_n = part_n;
+                p.part_batch = part_batch; p.part_split = part_batch * g.batch;
+                p.accumulate = g.accumulate; p.negate = g.negate; p.herm_lower = g.herm_lower && m0 == n0; p.sparse_b = g.sparse_b;
                 p.status = ctx.dstatus;
                 VTN_CUDA_TRY(cudaMemsetAsync(shift, 0, sizeof(int) * n_exp, ctx.stream));
                 const int kseg = (int)cdiv((long long)g.K * g.kb, MAX_KS);

@@ -221,3 +221,75 @@ def test_sliced_product_whose_last_term_is_not_finite(ctx, last):
     # (a + i b) (inf + 0 i) = a inf + i b inf beside finite terms
     want = torch.view_as_real(th[:, n - 1:]) * last
     assert torch.equal(torch.nan_to_num(torch.view_as_real(y)), torch.nan_to_num(want.expand(m, n, 2)))
+
+
+def _recording_context(monkeypatch):
+    """A context whose allocator notes the sizes that were asked for."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    sizes, held = [], {}
+
+    def alloc(nbytes, user):
+        sizes.append(nbytes)
+        t = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    fields = vtn.vtn_allocator._fields_
+    a = vtn.vtn_allocator(fields[0][1](alloc), fields[1][1](lambda p, user: (held.pop(p), None)[1]), None)
+    monkeypatch.setattr(vtn, "_torch_allocator", lambda device: a)
+    return vtn.vtn_create(0), sizes
+
+
+# more than 1 GiB of digits: of the left operand's rows; of a summation that is split over the CTAs
+@pytest.mark.parametrize("w_l,w_r,m,n", [(40, 1, 1024, 33), (1, 2049, 256, 64)])
+def test_sliced_products_in_pieces(monkeypatch, w_l, w_r, m, n):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(w_l)
+    ctx, sizes = _recording_context(monkeypatch)
+    Wi = vtn.make_core(w_l, 1, 1, range(w_l), [0] * w_l, np.ones((w_l, 1, 1), complex))
+    Wj = vtn.make_core(1, w_r, 1, [0] * w_r, range(w_r), np.ones((w_r, 1, 1), complex))
+    eye = lambda k: torch.eye(k, dtype=torch.complex128, device="cuda")[None]
+    L, R = (eye(m), _randn(rng, w_r, n, n)) if w_l == 1 else (_randn(rng, w_l, m, m), eye(n))
+    th, y = _randn(rng, m, n), torch.empty(m, n, dtype=torch.complex128, device="cuda")
+    vtn.vtn_heff_apply(ctx, Wi, Wj, m, n, L, R, th, y)
+    ref = L.sum(0) @ th @ R.sum(0)
+    # the reference's sums over channels and products: u sqrt(terms) each, with room
+    assert float(torch.linalg.norm(y - ref) / torch.linalg.norm(ref)) <= 2e-14
+    assert max(sizes) <= 1 << 30
+    vtn.vtn_destroy(ctx)
+
+
+@pytest.mark.parametrize("direction", [0, 1])
+def test_hermitian_sliced_product_in_pieces(monkeypatch, direction):
+    """The density matrix of a tensor with exactly known factors (Hadamard blocks of 4096 and 256), 1.2 GB of digits."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    ctx, sizes = _recording_context(monkeypatch)
+
+    def had(n):
+        H = torch.ones(1, 1, dtype=torch.float64, device="cuda")
+        while len(H) < n:
+            H = torch.cat([torch.cat([H, H], 1), torch.cat([H, -H], 1)], 0)
+        return H / n ** 0.5
+
+    n1, n2, k = 4096, 256, 24
+    n = n1 + n2
+    U = torch.zeros(n, n, dtype=torch.complex128, device="cuda")
+    U[:n1, :n1], U[n1:, n1:] = had(n1), 1j * had(n2)
+    U = U[torch.randperm(n, generator=torch.Generator().manual_seed(1)).cuda()]
+    S = torch.full((n,), 2.0 ** -10, dtype=torch.float64, device="cuda")
+    top = torch.arange(k, device="cuda") * (n // k)  # in both blocks
+    S[top] = torch.round(1024 * torch.linspace(1.0, 0.25, k, dtype=torch.float64, device="cuda")) / 1024
+    T = (U * S) @ U.flip(0).conj().T
+    left = torch.empty(n, k, dtype=torch.complex128, device="cuda")
+    right = torch.empty(k, n, dtype=torch.complex128, device="cuda")
+    _, lam, _ = vtn.vtn_truncate(ctx, n // 2, 2, 2, n // 2, direction, k, T, left, right)
+    u = 2.0 ** -53
+    assert np.abs(np.asarray(lam) - (S[top] ** 2).cpu().numpy()).max() <= 4 * n * u
+    ref = (U[:, top] * S[top]) @ U.flip(0)[:, top].conj().T
+    # gaps of about 1/16 between the kept part and the rest
+    assert float(torch.linalg.norm(left @ right - ref)) <= 64 * n * u * k ** 0.5
+    assert max(sizes) <= 1 << 30
+    vtn.vtn_destroy(ctx)
