@@ -75,3 +75,26 @@ def test_channels_of_a_collapse_core_stay_apart_from_non_finite_ones(ctx):
         # the flagged elements are summed in FP64 instead of exactly: u sqrt(w) of a norm, with room
         assert float(torch.linalg.norm((bad - out)[free])) <= 1e-14 * float(torch.linalg.norm(out[free]))
         assert not bool(torch.isfinite(torch.view_as_real(bad[~free])).all((1, 2, 3)).any())
+
+
+@pytest.mark.parametrize("side", [0, 1])
+def test_collapse_core_on_the_tensor_cores_matches_the_dense_core(ctx, side):
+    """Complex couplings between many channels at sizes where they are one sliced product, from either side."""
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(side)
+    wl, wr, d, cl, cr = 40, 56, 4, 96, 91
+    C = (rng.standard_normal((wl, wr)) + 1j * rng.standard_normal((wl, wr))) * (rng.random((wl, wr)) < 0.7)
+    a, b = np.nonzero(C)
+    core = vtn.make_core(wl, wr, d, a, b, C[a, b][:, None, None] * np.eye(d, dtype=complex))
+    z = lambda *s: torch.from_numpy(rng.standard_normal(s) + 1j * rng.standard_normal(s)).cuda()
+    A, W = z(cl, d, cr), torch.from_numpy(C).cuda()
+    w_in, w_out, ci, co = (wl, wr, cl, cr) if side == 0 else (wr, wl, cr, cl)
+    E, out = z(w_in, ci, ci), torch.empty(w_out, co, co, dtype=torch.complex128, device="cuda")
+    vtn.vtn_env_update(ctx, core, side, cl, cr, E, A, out)
+    if side == 0:
+        ref = torch.einsum("itl,ab,aij,jtk->blk", A.conj(), W, E, A)
+    else:
+        ref = torch.einsum("jtg,ab,bgp,itp->aji", A, W, E, A.conj())
+    # three contractions of at most 384 terms, u sqrt(terms) each, with room
+    assert float(torch.linalg.norm(out - ref) / torch.linalg.norm(ref)) <= 1e-14
