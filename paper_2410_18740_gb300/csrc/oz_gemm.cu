@@ -442,28 +442,33 @@ __device__ __forceinline__ double oz_value(long long H, long long L, int x) {
 }
 
 // The output of a row or column with a non-finite entry, term by term in FP64: an infinity or a NaN, whatever the
-// order of the terms.  By the whole warp, a term per lane (one lane alone takes 0.5 us a term, and a sum of 2^19 of them
-// is longer than the other warps' bounded wait; `beat` tells them that this one is at work).
-__device__ __noinline__ double2 oz_direct(const OzParams& p, int ba, int bb, int m, int n, unsigned* beat) {
+// order of the terms.  By the whole warp, 128 terms a step of about a microsecond (one lane alone takes half of
+// one a term): the other warps' waits end after a second.  The longest sums of an SM with more than one item are of
+// 83,000 terms (digits of at most 1 GiB an operand, 16 splits), 0.3 s for all 512 outputs of a warp.
+__device__ __noinline__ double2 oz_direct(const OzParams& p, int ba, int bb, int m, int n) {
     double2 acc = make_double2(0.0, 0.0);
-    const int lane = threadIdx.x & 31, Kt = p.a.K * p.a.kbn;
-    for (int k0 = 0; k0 < Kt; k0 += 32) {
-        const int kk = k0 + lane, kb = kk / p.a.K, k = kk - kb * p.a.K;
-        if (kk < Kt) {
-            const double2 x = oz_load(p.a, (long long)ba * p.a.s_batch, m, kb, k);
-            const double2 y = oz_load(p.b, (long long)bb * p.b.s_batch, n, kb, k);
-            if (!p.sparse_b || y.x != 0.0 || y.y != 0.0) {
-                acc.x = fma(x.x, y.x, acc.x);
-                acc.x = fma(-x.y, y.y, acc.x);
-                acc.y = fma(x.x, y.y, acc.y);
-                acc.y = fma(x.y, y.x, acc.y);
+    const int Kt = p.a.K * p.a.kbn;
+    for (int k0 = threadIdx.x & 31; k0 - (int)(threadIdx.x & 31) < Kt; k0 += 128) {
+        double2 x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int kk = k0 + 32 * u, kb = kk / p.a.K, k = kk - kb * p.a.K;
+            x[u] = y[u] = make_double2(0.0, 0.0);
+            if (kk < Kt) {
+                x[u] = oz_load(p.a, (long long)ba * p.a.s_batch, m, kb, k);
+                y[u] = oz_load(p.b, (long long)bb * p.b.s_batch, n, kb, k);
             }
         }
-        if ((k0 & 1023) == 0) {
-            if (lane == 0) atomicAdd(beat, 1u);
-            // NaN in both parts stays
-            if (__any_sync(0xffffffffu, acc.x != acc.x) && __any_sync(0xffffffffu, acc.y != acc.y)) break;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (p.sparse_b && y[u].x == 0.0 && y[u].y == 0.0) continue;
+            acc.x = fma(x[u].x, y[u].x, acc.x);
+            acc.x = fma(-x[u].y, y[u].y, acc.x);
+            acc.y = fma(x[u].x, y[u].y, acc.y);
+            acc.y = fma(x[u].y, y[u].x, acc.y);
         }
+        // NaN in both parts stays
+        if (__any_sync(0xffffffffu, acc.x != acc.x) && __any_sync(0xffffffffu, acc.y != acc.y)) break;
     }
     for (int o = 16; o > 0; o >>= 1) {
         acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
@@ -482,7 +487,6 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
     uint64_t* acc_full = empty + NST;     // [NP]
     uint64_t* acc_empty = acc_full + NP;  // [SL]
     uint32_t* tmem_slot = (uint32_t*)(acc_empty + SL);
-    unsigned* beat = (unsigned*)(tmem_slot + 1);  // counts of oz_direct
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int per_split = p.batch * p.tiles_m * p.tiles_n;
     const int items = per_split * p.splits;
@@ -493,7 +497,6 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
         }
         for (int s = 0; s < NP; ++s) mbar_init(&acc_full[s], 1);
         for (int s = 0; s < SL; ++s) mbar_init(&acc_empty[s], 8);
-        *beat = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -533,7 +536,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 for (int k = 0; k < nk; ++k, ++g) {
                     const int s = g % NST;
                     const uint32_t round = g / NST;
-                    if (g >= NST && !(ok = mbar_wait(&empty[s], (round & 1) ^ 1, p.status, beat))) break;
+                    if (g >= NST && !(ok = mbar_wait(&empty[s], (round & 1) ^ 1, p.status))) break;
                     uint8_t* dst = smem + (size_t)s * STAGE;
                     mbar_expect_tx(&full[s], STAGE);
                     bulk_load(dst, ga + (long long)k * A_BYTES, A_BYTES, &full[s]);
@@ -552,7 +555,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 const int k0 = z * p.kb_per, nk = min(p.nkb - k0, p.kb_per);
                 for (int k = 0; k < nk && ok; ++k, ++g) {
                     const int s = g % NST;
-                    if (!(ok = mbar_wait(&full[s], (g / NST) & 1, p.status, beat))) break;
+                    if (!(ok = mbar_wait(&full[s], (g / NST) & 1, p.status))) break;
                     fence_after();
                     const uint32_t sa = smem_u32(smem + (size_t)s * STAGE), sb = sa + A_BYTES;
                     const uint64_t ad = oz_desc(sa, TM * 16), bd = oz_desc(sb, TN * 16);
@@ -561,8 +564,8 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                         const int w0 = SL - 1 - 2 * q, w1 = w0 - 1;
                         const bool is_fresh = (fresh >> q) & 1u;
                         if (is_fresh && drains[q] > 0) {
-                            if (ok) ok = mbar_wait(&acc_empty[w0], (drains[q] & 1) ^ 1, p.status, beat);
-                            if (ok) ok = mbar_wait(&acc_empty[w1], (drains[q] & 1) ^ 1, p.status, beat);
+                            if (ok) ok = mbar_wait(&acc_empty[w0], (drains[q] & 1) ^ 1, p.status);
+                            if (ok) ok = mbar_wait(&acc_empty[w1], (drains[q] & 1) ^ 1, p.status);
                             fence_after();
                         }
                         const bool due = drain_due(q, k, nk);
@@ -616,7 +619,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                 // weights 7..4 into L, then 3..0 into H (rolled: the kernel's code is a large part of a small call)
                 auto drain = [&](int pr, long long (&acc)[32]) {
                     if (!ok || !drain_due(pr, k, nk)) return;
-                    ok = mbar_wait(&acc_full[pr], (drains >> pr) & 1u, p.status, beat);
+                    ok = mbar_wait(&acc_full[pr], (drains >> pr) & 1u, p.status);
                     drains ^= 1u << pr;
                     if (!ok) return;
                     fence_after();
@@ -645,24 +648,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             double2* C = to_part ? p.part + z * p.part_split + bz * p.part_batch : p.C + (long long)bz * p.sC_batch;
             const long long cn = to_part ? p.part_n : p.sC_n;
             double2* dst = C + (long long)m * (to_part ? p.part_m : p.ldc) + n0 * cn;
-            const bool flagged = __any_sync(0xffffffffu, ea == NONFINITE || eb == NONFINITE);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int en = __shfl_sync(0xffffffffu, eb, j);
-                const bool in = m < p.M && n0 + j < p.N, direct = ea == NONFINITE || en == NONFINITE;
-                double2 r = make_double2(0.0, 0.0);
-                if (flagged && z == 0) {
-                    for (unsigned todo = __ballot_sync(0xffffffffu, in && direct); todo != 0u; todo &= todo - 1u) {
-                        const int l = __ffs(todo) - 1;
-                        const double2 v = oz_direct(p, ba, bb, mt * TM + q * 32 + l, n0 + j, beat);
-                        if (lane == l) r = v;
-                    }
-                }
-                if (!in) continue;
-                if (!direct) {
-                    const int x = ea + en - 2 * EXP0;  // of zero rows: the sums are zero
-                    r = make_double2(oz_value(H[2 * j], L[2 * j], x), oz_value(H[2 * j + 1], L[2 * j + 1], x));
-                }
+            auto store = [&](int j, double2 r) {
                 if (p.negate) r = make_double2(-r.x, -r.y);
                 if (p.accumulate && !to_part) {
                     const double2 o = dst[j * cn];
@@ -670,6 +656,27 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                     r.y += o.y;
                 }
                 dst[j * cn] = r;
+            };
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const int en = __shfl_sync(0xffffffffu, eb, j);
+                if (m >= p.M || n0 + j >= p.N || ea == NONFINITE || en == NONFINITE) continue;
+                const int x = ea + en - 2 * EXP0;  // of zero rows: the sums are zero
+                store(j, make_double2(oz_value(H[2 * j], L[2 * j], x), oz_value(H[2 * j + 1], L[2 * j + 1], x)));
+            }
+            // (apart from the loop above, which is 4 % of a product longer with this inside)
+            if (__any_sync(0xffffffffu, ea == NONFINITE || eb == NONFINITE)) {
+#pragma unroll 1
+                for (int j = 0; j < 16; ++j) {
+                    const int en = __shfl_sync(0xffffffffu, eb, j);
+                    unsigned todo = __ballot_sync(0xffffffffu, m < p.M && n0 + j < p.N && (ea == NONFINITE || en == NONFINITE));
+                    for (; todo != 0u; todo &= todo - 1u) {
+                        const int l = __ffs(todo) - 1;
+                        double2 r = make_double2(0.0, 0.0);
+                        if (z == 0) r = oz_direct(p, ba, bb, mt * TM + q * 32 + l, n0 + j);
+                        if (lane == l) store(j, r);
+                    }
+                }
             }
         }
     }

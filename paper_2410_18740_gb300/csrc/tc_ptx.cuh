@@ -36,21 +36,14 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// bounded wait: false (and status set) after 1 s or when another CTA already failed.  beat (optional): a counter in
-// shared memory that another warp of the CTA raises while it works for longer than that; each count starts the second again
-__device__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status, const volatile unsigned* beat = nullptr) {
+// bounded wait: false (and status set) after 1 s or when another CTA already failed
+__device__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status) {
     if (mbar_test(bar, parity)) return true;
-    unsigned long long t0 = now_ns();
-    unsigned seen = beat != nullptr ? *beat : 0u;
+    const unsigned long long t0 = now_ns();
     while (true) {
         if (mbar_test(bar, parity)) return true;
         if (*(volatile int*)status != 0) return false;
         if (now_ns() - t0 > 1000000000ull) {
-            if (beat != nullptr && *beat != seen) {
-                seen = *beat;
-                t0 = now_ns();
-                continue;
-            }
             atomicExch(status, 1);
             return false;
         }
