@@ -264,12 +264,13 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
     // ---- Rayleigh-Ritz: the exact truncation of the projected tensor, by the full reduction: P, U1 and S are this
     // function's workspaces, and the range of a tensor larger than 4096 is itself of a size that suits the filter.
     // Its backward error u |rho| lies in m dimensions instead of n, so the vectors at the boundary mix more than
-    // those of the full reduction do; with the next k / 4 + 16 Ritz vectors at hand (k2 in all, 768 at most unless k
-    // is larger: the reduction's own limit is 775) a first-order correction from products takes that back.  Error
-    // of theta against twice the working precision, reduction of all of rho | without the correction | with it:
-    // 1.9 | 2.9 | 0.75e-15 at n = 1024, k = 128; 3.4 | 4.3 | 1.1e-15 at n = 1830, k = 300; of lam 1.2 | 3.9 | 1.2e-16.
-    // It takes 1.0 of 14.7 and 3.3 of 48.5 ms; with all m vectors 1.3 and 4.9 ms for 0.68 and 1.03e-15.
-    const int k2 = std::min(m, std::max(k, std::min(768, k + k / 4 + 16)));
+    // those of the full reduction do; with the next 16 Ritz vectors at hand (k2 in all, 768 at most unless k is
+    // larger: the reduction's own limit is 775) a first-order correction from products takes that back.  Error of
+    // theta against twice the working precision, reduction of all of rho | without the correction | with it:
+    // 1.9 | 2.9 | 0.83e-15 at n = 1024, k = 128; 3.4 | 4.4 | 1.2e-15 at n = 1830, k = 300; of lam 1.2 | 3.7 | 1.3e-16.
+    // It takes 0.4 of 14.0 and 1.9 of 47.1 ms; with k / 4 more vectors 14.6 and 48.3 ms for 0.75 and 1.09e-15,
+    // with all m 15.0 and 50.1 ms for 0.68 and 1.03e-15.
+    const int k2 = std::min(m, std::max(k, std::min(768, k + 16)));
     norm2_dev(ctx, theta, (long long)nL * nR, num + 6);
     ctx.timing = false;
     double2* U1 = (double2*)ctx.workspace(WS_FLT_U, sizeof(double2) * (size_t)m * k2);
