@@ -833,7 +833,7 @@ bool oz_gemm(Ctx& ctx, const GemmArgs& g, int splits, double2* part) {
                 VTN_REQUIRE(items < (1ll << 31) && ma + mb < (1ll << 31) && sa + sb < (1ll << 31), "GEMM too large");
                 oz_gemm_kernel<<<(unsigned)std::min<long long>(items, std::max(ctx.num_sms, 1)), THREADS, SMEM, ctx.stream>>>(p);
                 ctx.dstatus_due = true;
-                ctx.count_launch(4);
+                ctx.count_launch(prep ? 3 : 4);
                 ctx.check_launch("oz_gemm");
             }
         }
