@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 
 #include "vtn_internal.cuh"
 
@@ -328,6 +329,7 @@ bool truncate_filtered(Ctx& ctx, int nL, int nR, int direction, int k, int m, co
     ctx.sync();
     res.k = k;
     res.lam.assign(ctx.pinned, ctx.pinned + k);
+    std::sort(res.lam.begin(), res.lam.end(), std::greater<double>());  // equal ones differ in their last bits
     double kept = 0.0;
     for (double l : res.lam) kept += l;
     res.discarded = ctx.pinned[k] > 0.0 ? 1.0 - kept / ctx.pinned[k] : 0.0;

@@ -164,3 +164,15 @@ def test_large_truncation_is_as_accurate_as_its_roundings(ctx, n, d, k, directio
     # lam: a quotient of two sums whose roundings are below u each (a tree of a few levels), and one rounding
     assert np.linalg.norm(np.asarray(lam) - S[:k] ** 2) <= 2 * u * np.linalg.norm(S[:k] ** 2)
     assert abs(disc - (S[k:] ** 2).sum() / (S ** 2).sum()) <= 8 * u
+
+
+@pytest.mark.parametrize("direction", [0, 1])
+def test_eigenvalues_descend_where_many_are_equal(ctx, direction):
+    import torch
+    from paper_2410_18740_gb300 import vtn
+    rng = np.random.default_rng(direction)
+    T = _tensor(rng, 520, 512, _spectrum("degenerate top", 512, 64))
+    left = torch.empty(520, 64, dtype=torch.complex128, device="cuda")
+    right = torch.empty(64, 512, dtype=torch.complex128, device="cuda")
+    _, lam, _ = vtn.vtn_truncate(ctx, 65, 8, 8, 64, direction, 64, torch.from_numpy(np.ascontiguousarray(T)).cuda(), left, right)
+    assert (np.diff(np.asarray(lam)) <= 0).all()
