@@ -33,6 +33,10 @@
  *  - Errors: every call returns a vtn_status and never aborts or exits.  On failure
  *    the out-parameters are left untouched (vtn_sweep keeps the last valid MPS) and
  *    vtn_last_error(ctx) holds a one-line message.
+ *  - Device memory: a context keeps its workspaces until vtn_destroy; the digits of FP64
+ *    products among them take at most 1 GiB an operand (or one block of 128 rows) and are given
+ *    back earlier when another allocation of the context fails.  Each worker of vtn_sweep_batch
+ *    has its own for the call.
  *  - Threads: one context per host thread.
  */
 #ifndef VTN_H
@@ -62,9 +66,11 @@ typedef enum {
 } vtn_status;
 
 typedef enum {
-    VTN_FP64 = 0,          /* every contraction to IEEE double accuracy: FP64 FMA, or (large
-                              products) exact sums of 8-bit digit products on the tensor
-                              cores, rounded once                                        */
+    VTN_FP64 = 0,          /* FP64 FMA, or (products of 5.2e6 multiply-adds and more) sums of
+                              8-bit digit products on the tensor cores, exact but for less
+                              than 2^-57 (largest of the row) (largest of the column) a
+                              term, rounded once: below FP64 FMA's error in norm, but an
+                              output far below that product has fewer correct digits    */
     VTN_TF32X3 = 1,        /* reserved: three-term TF32 split products (VTN_EUNSUPPORTED) */
     VTN_BF16X3 = 2         /* H_eff psi and the environment updates on the tensor cores:
                               each FP64 operand split into bf16 hi + lo, products
@@ -433,8 +439,10 @@ vtn_status vtn_heff_ground(vtn_ctx ctx, const vtn_core* Wi, const vtn_core* Wj, 
  * density matrix, keeping k = min(k_max, chi_l d1, d2 chi_r) eigenpairs of largest
  * eigenvalue (squared Schmidt values, Eq. SurrogateEpsChi).  Where at most a third of the
  * eigenpairs of a matrix larger than 256 are kept they are found by Chebyshev-filtered subspace
- * iteration run until its residual is at rounding level, else (or when it would not pay) by
- * the full Householder reduction; the accuracy is the same:
+ * iteration run until its residual is at rounding level; where T's other side is at most half as
+ * long (and about 1.5 k at most, or the matrix larger than 4096) in T's own range, whatever
+ * part of it is kept; else (or when it would not pay) by the full Householder reduction.  The
+ * first two end in a first-order correction and are no less accurate than the reduction:
  *  direction 0: rho = T T^dag = U diag(lam) U^dag; left = U_k (chi_l,d1,k, left-canonical),
  *               right = U_k^dag T (k,d2,chi_r).
  *  direction 1: rho = T^dag T = V diag(lam) V^dag; left = T V_k (chi_l,d1,k),
@@ -479,6 +487,9 @@ vtn_status vtn_lbo_rotate(vtn_ctx ctx, int chi_l, int d, int D, int chi_r, const
  * nothing: the caller passes inputs and outputs, and every intermediate lives in one
  * file-scope device array of 32 MiB that every GPU which loads the library keeps until the
  * process exits.
+ *
+ * The products run on the FP64 units at every size: the tensor-core products of
+ * vtn_heff_apply need scratch that is allocated.
  *
  * Same contraction, layouts and argument meaning as vtn_heff_apply (FP64):
  *   y[i,t,u,l] = sum L[a,i,j] Wi[a,b,t,s] Wj[b,c,u,v] theta[j,s,v,k] R[c,k,l]

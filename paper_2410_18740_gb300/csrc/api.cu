@@ -1704,8 +1704,8 @@ vtn_status vtn_sample(vtn_ctx ctx, vtn_mpo mpo, vtn_mps mps, uint64_t seed, int 
         const int M = mpo->hp.M, D = mpo->hp.D, d = mpo->hp.d;
         const int chi = max_dim(mps->dims);
         const size_t env = (size_t)chi * chi;
-        // One CTA per sample walks all sites in one launch where that is the shorter: 16 D chi^2 FP64 operations a site
-        // at 3 G/s an SM against about 80 us for a site's four launches (both for one wave of samples).
+        // One CTA per sample walks all sites in one launch where that is the shorter: 8 D chi^2 FP64 multiply-adds a site
+        // at 3.2 G/s an SM and wave of samples, against about 80 us for a site's launches of the batched form.
         const bool fock = !mpo->hp.lbo && D == d;
         const double waves = std::ceil(n_samples / (double)std::max(c.num_sms, 1));
         const bool batched = waves * 8.0 * D * (double)chi * chi / 3.2e9 > 80e-6;

@@ -68,8 +68,9 @@ __global__ void __launch_bounds__(256) mix_kernel(int P, int d, int Q, const int
 // The same from the spelled-out terms: one output (channel, level, p, q) per thread.  FP64-issue bound, so
 // a term costs what its coefficient needs: two FMAs when real or imaginary (most entries of the GBS cores: x is
 // real, p imaginary, couplings real), four when complex, and none for a lone pass-through channel, which
-// is a copy.  Zero entries of the d x d operators (x and p have two a row) are not visited.  The terms keep
-// the order of the dense loop above, so the sums are the same.  The terms are the same for all threads of a
+// is a copy.  Zero entries of the d x d operators (x and p have two a row) are not visited: they are no terms, so a
+// non-finite level reaches the levels that are coupled to it only (the dense loop's 0 inf made them all NaN).  The
+// terms keep the order of the dense loop above, so finite sums are the same.  The terms are the same for all threads of a
 // block; their inputs come from L2 (each is used by a few outputs).
 // ACC: added to the output instead of replacing it (outputs without a term keep what they hold).
 template <bool ACC>

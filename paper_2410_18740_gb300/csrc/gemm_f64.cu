@@ -164,12 +164,12 @@ void gemm_c64(Ctx& ctx, const GemmArgs& g, int timing_class) {
     const long long gx = (g.N + BT - 1) / BT, gy = (g.M + BT - 1) / BT;
     VTN_REQUIRE(gy <= 4 * 65535LL, "gemm M too large");
     const double macs = (double)g.M * g.N * g.K * g.kb * g.batch * (g.herm_lower ? 0.5 : 1.0);
-    // The sliced product costs four launches, about 34 us, and then runs 35 times faster.  Measured, DFMA
-    // against sliced: 128^3 22 | 34 us, 160^3 34 | 35 us, 192^3 55 | 37 us, 256^3 136 | 38 us, 1024 x 16 x 1024
-    // (narrow: padded to 32 columns) 74 | 49 us; at 3072^3 200 ms against 6.2 ms.  (A shorter exponent pass has since
-    // taken 2 us off the sliced side: 36 us at 256^3; products at the line keep their side, whose order of additions
-    // the smallest solves' discarded weights show.)  Its row sums fit 96-bit integers
-    // for summations of up to 2^19 terms.
+    // The sliced product costs four launches, about 48 us back to back, and then runs 35 times faster; the FP64 units
+    // take a wave of 16 x 16 tiles after the other.  Measured, FP64 units | sliced: 128 x 128 x 256 (4.2e6) 43 | 48 us,
+    // 160 x 128 x 256 (5.2e6) 76 | 48 us, 160 x 160 x 256 76 | 48 us; at 3072^3 200 ms against 6.2 ms.  The line counts what is
+    // asked for, not the padding, which is the wrong way round at the worst by 1.5: 8 columns (padded to 16 and 32)
+    // 2048 x 8 x 256 (4.2e6) 76 | 50 us, rows that fill an eighth of a tile 24 x 16 x 16 x 4096 (2.5e7) 195 | 281 us.
+    // Its row sums fit 96-bit integers for summations of up to 2^19 terms.
     bool oz = g.prepA != nullptr || ctx.dstatus != nullptr && g.max_splits != 1 && macs >= 5.2e6 && (long long)g.K * g.kb <= (1LL << 19);
     int S = 1;
     if (oz) {

@@ -267,7 +267,9 @@ __global__ void __launch_bounds__(256) sample_kernel(SampleArgs a) {
 // (V null: the Fock basis, p[n] = rho[n][n]), the draw as in sample_kernel, and the next ell = sum_m V[n][m] X[m] /
 // sqrt(p[n]).  The D levels enter only here, so the two products of a site are D / d times smaller than on
 // rotated tensors and run for all samples at once (64 samples of a 100-mode chi = 96 chain: 78 ms as one CTA per
-// sample over all sites, FP64-pipe bound on 64 SMs).
+// sample over all sites, FP64-pipe bound on 64 SMs).  A level's probability has an error of a rounding of the
+// site's sum, not of itself; a level that feels it is below the resolution of the 53-bit uniform number, and the
+// next ell's scale drops out of the next site's draw.
 __global__ void __launch_bounds__(256) sample_site_kernel(int s, int M, int D, int d, int cr, unsigned k0, unsigned k1, int t0,
                                                           const double2* __restrict__ X, const double2* __restrict__ Y,
                                                           const double2* __restrict__ V, double2* __restrict__ ell,

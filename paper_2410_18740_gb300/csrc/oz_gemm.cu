@@ -7,12 +7,16 @@
 //   * each row of A (column of B) is written as fixed point relative to its largest exponent, 63 bits
 //     and a sign, cut into eight signed 8-bit digits (|digit| <= 128, exact in bf16);
 //   * digit i of A times digit j of B contributes at weight 256^-(i+j).  The 36 pairs with i + j <= 7
-//     are multiplied; what is left out is below 2^-60 of (largest of the row) x (largest of the column)
-//     per term, 2^-7 of an FP64 rounding of such a term;
+//     are multiplied.  The 28 others (at most 1.76 2^-60 a real product) and the cut of both operands
+//     to 63 bits (2^-60) leave out less than 6 2^-60 of (largest of the row) x (largest of the column)
+//     a complex term;
 //   * products of one weight s = i + j are summed in one FP32 tensor-memory accumulator while every
 //     partial sum is an integer of at most 2^24 (128 products-of-pairs deep: exact), then drained into
-//     64-bit integers.  The only roundings are the final conversion to double and that of C += ;
-//     the error is that of one rounding of the exact sum where a DFMA chain has one per term.
+//     64-bit integers.  The only roundings are the final conversion to double (of each part of a split
+//     summation) and that of C += : one rounding of the sum where a DFMA chain has one per term.
+// So the accuracy is relative to the largest entries of the row and the column (of the scaled operands: k_shift), not
+// to the terms themselves: in [[1, e], [1, 1]] [[0, 1], [1, 1]] the e of the first output has a relative error of
+// up to 2^-56 / e, where a DFMA chain gives it exactly.
 // Complex products take the real 2 x 2 block form of the split-precision mode (A~ rows (re, im), B~ rows
 // (re, -im) and (im, re)), so a real GEMM yields interleaved outputs.
 //
@@ -94,8 +98,9 @@ __device__ __forceinline__ int biased_exp(double x) { return (__double2hiint(x) 
 
 constexpr int EXP0 = 8192;           // stored row exponent = biased exponent (with its shift) + EXP0
 constexpr int NONFINITE = 1 << 20;
-// Bits that the row-times-column scaling may cost against the largest term of the sum before the summation
-// index is scaled too: the pairs left out then stay below 2^-56 of that term
+// Binades that the row-times-column scaling may cost against the largest term of the sum before the summation
+// index is scaled too: what is left out of a term then stays below 2^-51 of that largest one (mantissas add up to two
+// binades), and typically 2^-56
 constexpr int LOSS_BITS = 4;
 
 struct OzShift {

@@ -16,8 +16,9 @@
 // Measured (whole truncation; full reduction with sliced products -> here, when the step was made): n = 512, k = 64
 // 8.9 -> 7.2 ms; n = 1024, k = 128 29.8 -> 13.7 ms; n = 1830, k = 300 86 -> 40 ms (Schmidt values decaying by e^-9);
 // flat random spectra 8.9 -> 9.0, 29.8 -> 27.3, 86 -> 71 ms.  With the shorter Cholesky and tridiagonalisation chains
-// the middle two are 12.7 and 37.7 ms.  What is left is latency: the Cholesky chains (50 us per 32 rows and pass), the
-// m x m tridiagonalisation (10 us a column) and about 50 us a product.
+// and the correction of the Ritz vectors the decaying ones take 12.8 ms at n = 1024 and 39.2 ms at 1830.  What is left
+// is latency: the Cholesky chains (50 us per 32 rows and pass), the m x m tridiagonalisation (10 us a column) and about
+// 50 us a product.
 //
 // The host reads five numbers after each pass.  It gives up (false: the full eigendecomposition runs) when the
 // spectrum at k is so flat that the predicted polynomial degree costs more than the reduction, when the block is
